@@ -185,7 +185,7 @@ static_assert(P0 >= 1 && P1 >= 1 && N3 * N3 * N3 == kNc, "level split");
 template <typename T, bool FACE>
 __global__ void __cluster_dims__(kCR, 1, 1) __launch_bounds__(kCT)
     k_coarse_cluster(CoarseSet cs, const T* __restrict__ f_top, T* __restrict__ u_top,
-                     const double* __restrict__ aug, int zero_u) {
+                     const double* __restrict__ minv_g, int zero_u) {
     cg::cluster_group cluster = cg::this_cluster();
     const int self = (int)cluster.block_rank();
     extern __shared__ unsigned char smem_raw[];
@@ -222,12 +222,11 @@ __global__ void __cluster_dims__(kCR, 1, 1) __launch_bounds__(kCT)
         L[0].f[c] = f_top[self * sz[0] + c];
         L[0].u[c] = zero_u ? T(0) : u_top[self * sz[0] + c];
     }
-    // block 0: the 4^3 inverse (its kNc x kNc block of the augmented matrix),
-    // read once here so that the exact solve later runs from shared memory
+    // block 0: the 4^3 inverse, read once here so that the exact solve later runs from shared memory
     double* minv = reinterpret_cast<double*>(q);
     if (self == 0)
         for (int e = threadIdx.x; e < kNc * kNc; e += blockDim.x)
-            minv[e] = aug[(e / kNc) * kW + kNb + (e % kNc)];
+            minv[e] = minv_g[e];
     cluster.sync();
     // down: the two distributed levels
     for (int s = 0; s < cs.nu1; ++s)

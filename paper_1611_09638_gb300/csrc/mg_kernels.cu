@@ -265,96 +265,159 @@ __global__ void k_prolong_add(Dims df, Dims dc, int cx, int cy, int cz, const T*
     u[c] += acc;
 }
 
-// Coarsest level (64 nodes): Gauss-Jordan inversion with partial pivoting of
-// the bordered system [L 1; 1^T 0] (65 x 65), in FP64, by one block working
-// on the augmented matrix [M | I] (65 x 130) in shared memory; the result is
-// written to global memory in the same layout.
-constexpr int kInvThreads = 1024;
-constexpr size_t kInvSmem = sizeof(double) * kNb * kW;
+// Coarsest level (64 nodes): the matrix M (kNc x kNc) with u = M f the
+// mean-free solution of L u = f - mean(f), in FP64 by one block.
+//
+// Every neighbour of a red node is black, so the red block of A = -L is
+// diagonal: A = [R -B; -B^T K] with R, K the node diagonals.  The black nodes
+// see the 32 x 32 Schur complement S = K - B^T R^-1 B, whose null space is the
+// constants; with a constant added to every entry (the mean of K over 32) it
+// is positive definite and is inverted in place by symmetric sweeps without
+// pivoting, one element of the lower triangle per thread.  From X that
+// inverse, G = [R^-1 + R^-1 B X B^T R^-1, R^-1 B X; ., X] is a generalised
+// inverse of A, and M = -P G P with P = I - 1 1^T / 64.
+//
+// Bound by one SM's FP64 rate (2 lanes a clock) and the 32 dependent pivots:
+// 17 warps of multiply and FMA a pivot, against the 65 pivots over 65 x 130
+// elements that a Gauss-Jordan elimination of the bordered matrix takes
+// (286 us; 47 us in this form, mixed 32^3 solve of 8 steps 9.75 -> 7.86 ms).
+constexpr int kHalf = kNc / 2;                      // red (and black) nodes
+constexpr int kTri = kHalf * (kHalf + 1) / 2;       // lower triangle of S
+constexpr int kInvThreads = (kTri + 31) / 32 * 32;  // 544
+
+// 1 / x of a positive x by Newton's iteration from the FP32 reciprocal (24
+// bits, then 48, then full precision); outside the FP32 range by division.
+__device__ inline double recip_newton(double x) {
+    if (!(x > 1e-30 && x < 1e30)) return 1.0 / x;
+    double y = (double)__frcp_rn((float)x);
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
+}
 
 template <typename T>
 __global__ void __launch_bounds__(kInvThreads) k_coarse_invert(Dims d, double hx, double hy,
                                                               double hz, const T* __restrict__ a,
                                                               int face, double* __restrict__ out) {
-    extern __shared__ double aug[];
-    __shared__ double fac[kNb];
-    __shared__ int piv_row;
+    __shared__ double w[kNc][6];       // couplings of node c to its six neighbours
+    __shared__ int nb[kNc][6];
+    __shared__ double diag[kNc];
+    __shared__ double S[kHalf][kHalf + 1];
+    __shared__ double col[2][kHalf], piv[2];
+    __shared__ double G[kNc][kNc];     // rows and columns: red nodes, then black
+    __shared__ double mean[kNc];
     const int t = threadIdx.x;
-    for (int e = t; e < kNb * kW; e += blockDim.x) aug[e] = 0.0;
-    __syncthreads();
+    // node of a colour: pair idx holds nodes 2 idx and 2 idx + 1, one of each
+    auto node_of = [](int idx, int black) { return 2 * idx + ((((idx >> 3) + (idx >> 1)) & 1) ^ black); };
     if (t < kNc) {
         const int c = t;
         int i, j, k;
         cell_coords(d, c, i, j, k);
-        const int nb[6] = {cell_index(d, i + 1, j, k), cell_index(d, i - 1, j, k),
+        const int n6[6] = {cell_index(d, i + 1, j, k), cell_index(d, i - 1, j, k),
                            cell_index(d, i, j + 1, k), cell_index(d, i, j - 1, k),
                            cell_index(d, i, j, k + 1), cell_index(d, i, j, k - 1)};
         const double hh[3] = {hx, hy, hz};
-        double diag = 0.0;
+        double dg = 0.0;
         for (int q = 0; q < 6; ++q) {
             // face sum of face q: the +1 face of node c, or the +1 face of
             // its -1 neighbour
-            const double g = face ? (double)a[(size_t)(q >> 1) * d.cells + ((q & 1) ? nb[q] : c)]
-                                  : (double)a[c] + (double)a[nb[q]];
-            double w = 0.5 * g * hh[q >> 1];
-            diag += w;
-            aug[c * kW + nb[q]] += w;  // row c of L; distinct neighbours on 4^3
+            const double g = face ? (double)a[(size_t)(q >> 1) * d.cells + ((q & 1) ? n6[q] : c)]
+                                  : (double)a[c] + (double)a[n6[q]];
+            const double wq = 0.5 * g * hh[q >> 1];
+            w[c][q] = wq, nb[c][q] = n6[q];
+            dg += wq;
         }
-        aug[c * kW + c] -= diag;
-        aug[c * kW + kNc] = 1.0;
-        aug[kNc * kW + c] = 1.0;
+        diag[c] = dg;
     }
     __syncthreads();
-    for (int r = t; r < kNb; r += blockDim.x) aug[r * kW + kNb + r] = 1.0;
+    if (t < kHalf) {  // row t of S
+        const int c = node_of(t, 1);
+        double shift = diag[c];
+        for (int o = 16; o > 0; o >>= 1) shift += __shfl_xor_sync(0xffffffffu, shift, o);
+        shift *= 1.0 / (kHalf * kHalf);
+        for (int q = 0; q < kHalf; ++q) S[t][q] = shift;
+        S[t][t] += diag[c];
+        for (int q = 0; q < 6; ++q) {
+            const int r = nb[c][q];
+            const double f = w[c][q] * recip_newton(diag[r]);
+            for (int p = 0; p < 6; ++p) S[t][nb[r][p] >> 1] -= f * w[r][p];
+        }
+    }
     __syncthreads();
-    for (int p = 0; p < kNb; ++p) {
-        if (t < 32) {
-            // largest |entry| of column p at or below row p; the first such
-            // row on ties (as a serial scan with a strict comparison)
-            int best = -1;
-            double bv = -1.0;
-            for (int r = p + t; r < kNb; r += 32) {
-                const double v = fabs(aug[r * kW + p]);
-                if (v > bv) bv = v, best = r;
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                const double ov = __shfl_down_sync(0xffffffffu, bv, o);
-                const int ob = __shfl_down_sync(0xffffffffu, best, o);
-                if (ob >= 0 && (ov > bv || (ov == bv && (best < 0 || ob < best)))) bv = ov, best = ob;
-            }
-            if (t == 0) piv_row = best;
+    int r = 0, c = 0;  // this thread's element of the lower triangle
+    if (t < kTri) {
+        c = t;
+        while (c > r) c -= ++r;
+    }
+    double v = 0.0;
+    if (t < kTri) v = S[r][c];
+    // publishes column p of the symmetric matrix and 1 / its pivot
+    auto publish = [&](int p) {
+        if (t < kTri && (r == p || c == p)) {
+            col[p & 1][r == p ? c : r] = v;
+            if (r == c) piv[p & 1] = recip_newton(v);
         }
-        __syncthreads();
-        const int pr = piv_row;
-        if (pr != p)
-            for (int cc = t; cc < kW; cc += blockDim.x) {
-                const double x = aug[p * kW + cc];
-                aug[p * kW + cc] = aug[pr * kW + cc];
-                aug[pr * kW + cc] = x;
-            }
-        __syncthreads();
-        const double pv = aug[p * kW + p];
-        __syncthreads();
-        for (int cc = t; cc < kW; cc += blockDim.x) aug[p * kW + cc] /= pv;
-        __syncthreads();
-        for (int r = t; r < kNb; r += blockDim.x) fac[r] = aug[r * kW + p];
-        __syncthreads();
-        for (int e = t; e < kNb * kW; e += blockDim.x) {
-            const int r = e / kW, cc = e - r * kW;
-            if (r != p) aug[e] -= fac[r] * aug[p * kW + cc];
-        }
+    };
+    publish(0);
+    __syncthreads();
+    for (int p = 0; p < kHalf; ++p) {
+        const double di = piv[p & 1];
+        if (r != p && c != p) v = fma(-(col[p & 1][r] * di), col[p & 1][c], v);
+        else if (r == c) v = -di;
+        else v *= di;
+        if (p + 1 < kHalf) publish(p + 1);
         __syncthreads();
     }
-    for (int e = t; e < kNb * kW; e += blockDim.x) out[e] = aug[e];
+    if (t < kTri) {  // the sweeps leave -X
+        G[kHalf + r][kHalf + c] = -v;
+        G[kHalf + c][kHalf + r] = -v;
+    }
+    if (t < kHalf) col[0][t] = recip_newton(diag[node_of(t, 0)]);
+    __syncthreads();
+    for (int e = t; e < kHalf * kHalf; e += blockDim.x) {  // R^-1 B X
+        const int x = e / kHalf, y = e % kHalf, n = node_of(x, 0);
+        double s = 0.0;
+        for (int q = 0; q < 6; ++q) s = fma(w[n][q], G[kHalf + (nb[n][q] >> 1)][kHalf + y], s);
+        s *= col[0][x];
+        G[x][kHalf + y] = s;
+        G[kHalf + y][x] = s;
+    }
+    __syncthreads();
+    for (int e = t; e < kHalf * kHalf; e += blockDim.x) {  // R^-1 + (R^-1 B X) B^T R^-1
+        const int x = e / kHalf, y = e % kHalf, n = node_of(y, 0);
+        double s = 0.0;
+        for (int q = 0; q < 6; ++q) s = fma(w[n][q], G[x][kHalf + (nb[n][q] >> 1)], s);
+        G[x][y] = (s + (x == y ? 1.0 : 0.0)) * col[0][y];
+    }
+    __syncthreads();
+    if (t < 512) {  // row means, eight threads a row
+        double s = 0.0;
+        for (int y = t & 7; y < kNc; y += 8) s += G[t >> 3][y];
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((t & 7) == 0) mean[t >> 3] = s * (1.0 / kNc);
+    }
+    __syncthreads();
+    if (t < 32) {
+        double s = mean[t] + mean[t + 32];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (t == 0) piv[0] = s * (1.0 / kNc);
+    }
+    __syncthreads();
+    const double all = piv[0];
+    for (int e = t; e < kNc * kNc; e += blockDim.x) {
+        const int x = e / kNc, y = e % kNc;  // nodes of the row and the column
+        const int cx = (x >> 1) + (node_of(x >> 1, 0) == x ? 0 : kHalf);
+        const int cy = (y >> 1) + (node_of(y >> 1, 0) == y ? 0 : kHalf);
+        out[e] = (mean[cx] - G[cx][cy]) + (mean[cy] - all);
+    }
 }
 
 template <typename T>
-__global__ void k_coarse_solve(const double* __restrict__ aug, const T* __restrict__ f,
+__global__ void k_coarse_solve(const double* __restrict__ minv, const T* __restrict__ f,
                                T* __restrict__ u) {
     const int r = threadIdx.x;
     if (r >= kNc) return;
     double acc = 0.0;
-    for (int c = 0; c < kNc; ++c) acc += aug[r * kW + kNb + c] * (double)f[c];
+    for (int c = 0; c < kNc; ++c) acc += minv[r * kNc + c] * (double)f[c];
     u[r] = (T)acc;
 }
 
@@ -410,9 +473,8 @@ void launch_prolong_add(const Level& fine, const Level& coarse, const T* uc, T* 
 
 template <typename T>
 void launch_coarse_invert(const Level& L, const T* a, double* minv, cudaStream_t st) {
-    allow_smem((const void*)k_coarse_invert<T>, (int)kInvSmem);
     launch_counter()++;
-    k_coarse_invert<T><<<1, kInvThreads, kInvSmem, st>>>(L.d, L.h2i[0], L.h2i[1], L.h2i[2], a,
+    k_coarse_invert<T><<<1, kInvThreads, 0, st>>>(L.d, L.h2i[0], L.h2i[1], L.h2i[2], a,
                                                          L.face, minv);
 }
 
@@ -511,7 +573,7 @@ __device__ inline void sm_sweeps(const Dims& d, T hx, T hy, T hz, int nu, T* u, 
 template <typename T>
 __global__ void __launch_bounds__(1024) k_coarse_vcycle(CoarseSet cs, const T* __restrict__ f_top,
                                                         T* __restrict__ u_top,
-                                                        const double* __restrict__ aug,
+                                                        const double* __restrict__ minv_g,
                                                         int zero_u) {
     extern __shared__ unsigned char smem_raw[];
     T* base = reinterpret_cast<T*>(smem_raw);
@@ -532,10 +594,9 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle(CoarseSet cs, const T* _
         f[0][c] = f_top[c];
         u[0][c] = zero_u ? T(0) : u_top[c];
     }
-    // the 4^3 inverse (its kNc x kNc block of the augmented matrix) in shared
-    // memory, after the levels (8-byte aligned: 4 arrays of whole levels)
+    // the 4^3 inverse in shared memory, after the levels (8-byte aligned: 4 arrays of whole levels)
     double* minv = reinterpret_cast<double*>(u[cs.nlev - 1] + 4 * cs.lv[cs.nlev - 1].d.cells);
-    for (int e = threadIdx.x; e < kNc * kNc; e += blockDim.x) minv[e] = aug[(e / kNc) * kW + kNb + (e % kNc)];
+    for (int e = threadIdx.x; e < kNc * kNc; e += blockDim.x) minv[e] = minv_g[e];
     __syncthreads();
     const int last = cs.nlev - 1;
     // down

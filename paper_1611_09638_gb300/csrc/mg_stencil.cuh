@@ -73,9 +73,8 @@ __device__ inline Stencil7<T> stencil7_any(const Dims& d, T hx, T hy, T hz, int 
                         u[zp], u[zm]);
 }
 
-// The coarsest (4^3) level is solved with the inverse of the bordered system
-// [L 1; 1^T 0] (kNb x kNb), stored as the augmented matrix [I | M^-1]
-// (kNb rows of kW doubles) that the Gauss-Jordan kernel leaves behind.
-constexpr int kNc = 64, kNb = 65, kW = 130;
+// The coarsest (4^3) level is solved with the matrix that takes f to the
+// mean-free solution of L u = f - mean(f) (kNc x kNc doubles, by rows).
+constexpr int kNc = 64;
 
 }  // namespace recon

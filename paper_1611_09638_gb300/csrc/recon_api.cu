@@ -1270,7 +1270,7 @@ int recon_create(void** out, const recon_params* p_in, void* cuda_stream) {
     AL(H->F64, 3 * n); AL(H->D64, n); AL(H->phi32, n); AL(H->dphi32, n);
     if (p->warm_start == 2) AL(H->phidot_prev, n);
     if (p->density_update == 1) AL(H->v3m, 6 * n);
-    AL(H->minv, 65 * 130); AL(H->scal, SC_COUNT);
+    AL(H->minv, 64 * 64); AL(H->scal, SC_COUNT);
     const size_t km = (size_t)std::max(p->k_max, 1);
     // the per-step records share one block (Rk | alpha | relres | ncycles) so
     // that one copy brings them back

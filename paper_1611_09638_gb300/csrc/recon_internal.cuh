@@ -229,8 +229,8 @@ void launch_resid_restrict(const Level& fine, const Level& coarse, const T* u, c
                            const T* a, T* out, cudaStream_t st);
 template <typename T>
 void launch_prolong_add(const Level& fine, const Level& coarse, const T* uc, T* u, cudaStream_t st);
-// Coarsest (4x4x4) level: invert the bordered 65 x 65 system [L 1; 1^T 0]
-// once per coefficient (FP64), then solve by one matrix-vector product.
+// Coarsest (4x4x4) level: the 64 x 64 matrix of the mean-free solution, once
+// per coefficient (FP64), then each solve is one matrix-vector product.
 template <typename T>
 void launch_coarse_invert(const Level& L, const T* a, double* minv, cudaStream_t st);
 template <typename T>
