@@ -335,8 +335,6 @@ bool launch_coarse_cluster(const CoarseSet& cs, const T* f, T* u, const double* 
 
 template bool launch_coarse_cluster<float>(const CoarseSet&, const float*, float*, const double*, bool,
                                            cudaStream_t);
-template bool launch_coarse_cluster<double>(const CoarseSet&, const double*, double*, const double*, bool,
-                                            cudaStream_t);
 
 int bounds_fail_cluster() { return bounds_fail_take(); }
 

@@ -35,14 +35,18 @@ __global__ void k_rbgs_colour(Dims d, T hx, T hy, T hz, int colour, T* __restric
     u[c] = (s.off - f[c]) / s.diag;
 }
 
-// One colour of a red-black sweep of the finest FP64 level (unit spacing)
-// from the stored face coefficients A = (a_c + a_n) / 2 (F: +x, +y, +z face
-// of each node) and the inverse of the node's diagonal D = sum of its six A:
+// One colour of a red-black sweep of an FP64 level from its stored face
+// coefficients A = h^-2 (a_c + a_n) / 2 (F: +x, +y, +z face of each node) and
+// the inverse of the node's diagonal D = sum of its six A:
 // u_c = (sum_n A_n u_n - f_c) / D_c in 8 FP64 instructions per node, since
-// FP64 issue, not memory, bounds this sweep on GB300.
-__global__ void k_rbgs_colour64_unit(Dims d, int colour, double* __restrict__ u,
-                                     const double* __restrict__ f, const double* __restrict__ F,
-                                     const double* __restrict__ inv_d) {
+// FP64 issue (2 lanes a clock and SM), not memory, bounds this sweep on GB300:
+// 18.3 us a colour of 128^3 against 13.6 us of issue.  Forming the faces and
+// dividing in each sweep took some 45 instructions, 14 us a colour of 64^3.
+// zero: u is 0 on entry and is not read (the red colour of a first sweep; the
+// black one reads red values only, so u need not be cleared).
+__global__ void k_rbgs_colour64(Dims d, int colour, int zero, double* __restrict__ u,
+                                const double* __restrict__ f, const double* __restrict__ F,
+                                const double* __restrict__ inv_d) {
     const int half = d.cells >> 1;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= half) return;
@@ -52,6 +56,10 @@ __global__ void k_rbgs_colour64_unit(Dims d, int colour, double* __restrict__ u,
     const int i = t >> (d.s1 + hs2);
     const int k = 2 * kk + ((i + j + colour) & 1);
     const int c = cell_index(d, i, j, k);
+    if (zero) {
+        u[c] = -f[c] * inv_d[c];
+        return;
+    }
     const int n0 = cell_index(d, i + 1, j, k), n1 = cell_index(d, i - 1, j, k);
     const int n2 = cell_index(d, i, j + 1, k), n3 = cell_index(d, i, j - 1, k);
     const int n4 = cell_index(d, i, j, k + 1), n5 = cell_index(d, i, j, k - 1);
@@ -63,6 +71,29 @@ __global__ void k_rbgs_colour64_unit(Dims d, int colour, double* __restrict__ u,
     o = fma(F[2 * n + c], u[n4], o);
     o = fma(F[2 * n + n5], u[n5], o);
     u[c] = (o - f[c]) * inv_d[c];
+}
+
+// r = f - L u of an FP64 level, from the same coefficients, for the
+// restriction: 7 FMAs a node.  Restricting a stored residual instead of
+// evaluating it at the 27 fine nodes of every coarse node (each evaluation
+// with its faces) takes this step at 128^3 from 280 to 45 us.
+__global__ void k_residual64(Dims d, const double* __restrict__ u, const double* __restrict__ f,
+                             const double* __restrict__ F, const double* __restrict__ D,
+                             double* __restrict__ r) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= d.cells) return;
+    int i, j, k;
+    cell_coords(d, c, i, j, k);
+    const size_t n = (size_t)d.cells;
+    const int n1 = cell_index(d, i - 1, j, k), n3 = cell_index(d, i, j - 1, k), n5 = cell_index(d, i, j, k - 1);
+    double v = fma(D[c], u[c], f[c]);
+    v = fma(-F[c], u[cell_index(d, i + 1, j, k)], v);
+    v = fma(-F[n1], u[n1], v);
+    v = fma(-F[n + c], u[cell_index(d, i, j + 1, k)], v);
+    v = fma(-F[n + n3], u[n3], v);
+    v = fma(-F[2 * n + c], u[cell_index(d, i, j, k + 1)], v);
+    v = fma(-F[2 * n + n5], u[n5], v);
+    r[c] = v;
 }
 
 // FP64 residual r = f - L u of the finest level (unit spacing) from the
@@ -115,10 +146,11 @@ __global__ void k_residual64_to32(Dims d, const double* __restrict__ u,
     if (threadIdx.x == 0) partials[blockIdx.x] = acc;
 }
 
-// Face coefficients A = (a_c + a_{c + e_a}) / 2 of a unit-spacing level, one
-// array per axis, the node diagonal D = sum of the node's six A, and
-// optionally 1 / D.
-__global__ void k_faces64(Dims d, const double* __restrict__ a, double* __restrict__ F,
+// Face coefficients A = h^-2 (a_c + a_{c + e_a}) / 2 of a level, one array per
+// axis (wx, wy, wz: h^-2 / 2 of that axis), the node diagonal D = sum of the
+// node's six A, and optionally 1 / D.
+__global__ void k_faces64(Dims d, double wx, double wy, double wz, const double* __restrict__ a,
+                          double* __restrict__ F,
                           double* __restrict__ D, double* __restrict__ inv_d) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= d.cells) return;
@@ -126,12 +158,12 @@ __global__ void k_faces64(Dims d, const double* __restrict__ a, double* __restri
     cell_coords(d, c, i, j, k);
     const size_t n = (size_t)d.cells;
     const double ac = a[c];
-    const double xp = 0.5 * (ac + a[cell_index(d, i + 1, j, k)]);
-    const double xm = 0.5 * (ac + a[cell_index(d, i - 1, j, k)]);
-    const double yp = 0.5 * (ac + a[cell_index(d, i, j + 1, k)]);
-    const double ym = 0.5 * (ac + a[cell_index(d, i, j - 1, k)]);
-    const double zp = 0.5 * (ac + a[cell_index(d, i, j, k + 1)]);
-    const double zm = 0.5 * (ac + a[cell_index(d, i, j, k - 1)]);
+    const double xp = wx * (ac + a[cell_index(d, i + 1, j, k)]);
+    const double xm = wx * (ac + a[cell_index(d, i - 1, j, k)]);
+    const double yp = wy * (ac + a[cell_index(d, i, j + 1, k)]);
+    const double ym = wy * (ac + a[cell_index(d, i, j - 1, k)]);
+    const double zp = wz * (ac + a[cell_index(d, i, j, k + 1)]);
+    const double zm = wz * (ac + a[cell_index(d, i, j, k - 1)]);
     F[c] = xp, F[n + c] = yp, F[2 * n + c] = zp;
     const double dg = ((xp + xm) + (yp + ym)) + (zp + zm);
     D[c] = dg;
@@ -159,6 +191,32 @@ __global__ void k_restrict(Dims df, Dims dc, int cx, int cy, int cz, const T* __
         }
     }
     out[c] = acc;
+}
+
+// Full weighting in FP64 one axis after another, halved once at the end: 2
+// FP64 instructions a value and axis instead of 4 a stencil point.
+__device__ inline double full_weight(const Dims& df, const Dims& dc, int cx, int cy, int cz,
+                                     const double* __restrict__ in, int c) {
+    int I, J, K;
+    cell_coords(dc, c, I, J, K);
+    const int fi = cx ? 2 * I : I, fj = cy ? 2 * J : J, fk = cz ? 2 * K : K;
+    auto along_k = [&](int i, int j) {
+        const double v = in[cell_index(df, i, j, fk)];
+        return cz ? fma(0.5, in[cell_index(df, i, j, fk - 1)] + in[cell_index(df, i, j, fk + 1)], v) : v;
+    };
+    auto along_j = [&](int i) {
+        const double v = along_k(i, fj);
+        return cy ? fma(0.5, along_k(i, fj - 1) + along_k(i, fj + 1), v) : v;
+    };
+    double acc = along_j(fi);
+    if (cx) acc = fma(0.5, along_j(fi - 1) + along_j(fi + 1), acc);
+    return acc * ((cx ? 0.5 : 1.0) * ((cy ? 0.5 : 1.0) * (cz ? 0.5 : 1.0)));
+}
+
+__global__ void k_restrict64(Dims df, Dims dc, int cx, int cy, int cz, const double* __restrict__ in,
+                             double* __restrict__ out) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c < dc.cells) out[c] = full_weight(df, dc, cx, cy, cz, in, c);
 }
 
 // Residual r = f - L u evaluated at the fine nodes of each coarse node's
@@ -263,6 +321,59 @@ __global__ void k_prolong_add(Dims df, Dims dc, int cx, int cy, int cz, const T*
             for (int r = 0; r < nk; ++r)
                 acc += wi[p] * wj[q] * wk[r] * uc[cell_index(dc, ii[p], jj[q], kk[r])];
     u[c] += acc;
+}
+
+// Trilinear prolongation in FP64 as one sum per node, weighted once (1/2 per
+// odd coarsened axis); returns v + P(uc) at fine node c.
+__device__ inline double prolonged(const Dims& df, const Dims& dc, int cx, int cy, int cz,
+                                   const double* __restrict__ uc, int c, double v) {
+    int i, j, k;
+    cell_coords(df, c, i, j, k);
+    const int oi = cx & i, oj = cy & j, ok = cz & k;  // odd along a coarsened axis
+    const int I = cx ? i >> 1 : i, J = cy ? j >> 1 : j, K = cz ? k >> 1 : k;
+    double acc = 0.0;
+    for (int p = 0; p <= oi; ++p)
+        for (int q = 0; q <= oj; ++q)
+            for (int r = 0; r <= ok; ++r) acc += uc[cell_index(dc, I + p, J + q, K + r)];
+    return fma(acc, (oi ? 0.5 : 1.0) * ((oj ? 0.5 : 1.0) * (ok ? 0.5 : 1.0)), v);
+}
+
+__global__ void k_prolong_add64(Dims df, Dims dc, int cx, int cy, int cz, const double* __restrict__ uc,
+                                double* __restrict__ u) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c < df.cells) u[c] = prolonged(df, dc, cx, cy, cz, uc, c, u[c]);
+}
+
+// The same where k is coarsened, a thread a pair (2K, 2K + 1) of fine nodes:
+// the sums over the coarse rows around the pair serve both nodes, 2.75 FP64
+// instructions a node on average (the FP64 rate bounds it) against 7.5 with a
+// thread a node, whose warps also run the odd nodes' longer sums for all
+// (128^3: 42 -> 16 us).
+__global__ void k_prolong_pair64(Dims df, Dims dc, int cx, int cy, const double* __restrict__ uc,
+                                 double* __restrict__ u) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= df.cells >> 1) return;
+    int i, j, k;
+    cell_coords(df, 2 * t, i, j, k);
+    const int oi = cx & i, oj = cy & j;
+    const int I = cx ? i >> 1 : i, J = cy ? j >> 1 : j, K = k >> 1;
+    auto rows = [&](int kk) {
+        double s = uc[cell_index(dc, I, J, kk)];
+        if (oi) s += uc[cell_index(dc, I + 1, J, kk)];
+        if (oj) {
+            s += uc[cell_index(dc, I, J + 1, kk)];
+            if (oi) s += uc[cell_index(dc, I + 1, J + 1, kk)];
+        }
+        return s;
+    };
+    const double a = rows(K), b = rows(K + 1);
+    const int halvings = oi + oj;
+    const double w = halvings == 0 ? 1.0 : halvings == 1 ? 0.5 : 0.25;
+    double2* p = reinterpret_cast<double2*>(u + 2 * t);
+    double2 v = *p;
+    v.x = fma(a, w, v.x);
+    v.y = fma(a + b, halvings == 0 ? 0.5 : halvings == 1 ? 0.25 : 0.125, v.y);
+    *p = v;
 }
 
 // Coarsest level (64 nodes): the matrix M (kNc x kNc) with u = M f the
@@ -442,10 +553,19 @@ void launch_rbgs_sweep(const Level& L, T* u, const T* f, const T* a, cudaStream_
                                                              (T)L.h2i[2], colour, u, f, a, L.face);
 }
 
-template <typename T>
-void launch_restrict(const Level& fine, const Level& coarse, const T* in, T* out, cudaStream_t st) {
+template <>
+void launch_restrict<float>(const Level& fine, const Level& coarse, const float* in, float* out,
+                            cudaStream_t st) {
     launch_counter()++;
-    k_restrict<T><<<nblocks(coarse.d.cells), kThreads, 0, st>>>(
+    k_restrict<float><<<nblocks(coarse.d.cells), kThreads, 0, st>>>(
+        fine.d, coarse.d, fine.coarsen[0], fine.coarsen[1], fine.coarsen[2], in, out);
+}
+
+template <>
+void launch_restrict<double>(const Level& fine, const Level& coarse, const double* in, double* out,
+                             cudaStream_t st) {
+    launch_counter()++;
+    k_restrict64<<<nblocks(coarse.d.cells), kThreads, 0, st>>>(
         fine.d, coarse.d, fine.coarsen[0], fine.coarsen[1], fine.coarsen[2], in, out);
 }
 
@@ -464,10 +584,24 @@ void launch_faces_line(const Level& fine, const Level& coarse, const float* in, 
     k_faces_line<<<nblocks(coarse.d.cells), kThreads, 0, st>>>(fine.d, coarse.d, in, fine.face, out);
 }
 
-template <typename T>
-void launch_prolong_add(const Level& fine, const Level& coarse, const T* uc, T* u, cudaStream_t st) {
+template <>
+void launch_prolong_add<float>(const Level& fine, const Level& coarse, const float* uc, float* u,
+                               cudaStream_t st) {
     launch_counter()++;
-    k_prolong_add<T><<<nblocks(fine.d.cells), kThreads, 0, st>>>(
+    k_prolong_add<float><<<nblocks(fine.d.cells), kThreads, 0, st>>>(
+        fine.d, coarse.d, fine.coarsen[0], fine.coarsen[1], fine.coarsen[2], uc, u);
+}
+
+template <>
+void launch_prolong_add<double>(const Level& fine, const Level& coarse, const double* uc, double* u,
+                                cudaStream_t st) {
+    launch_counter()++;
+    if (fine.coarsen[2]) {
+        k_prolong_pair64<<<nblocks(fine.d.cells >> 1), kThreads, 0, st>>>(fine.d, coarse.d, fine.coarsen[0],
+                                                                          fine.coarsen[1], uc, u);
+        return;
+    }
+    k_prolong_add64<<<nblocks(fine.d.cells), kThreads, 0, st>>>(
         fine.d, coarse.d, fine.coarsen[0], fine.coarsen[1], fine.coarsen[2], uc, u);
 }
 
@@ -501,18 +635,26 @@ void launch_residual_norm64(const Level& L, const double* u, const double* f, co
     k_residual64_to32<<<kRedBlocks, kRedThreads, 0, st>>>(L.d, u, f, F, D, nullptr, partials);
 }
 
-void launch_rbgs_sweep64_unit(const Level& L, double* u, const double* f, const double* F,
-                              const double* inv_d, cudaStream_t st) {
+void launch_rbgs_sweep64(const Level& L, double* u, const double* f, const double* F,
+                         const double* inv_d, bool zero_u, cudaStream_t st) {
     const int half = L.d.cells >> 1;
     launch_counter() += 2;
     for (int colour = 0; colour < 2; ++colour)
-        k_rbgs_colour64_unit<<<nblocks(half), kThreads, 0, st>>>(L.d, colour, u, f, F, inv_d);
+        k_rbgs_colour64<<<nblocks(half), kThreads, 0, st>>>(L.d, colour, zero_u && colour == 0 ? 1 : 0, u, f, F,
+                                                            inv_d);
+}
+
+void launch_residual64(const Level& L, const double* u, const double* f, const double* F, const double* D,
+                       double* r, cudaStream_t st) {
+    launch_counter()++;
+    k_residual64<<<nblocks(L.d.cells), kThreads, 0, st>>>(L.d, u, f, F, D, r);
 }
 
 void launch_faces64(const Level& L, const double* a, double* F, double* D, double* inv_d,
                     cudaStream_t st) {
     launch_counter()++;
-    k_faces64<<<nblocks(L.d.cells), kThreads, 0, st>>>(L.d, a, F, D, inv_d);
+    k_faces64<<<nblocks(L.d.cells), kThreads, 0, st>>>(L.d, 0.5 * L.h2i[0], 0.5 * L.h2i[1], 0.5 * L.h2i[2], a, F,
+                                                       D, inv_d);
 }
 
 void launch_correct(int cells, double* u, const float* e, cudaStream_t st) {
@@ -520,18 +662,12 @@ void launch_correct(int cells, double* u, const float* e, cudaStream_t st) {
     k_correct<<<nblocks(cells), kThreads, 0, st>>>(cells, u, e);
 }
 
-#define RECON_INSTANTIATE(T)                                                                    \
-    template void launch_rbgs_sweep<T>(const Level&, T*, const T*, const T*, cudaStream_t);   \
-    template void launch_restrict<T>(const Level&, const Level&, const T*, T*, cudaStream_t);  \
-    template void launch_resid_restrict<T>(const Level&, const Level&, const T*, const T*,     \
-                                           const T*, T*, cudaStream_t);                       \
-    template void launch_prolong_add<T>(const Level&, const Level&, const T*, T*,              \
-                                        cudaStream_t);                                        \
-    template void launch_coarse_invert<T>(const Level&, const T*, double*, cudaStream_t);      \
-    template void launch_coarse_solve<T>(const double*, const T*, T*, cudaStream_t);
-RECON_INSTANTIATE(float)
-RECON_INSTANTIATE(double)
-#undef RECON_INSTANTIATE
+template void launch_rbgs_sweep<float>(const Level&, float*, const float*, const float*, cudaStream_t);
+template void launch_resid_restrict<float>(const Level&, const Level&, const float*, const float*,
+                                           const float*, float*, cudaStream_t);
+template void launch_coarse_invert<float>(const Level&, const float*, double*, cudaStream_t);
+template void launch_coarse_invert<double>(const Level&, const double*, double*, cudaStream_t);
+template void launch_coarse_solve<float>(const double*, const float*, float*, cudaStream_t);
 
 }  // namespace recon
 
@@ -690,7 +826,107 @@ bool launch_coarse_vcycle(const CoarseSet& cs, const T* f_top, T* u_top, const d
 
 template bool launch_coarse_vcycle<float>(const CoarseSet&, const float*, float*, const double*,
                                           bool, cudaStream_t);
-template bool launch_coarse_vcycle<double>(const CoarseSet&, const double*, double*,
-                                           const double*, bool, cudaStream_t);
+// The same for FP64 levels (at most kCoarse64Cells nodes on the first), from
+// their stored faces and diagonals: 8 FP64 instructions a node and colour.
+// One block holds a level of 8^3 nodes (a node a thread and phase); above
+// that its two FP64 lanes a clock would bound it (329 us for one V(2,2) of
+// 32^3 over a cluster of 8 blocks with the faces formed in every phase;
+// 88 us as one launch per phase over the whole chip down to 8^3).
+namespace {
+
+__global__ void __launch_bounds__(512) k_coarse_vcycle64(CoarseSet64 cs, const double* __restrict__ f_top,
+                                                         double* __restrict__ u_top,
+                                                         const double* __restrict__ minv, int zero_u) {
+    extern __shared__ double sm64[];
+    double *u[kCoarseMaxLevels], *f[kCoarseMaxLevels], *r[kCoarseMaxLevels], *F[kCoarseMaxLevels],
+        *D[kCoarseMaxLevels], *I[kCoarseMaxLevels];
+    double* q = sm64;
+    for (int l = 0; l < cs.nlev; ++l) {
+        const int n = cs.lv[l].d.cells;
+        u[l] = q, f[l] = q + n, r[l] = q + 2 * n, F[l] = q + 3 * n, D[l] = q + 6 * n, I[l] = q + 7 * n;
+        q += 8 * n;
+        if (l + 1 == cs.nlev) continue;  // the 4^3 level is solved with minv
+        for (int c = threadIdx.x; c < 3 * n; c += blockDim.x) F[l][c] = cs.F[l][c];
+        for (int c = threadIdx.x; c < n; c += blockDim.x) D[l][c] = cs.D[l][c], I[l][c] = cs.inv[l][c];
+    }
+    for (int c = threadIdx.x; c < cs.lv[0].d.cells; c += blockDim.x) {
+        f[0][c] = f_top[c];
+        u[0][c] = zero_u ? 0.0 : u_top[c];
+    }
+    double* mi = q;
+    for (int e = threadIdx.x; e < kNc * kNc; e += blockDim.x) mi[e] = minv[e];
+    __syncthreads();
+    // sum_n A_n u_n of node (i, j, k)
+    auto off = [&](int l, int i, int j, int k, int c) {
+        const Dims& d = cs.lv[l].d;
+        const int n = d.cells;
+        const int n1 = cell_index(d, i - 1, j, k), n3 = cell_index(d, i, j - 1, k), n5 = cell_index(d, i, j, k - 1);
+        double o = F[l][c] * u[l][cell_index(d, i + 1, j, k)];
+        o = fma(F[l][n1], u[l][n1], o);
+        o = fma(F[l][n + c], u[l][cell_index(d, i, j + 1, k)], o);
+        o = fma(F[l][n + n3], u[l][n3], o);
+        o = fma(F[l][2 * n + c], u[l][cell_index(d, i, j, k + 1)], o);
+        return fma(F[l][2 * n + n5], u[l][n5], o);
+    };
+    auto sweeps = [&](int l, int nu) {
+        const Dims& d = cs.lv[l].d;
+        const int half = d.cells >> 1, hs2 = d.s2 - 1;
+        for (int s = 0; s < 2 * nu; ++s) {
+            for (int t = threadIdx.x; t < half; t += blockDim.x) {
+                const int j = (t >> hs2) & (d.n1 - 1), i = t >> (d.s1 + hs2);
+                const int k = 2 * (t & ((1 << hs2) - 1)) + ((i + j + s) & 1);
+                const int c = cell_index(d, i, j, k);
+                u[l][c] = (off(l, i, j, k, c) - f[l][c]) * I[l][c];
+            }
+            __syncthreads();
+        }
+    };
+    const int last = cs.nlev - 1;
+    for (int l = 0; l < last; ++l) {
+        const Dims &d = cs.lv[l].d, &dc = cs.lv[l + 1].d;
+        sweeps(l, cs.nu1);
+        for (int c = threadIdx.x; c < d.cells; c += blockDim.x) {
+            int i, j, k;
+            cell_coords(d, c, i, j, k);
+            r[l][c] = fma(D[l][c], u[l][c], f[l][c]) - off(l, i, j, k, c);
+        }
+        __syncthreads();
+        for (int c = threadIdx.x; c < dc.cells; c += blockDim.x) {
+            f[l + 1][c] = full_weight(d, dc, cs.lv[l].coarsen[0], cs.lv[l].coarsen[1], cs.lv[l].coarsen[2], r[l], c);
+            u[l + 1][c] = 0.0;
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x < 4 * kNc) {  // u = M f, four threads a row
+        const int row = threadIdx.x >> 2;
+        double acc = 0.0;
+        for (int c = threadIdx.x & 3; c < kNc; c += 4) acc = fma(mi[row * kNc + c], f[last][c], acc);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        if ((threadIdx.x & 3) == 0) u[last][row] = acc;
+    }
+    __syncthreads();
+    for (int l = last - 1; l >= 0; --l) {
+        for (int c = threadIdx.x; c < cs.lv[l].d.cells; c += blockDim.x)
+            u[l][c] = prolonged(cs.lv[l].d, cs.lv[l + 1].d, cs.lv[l].coarsen[0], cs.lv[l].coarsen[1],
+                                cs.lv[l].coarsen[2], u[l + 1], c, u[l][c]);
+        __syncthreads();
+        sweeps(l, cs.nu2);
+    }
+    for (int c = threadIdx.x; c < cs.lv[0].d.cells; c += blockDim.x) u_top[c] = u[0][c];
+}
+
+}  // namespace
+
+void launch_coarse_vcycle64(const CoarseSet64& cs, const double* f_top, double* u_top, const double* minv,
+                            bool zero_u, cudaStream_t st) {
+    size_t cells = 0;
+    for (int l = 0; l < cs.nlev; ++l) cells += cs.lv[l].d.cells;
+    // at most 2 x kCoarse64Cells nodes over all levels
+    const size_t sm = (8 * cells + kNc * kNc) * sizeof(double);
+    allow_smem((const void*)k_coarse_vcycle64, (int)((16 * kCoarse64Cells + kNc * kNc) * sizeof(double)));
+    launch_counter()++;
+    k_coarse_vcycle64<<<1, 512, sm, st>>>(cs, f_top, u_top, minv, zero_u ? 1 : 0);
+}
 
 }  // namespace recon

@@ -71,7 +71,6 @@ struct Handle {
     void* stage = nullptr;
     size_t stage_bytes = 0;
     double* e6 = nullptr;  // triad I + Hess phi of the current step, 6 x cells
-    double* inv64 = nullptr;  // FP64 mode: 1 / diagonal of the finest level
     double* F64 = nullptr;    // face coefficients (a_c + a_{c+e}) / 2 of the finest level, 3 x cells
     double* D64 = nullptr;    // node diagonal: sum of the node's six face coefficients
     float *phi32 = nullptr, *dphi32 = nullptr;  // FP32 copies for the limiter's screen
@@ -79,10 +78,12 @@ struct Handle {
     unsigned long long* mfix = nullptr;
     // multigrid per level: FP64 (FP64 mode) or FP32 (mixed mode)
     std::vector<double*> u64, f64, c64, r64;
+    std::vector<double*> F64l, D64l, I64l;  // FP64 mode: each level's faces, diagonal and 1 / diagonal
     std::vector<float*> u32, f32, c32, r32;
     double* minv = nullptr;
     int l0 = -1;        // first level of the single-block coarse V-cycle
-    CoarseSet cs{};     // those levels and their coefficients
+    CoarseSet cs{};     // those levels and their coefficients (mixed mode)
+    CoarseSet64 cs64{};  // the same in FP64 mode
     int lc = -1;        // the 32^3 level whose V-cycle runs as one cluster launch
     CoarseSet cc{};     // the levels from it down
     double* part[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -212,14 +213,7 @@ void sweeps_unprofiled(Handle* H, int l, int nu, T** cur, T** oth, const T* f, c
             s += k;
         } else {
             if (zero) cudaMemsetAsync(*cur, 0, sizeof(T) * H->lv[l].d.cells, H->st);
-            if constexpr (sizeof(T) == sizeof(double)) {
-                if (l == 0 && H->inv64)
-                    launch_rbgs_sweep64_unit(H->lv[0], *cur, f, H->F64, H->inv64, H->st);
-                else
-                    launch_rbgs_sweep<T>(H->lv[l], *cur, f, c, H->st);
-            } else {
-                launch_rbgs_sweep<T>(H->lv[l], *cur, f, c, H->st);
-            }
+            launch_rbgs_sweep<T>(H->lv[l], *cur, f, c, H->st);
             s += 1;
         }
         zero = false;
@@ -415,9 +409,44 @@ bool vcycle(Handle* H, MG<T>& g, int l, T* u, const T* f, bool zero_u,
     return corrected;
 }
 
+// One V(nu1, nu2) cycle in FP64 of level l on L u = f, u updated in place
+// (zero_u: u = 0 on entry): every level sweeps with its stored faces, and its
+// residual is stored before it is restricted.
+void vcycle64(Handle* H, int l, double* u, const double* f, bool zero_u) {
+    if (l == H->l0) {
+        launch_coarse_vcycle64(H->cs64, f, u, H->minv, zero_u, H->st);
+        return;
+    }
+    const Level& L = H->lv[l];
+    auto sweeps = [&](int nu, bool zero) {
+        // the finest level's full sweeps are timed with params.profile
+        const bool mark = H->p.profile && l == 0 && nu > 0;
+        if (mark) prof_mark(H);
+        for (int s = 0; s < nu; ++s)
+            launch_rbgs_sweep64(L, u, f, H->F64l[l], H->I64l[l], zero && s == 0, H->st);
+        if (mark) prof_mark(H), H->prof_sweeps += nu;
+    };
+    if (zero_u && H->p.nu1 == 0) cudaMemsetAsync(u, 0, sizeof(double) * L.d.cells, H->st);
+    sweeps(H->p.nu1, zero_u);
+    launch_residual64(L, u, f, H->F64l[l], H->D64l[l], H->r64[l], H->st);
+    launch_restrict<double>(L, H->lv[l + 1], H->r64[l], H->f64[l + 1], H->st);
+    vcycle64(H, l + 1, H->u64[l + 1], H->f64[l + 1], true);
+    launch_prolong_add<double>(L, H->lv[l + 1], H->u64[l + 1], u, H->st);
+    sweeps(H->p.nu2, false);
+}
+
 template <typename T>
 void build_hierarchy(Handle* H, std::vector<T*>& c) {
-    launch_faces64(H->lv[0], H->a64, H->F64, H->D64, H->inv64, H->st);
+    if constexpr (sizeof(T) == sizeof(double)) {
+        for (size_t l = 0; l < H->lv.size(); ++l) {
+            if (l) launch_restrict<double>(H->lv[l - 1], H->lv[l], c[l - 1], c[l], H->st);
+            if (l + 1 < H->lv.size())
+                launch_faces64(H->lv[l], c[l], H->F64l[l], H->D64l[l], H->I64l[l], H->st);
+        }
+        launch_coarse_invert<double>(H->lv.back(), c.back(), H->minv, H->st);
+        return;
+    }
+    launch_faces64(H->lv[0], H->a64, H->F64, H->D64, nullptr, H->st);
     for (size_t l = 0; l + 1 < H->lv.size(); ++l) {
         if constexpr (sizeof(T) == sizeof(float)) {
             if (H->lv[l + 1].face) {
@@ -533,8 +562,7 @@ void mg_iter(Handle* H, const CtlHandles& h) {
         return;
     }
     if (!H->mixed) {
-        MG<double> g{H->u64, H->f64, H->c64, H->r64};
-        vcycle<double>(H, g, 0, H->phidot, H->s, false);
+        vcycle64(H, 0, H->phidot, H->s, false);
         launch_residual_norm64(L0, H->phidot, H->s, H->F64, H->D64, H->part[0], H->st);
     } else {
         MG<float> g{H->u32, H->f32, H->c32, H->r32};
@@ -1292,10 +1320,13 @@ int recon_create(void** out, const recon_params* p_in, void* cuda_stream) {
             H->r64.assign(nl, nullptr);
         H->u64[0] = H->phidot, H->f64[0] = H->s, H->c64[0] = H->a64;
         AL(H->r64[0], n);
-        AL(H->inv64, n);
+        H->F64l.assign(nl, nullptr), H->D64l.assign(nl, nullptr), H->I64l.assign(nl, nullptr);
+        H->F64l[0] = H->F64, H->D64l[0] = H->D64;
+        AL(H->I64l[0], n);
         for (int l = 1; l < nl; ++l) {
             size_t cl = H->lv[l].d.cells;
             AL(H->u64[l], cl); AL(H->f64[l], cl); AL(H->c64[l], cl); AL(H->r64[l], cl);
+            AL(H->F64l[l], 3 * cl); AL(H->D64l[l], cl); AL(H->I64l[l], cl);
         }
     } else {
         H->u32.assign(nl, nullptr), H->f32.assign(nl, nullptr), H->c32.assign(nl, nullptr),
@@ -1334,30 +1365,39 @@ int recon_create(void** out, const recon_params* p_in, void* cuda_stream) {
             return fail(RECON_E_CUDA, "tuning the streaming kernels failed");
         }
     }
-    // the levels from the first one of at most 16^3 nodes down run in one block
+    // the levels from the first one of at most 16^3 nodes (8^3 in FP64) down
+    // run in one block
     for (int l = 0; l < nl; ++l)
-        if (H->lv[l].d.cells <= 4096 && nl - l <= kCoarseMaxLevels && !H->lv[l].face) {
+        if (H->lv[l].d.cells <= (H->mixed ? 4096 : kCoarse64Cells) && nl - l <= kCoarseMaxLevels &&
+            !H->lv[l].face) {
             H->l0 = l;
             break;
         }
     // a 32^3 level with 16^3, 8^3 and 4^3 below it runs in one cluster launch
-    if (nl >= 4) {
+    if (H->mixed && nl >= 4) {
         CoarseSet& cc = H->cc;
         cc.nlev = 4;
         cc.nu1 = p->nu1, cc.nu2 = p->nu2;
         for (int l = 0; l < 4; ++l) {
             cc.lv[l] = H->lv[nl - 4 + l];
-            cc.a[l] = H->mixed ? (const void*)H->c32[nl - 4 + l] : (const void*)H->c64[nl - 4 + l];
+            cc.a[l] = (const void*)H->c32[nl - 4 + l];
         }
-        // (not the finest FP64 level, which sweeps with its stored faces)
-        if (coarse_cluster_fits(cc) && (H->mixed || nl > 4)) H->lc = nl - 4;
+        if (coarse_cluster_fits(cc)) H->lc = nl - 4;
     }
-    if (H->l0 >= 0) {
+    if (!H->mixed) {
+        CoarseSet64& cs = H->cs64;
+        cs.nlev = nl - H->l0;
+        cs.nu1 = p->nu1, cs.nu2 = p->nu2;
+        for (int l = H->l0; l < nl; ++l) {
+            cs.lv[l - H->l0] = H->lv[l];
+            cs.F[l - H->l0] = H->F64l[l], cs.D[l - H->l0] = H->D64l[l], cs.inv[l - H->l0] = H->I64l[l];
+        }
+    } else if (H->l0 >= 0) {
         H->cs.nlev = nl - H->l0;
         H->cs.nu1 = p->nu1, H->cs.nu2 = p->nu2;
         for (int l = H->l0; l < nl; ++l) {
             H->cs.lv[l - H->l0] = H->lv[l];
-            H->cs.a[l - H->l0] = H->mixed ? (const void*)H->c32[l] : (const void*)H->c64[l];
+            H->cs.a[l - H->l0] = (const void*)H->c32[l];
         }
     }
     if (cudaMallocHost((void**)&H->hscal, SC_COUNT * sizeof(double)) != cudaSuccess ||

@@ -235,15 +235,26 @@ template <typename T>
 void launch_coarse_invert(const Level& L, const T* a, double* minv, cudaStream_t st);
 template <typename T>
 void launch_coarse_solve(const double* minv, const T* f, T* u, cudaStream_t st);
-// V-cycle of the levels in cs in one block: L u = f on the first of them,
+// The FP64 levels from the first one of at most kCoarse64Cells nodes down, in
+// one block from their stored faces, diagonals and inverse diagonals.
+constexpr int kCoarse64Cells = 512;
+struct CoarseSet64 {
+    int nlev;
+    int nu1, nu2;
+    Level lv[kCoarseMaxLevels];
+    const double *F[kCoarseMaxLevels], *D[kCoarseMaxLevels], *inv[kCoarseMaxLevels];
+};
+void launch_coarse_vcycle64(const CoarseSet64& cs, const double* f_top, double* u_top, const double* minv,
+                            bool zero_u, cudaStream_t st);
+// V-cycle of the FP32 levels in cs in one block: L u = f on the first of them,
 // u updated in place (zero_u: u = 0 on entry, not read); returns false,
 // launching nothing, if they do not fit.
 template <typename T>
 bool launch_coarse_vcycle(const CoarseSet& cs, const T* f_top, T* u_top, const double* minv,
                           bool zero_u, cudaStream_t st);
-// Finest FP64 level (unit spacing): face coefficients F (3 x cells:
-// A = (a_c + a_{c+e}) / 2 for the +x, +y, +z face of each node), the node
-// diagonal D = sum of its six A, and optionally inv_d = 1 / D.
+// An FP64 level: face coefficients F (3 x cells: A = h^-2 (a_c + a_{c+e}) / 2
+// for the +x, +y, +z face of each node), the node diagonal D = sum of its six
+// A, and optionally inv_d = 1 / D.
 void launch_faces64(const Level& L, const double* a, double* F, double* D, double* inv_d,
                     cudaStream_t st);
 // FP64 residual of level 0 in mixed mode: r32 = f - L u (FP64), plus sum r^2
@@ -252,9 +263,13 @@ void launch_residual64_to32(const Level& L, const double* u, const double* f, co
 // FP64 residual norm only: partials of (f - L u)^2
 void launch_residual_norm64(const Level& L, const double* u, const double* f, const double* F,
                             const double* D, double* partials, cudaStream_t st);
-// FP64 red-black sweep of the finest level: u_c = (sum_n A_n u_n - f_c) / D_c
-void launch_rbgs_sweep64_unit(const Level& L, double* u, const double* f, const double* F,
-                              const double* inv_d, cudaStream_t st);
+// FP64 red-black sweep of a level from its stored faces and inverse diagonal:
+// u_c = (sum_n A_n u_n - f_c) / D_c; zero_u: u = 0 on entry, not read
+void launch_rbgs_sweep64(const Level& L, double* u, const double* f, const double* F,
+                         const double* inv_d, bool zero_u, cudaStream_t st);
+// FP64 residual r = f - L u of a level from its stored faces and diagonal
+void launch_residual64(const Level& L, const double* u, const double* f, const double* F, const double* D,
+                       double* r, cudaStream_t st);
 // u64 += e32
 void launch_correct(int cells, double* u, const float* e, cudaStream_t st);
 
