@@ -361,7 +361,7 @@ bool vcycle(Handle* H, MG<T>& g, int l, T* u, const T* f, bool zero_u,
             double* correct_into = nullptr) {
     const int last = (int)H->lv.size() - 1;
     const Level& L = H->lv[l];
-    if (l == H->lc && launch_coarse_cluster<T>(H->cc, f, u, H->minv, zero_u, H->st)) return false;
+    if (l == H->lc && launch_coarse_cluster(H->cc, f, u, H->minv, zero_u, 1, H->st)) return false;
     if (l == H->l0 && launch_coarse_vcycle<T>(H->cs, f, u, H->minv, zero_u, H->st)) return false;
     if (l == last) {
         launch_coarse_solve<T>(H->minv, f, u, H->st);
@@ -534,8 +534,10 @@ void mg_head(Handle* H, const CtlHandles& h, bool warm) {
 void mg_block(Handle* H, const CtlHandles& h) {
     MG<float> g{H->u32, H->f32, H->c32, H->r32};
     launch_zero_if_fresh(H->ctl, H->u32[0], H->cells, H->st);
-    for (int v = 0; v < H->p.inner_vcycles; ++v)
-        vcycle<float>(H, g, 0, H->u32[0], H->f32[0], false, nullptr);
+    // (a 32^3 finest level: all of them in one launch)
+    if (!(H->lc == 0 && launch_coarse_cluster(H->cc, H->f32[0], H->u32[0], H->minv, false, H->p.inner_vcycles, H->st)))
+        for (int v = 0; v < H->p.inner_vcycles; ++v)
+            vcycle<float>(H, g, 0, H->u32[0], H->f32[0], false, nullptr);
     launch_ctl_block(H->ctl, H->arr, H->p.inner_vcycles, H->p.max_vcycles, h, H->st);
 }
 
@@ -567,10 +569,12 @@ void mg_iter(Handle* H, const CtlHandles& h) {
     } else {
         MG<float> g{H->u32, H->f32, H->c32, H->r32};
         bool corrected = false;
-        for (int v = 0; v < H->p.inner_vcycles; ++v) {
-            const bool last = v + 1 == H->p.inner_vcycles;
-            corrected = vcycle<float>(H, g, 0, H->u32[0], H->f32[0], v == 0, last ? H->phidot : nullptr);
-        }
+        if (!(H->lc == 0 &&
+              launch_coarse_cluster(H->cc, H->f32[0], H->u32[0], H->minv, true, H->p.inner_vcycles, H->st)))
+            for (int v = 0; v < H->p.inner_vcycles; ++v) {
+                const bool last = v + 1 == H->p.inner_vcycles;
+                corrected = vcycle<float>(H, g, 0, H->u32[0], H->f32[0], v == 0, last ? H->phidot : nullptr);
+            }
         if (!corrected) launch_correct(H->cells, H->phidot, H->u32[0], H->st);
         launch_residual64_to32(L0, H->phidot, H->s, H->F64, H->D64, H->f32[0], H->part[0], H->st);
     }

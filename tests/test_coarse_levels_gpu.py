@@ -38,3 +38,20 @@ def test_coarse_levels_match_the_oracle(shape, precision):
         phi = R.field("phi").cpu().numpy()
     assert st.steps == ref.steps
     assert np.linalg.norm(phi - ref.phi) <= BARS[precision] * np.linalg.norm(ref.phi)
+
+
+@pytest.mark.parametrize("nu", [(1, 1), (2, 1), (0, 2), (2, 0)])
+@pytest.mark.parametrize("n,faces", [(32, 0), (64, 0), (64, 1)])
+def test_cluster_schedules_match_the_oracle(n, faces, nu):
+    """The cluster's V-cycle under every form of its schedule (no sweep before
+    the restriction, none after the prolongation) and both coefficient forms,
+    alone (32^3: several cycles a launch) and below a finer level."""
+    rho = _rough((n, n, n), 7 * n + faces)
+    ref = O.solve(O.OracleParams(n=(n, n, n), k_max=1), rho)
+    with Recon((n, n, n), precision="mixed", k_max=1, replay_alpha=ref.alpha, coarse_faces=faces,
+               nu1=nu[0], nu2=nu[1]) as R:
+        R.deposit_grid(torch.from_numpy(rho).cuda())
+        st = R.solve()
+        phi = R.field("phi").cpu().numpy()
+    assert st.steps == 1 and st.relres[0] <= 1e-8
+    assert np.linalg.norm(phi - ref.phi) <= BARS["mixed"] * np.linalg.norm(ref.phi)
