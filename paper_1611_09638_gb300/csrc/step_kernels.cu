@@ -340,67 +340,109 @@ __global__ void k_smooth_axis(Dims d, int axis, double ws, const double* __restr
     }
 }
 
-// S in one pass: a block takes SJ x SK tiles of the (j, k) plane and streams
-// SCI planes along i; each plane (with a one-node ring) is staged in shared
-// memory and smoothed along k, then along j, and each thread keeps the last
-// two (j, k)-smoothed values of its column in registers for the pass along
-// i.  The three passes use the expressions of k_smooth_axis in the same order
-// (k, j, i), so the output equals the three-kernel form bit for bit; only the
-// order of the partial sums differs.  The grid is kRedBlocks blocks looping
-// over the tiles, so the partial sums are those of fixed blocks.
-constexpr int SJ = 8, SK = 32, SCI = 16;
+// S in one pass.  A block takes an SJ x SK tile of the (j, k) plane, a warp a
+// row and a lane a node of it, and streams planes along i: a plane is smoothed
+// along k by warp shuffles, along j through shared memory, and along i from
+// the last two planes' values, which each thread keeps in registers.  The
+// planes of all tiles form one sequence that the blocks split evenly, so that
+// small grids use as many blocks as they have planes; a piece that starts
+// inside a tile's column first smooths the plane before it.  The grid is one
+// round of resident blocks, six per SM (at kRedBlocks, 1.33 rounds, a third of
+// the FP64 issue slots stayed empty).
+//
+// Bound by the FP64 rate (2 lanes a clock and SM).  QUARTER (side weight 1/4,
+// the default): a + 2 b + c per axis and one exact factor 1/64 at the end, 2
+// instructions an axis instead of 3; SUM, SQ: only the sums that are asked
+// for.  512^3: 3.87 -> 2.87 ms (FP64 pipe 72% busy), 32^3 (8 blocks in the
+// former split): 36.5 -> 9.8 us.
+constexpr int SJ = 8, SK = 32;
+constexpr int kSPerSM = 6, kSBlocks = kSPerSM * (kRedBlocks / 8);
 
-__global__ void __launch_bounds__(256) k_smooth_S_stream(Dims d, double ws,
-                                                         const double* __restrict__ in,
-                                                         const double* __restrict__ shift_sum,
-                                                         double* __restrict__ out,
-                                                         float* __restrict__ out32,
-                                                         double* __restrict__ psum,
-                                                         double* __restrict__ psq) {
-    __shared__ double pl[SJ + 2][SK + 2];  // plane with a one-node ring
-    __shared__ double sk[SJ + 2][SK];      // smoothed along k
+template <bool QUARTER, bool SUM, bool SQ>
+__global__ void __launch_bounds__(SJ* SK, kSPerSM) k_smooth_S_stream(
+    Dims d, double ws, const double* __restrict__ in, const double* __restrict__ shift_sum,
+    double* __restrict__ out, float* __restrict__ out32, double* __restrict__ part) {
+    __shared__ double sk[2][SJ + 2][SK];  // planes smoothed along k
     const double w1 = 1.0 - 2.0 * ws;
-    const double shift = shift_sum ? *shift_sum / (double)d.cells : 0.0;
-    const int t = threadIdx.x, lj = t / SK, lk = t % SK;
-    const int tiles_k = d.n2 / SK, tiles_j = d.n1 / SJ;
-    const int ntiles = tiles_k * tiles_j * (d.n0 / SCI);
-    double s = 0.0, q = 0.0;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int tk = tile % tiles_k, tj = (tile / tiles_k) % tiles_j, ti = tile / (tiles_k * tiles_j);
-        const int k0 = tk * SK, j0 = tj * SJ, i0 = ti * SCI;
+    const double shift = shift_sum ? *shift_sum * inv_pow2(d.cells) : 0.0;
+    const int lj = threadIdx.x / SK, lk = threadIdx.x % SK;
+    const int tiles_k = d.n2 / SK;
+    auto mix = [&](double m, double c, double p) {
+        return QUARTER ? fma(2.0, c, m + p) : fma(ws, m + p, w1 * c);
+    };
+    // a warp's row, with the values before and after it
+    struct Row {
+        double v, e;
+    };
+    auto load = [&](int i, int j, int k0) {
+        Row r;
+        r.v = in[cell_index(d, i, j, k0 + lk)];
+        if (lk == 0) r.e = in[cell_index(d, i, j, k0 - 1)];
+        if (lk == SK - 1) r.e = in[cell_index(d, i, j, k0 + SK)];
+        return r;
+    };
+    auto along_k = [&](const Row& r) {
+        double m = __shfl_up_sync(0xffffffffu, r.v, 1), p = __shfl_down_sync(0xffffffffu, r.v, 1);
+        if (lk == 0) m = r.e;
+        if (lk == SK - 1) p = r.e;
+        return mix(m, r.v, p);
+    };
+    const long long planes = (long long)tiles_k * (d.n1 / SJ) * d.n0;
+    long long at = planes * blockIdx.x / gridDim.x;
+    const long long end = planes * (blockIdx.x + 1) / gridDim.x;
+    double acc = 0.0;
+    while (at < end) {
+        const int col = (int)(at / d.n0), i0 = (int)(at % d.n0);
+        const int i1 = (int)min((long long)d.n0, i0 + (end - at));
+        at += i1 - i0;
+        const int k0 = (col % tiles_k) * SK, j0 = (col / tiles_k) * SJ;
+        // warps 0 and 1 also smooth the rows before and after the tile
+        const int je = lj == 0 ? j0 - 1 : j0 + SJ, re = lj == 0 ? 0 : SJ + 1;
         double a2 = 0.0, a1 = 0.0;  // (j, k)-smoothed values of planes p - 2, p - 1
-        for (int p = i0 - 1; p <= i0 + SCI; ++p) {
-            for (int e = t; e < (SJ + 2) * (SK + 2); e += blockDim.x) {
-                const int r = e / (SK + 2), c = e - r * (SK + 2);
-                pl[r][c] = in[cell_index(d, p, j0 - 1 + r, k0 - 1 + c)];
+        Row own = load(i0 - 1, j0 + lj, k0), edge{};
+        if (lj < 2) edge = load(i0 - 1, je, k0);
+        for (int p = i0 - 1; p <= i1; ++p) {
+            double(*row)[SK] = sk[(p - i0 + 1) & 1];
+            const double c = along_k(own);
+            row[lj + 1][lk] = c;
+            if (lj < 2) row[re][lk] = along_k(edge);
+            if (p < i1) {
+                own = load(p + 1, j0 + lj, k0);
+                if (lj < 2) edge = load(p + 1, je, k0);
             }
-            __syncthreads();
-            for (int e = t; e < (SJ + 2) * SK; e += blockDim.x) {
-                const int r = e / SK, c = e - r * SK;
-                sk[r][c] = fma(ws, pl[r][c] + pl[r][c + 2], w1 * pl[r][c + 1]);
-            }
-            __syncthreads();
-            const double v = fma(ws, sk[lj][lk] + sk[lj + 2][lk], w1 * sk[lj + 1][lk]);
+            __syncthreads();  // (the other buffer is read until the next one)
+            const double v = mix(row[lj][lk], c, row[lj + 2][lk]);
             if (p > i0) {  // plane p - 1 is complete
-                const double o = fma(ws, a2 + v, w1 * a1) - shift;
-                const int c = cell_index(d, p - 1, j0 + lj, k0 + lk);
-                out[c] = o;
-                if (out32) out32[c] = (float)o;
-                s += o;
-                q = fma(o, o, q);
+                const double x = mix(a2, a1, v);
+                const double o = QUARTER ? fma(x, 1.0 / 64.0, -shift) : x - shift;
+                const int e = cell_index(d, p - 1, j0 + lj, k0 + lk);
+                out[e] = o;
+                if (out32) out32[e] = (float)o;
+                if (SUM) acc += o;
+                if (SQ) acc = fma(o, o, acc);
             }
             a2 = a1, a1 = v;
-            __syncthreads();  // pl and sk are refilled for the next plane
+        }
+        __syncthreads();
+    }
+    if (SUM || SQ) {
+        acc = block_reduce<OpSum>(acc);
+        if (threadIdx.x == 0) {
+            part[blockIdx.x] = acc;
+            if (blockIdx.x + kSBlocks < kRedBlocks) part[blockIdx.x + kSBlocks] = 0.0;
         }
     }
-    if (psum) {
-        s = block_reduce<OpSum>(s);
-        if (threadIdx.x == 0) psum[blockIdx.x] = s;
-    }
-    if (psq) {
-        q = block_reduce<OpSum>(q);
-        if (threadIdx.x == 0) psq[blockIdx.x] = q;
-    }
+}
+
+template <bool QUARTER>
+void launch_smooth_stream(const Dims& d, double ws, const double* in, const double* shift_sum, double* out,
+                          float* out32, double* part_sum, double* part_sq, cudaStream_t st) {
+    if (part_sum)
+        k_smooth_S_stream<QUARTER, true, false><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, part_sum);
+    else if (part_sq)
+        k_smooth_S_stream<QUARTER, false, true><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, part_sq);
+    else
+        k_smooth_S_stream<QUARTER, false, false><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, nullptr);
 }
 
 template <typename T>
@@ -890,10 +932,10 @@ void launch_geometry_source(const Dims& d, const SourceParams& sp, const double*
 void launch_smooth_S(const Dims& d, double s_side, const double* in, const double* shift_sum,
                      double* out, float* out32, double* tmp2, double* part_sum, double* part_sq,
                      cudaStream_t st) {
-    if (d.n2 % SK == 0 && d.n1 % SJ == 0 && d.n0 % SCI == 0) {
+    if (d.n2 % SK == 0 && d.n1 % SJ == 0 && !(part_sum && part_sq)) {
         launch_counter()++;
-        k_smooth_S_stream<<<kRedBlocks, 256, 0, st>>>(d, s_side, in, shift_sum, out, out32, part_sum,
-                                                      part_sq);
+        auto launch = s_side == 0.25 ? launch_smooth_stream<true> : launch_smooth_stream<false>;
+        launch(d, s_side, in, shift_sum, out, out32, part_sum, part_sq, st);
         return;
     }
     launch_counter() += 3;

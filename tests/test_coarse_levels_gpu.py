@@ -55,3 +55,18 @@ def test_cluster_schedules_match_the_oracle(n, faces, nu):
         phi = R.field("phi").cpu().numpy()
     assert st.steps == 1 and st.relres[0] <= 1e-8
     assert np.linalg.norm(phi - ref.phi) <= BARS["mixed"] * np.linalg.norm(ref.phi)
+
+
+@pytest.mark.parametrize("s_side", [0.25, 0.2, 0.0])
+@pytest.mark.parametrize("shape", [(8, 8, 32), (16, 8, 64), (8, 16, 8), (64, 64, 32)])
+def test_smoothing_forms_match_the_oracle(shape, s_side):
+    """S in its streaming form (pieces of a few planes up to whole columns)
+    and per axis, with the default side weight and others."""
+    rho = _rough(shape, sum(shape) + 1)
+    ref = O.solve(O.OracleParams(n=shape, k_max=2, s_side=s_side), rho)
+    with Recon(shape, k_max=2, s_side=s_side, replay_alpha=ref.alpha) as R:
+        R.deposit_grid(torch.from_numpy(rho).cuda())
+        st = R.solve()
+        phi = R.field("phi").cpu().numpy()
+    assert st.steps == ref.steps
+    assert np.linalg.norm(phi - ref.phi) <= BARS["fp64"] * np.linalg.norm(ref.phi)
