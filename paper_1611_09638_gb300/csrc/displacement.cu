@@ -1,0 +1,262 @@
+// displacement.cu -- the node displacements of a step, alpha V = alpha e^-1 G
+// with e = I + Hess phi and G the central-difference gradient of dphi (the
+// mesh points' motion seen by the tracers, Sec. II of Zhu et al. 2016), in
+// fixed point with kDispBits fractional bits for the tracer advance.
+//
+// In FP64 a node takes some 70 instructions (the Hessian, six cofactors, a
+// division, three products), 10 ms at 512^3 with the Hessian read back from
+// memory.  Here only FP32 and integer instructions run: phi and dphi are
+// brought to 64-bit fixed point as a plane is loaded, Hessian and gradient are
+// exact integer sums, and e U = alpha G is solved by iterative refinement: X ~
+// e^-1 in FP32 gives a first U, and each further piece comes from the exact
+// residual alpha G - e U, formed modulo 2^64 (its leading bits cancel, so the
+// low 64 bits of the products suffice).  A piece carries 18 bits, so two
+// residuals leave an error below the 2^-53 cells of the result; badly
+// conditioned nodes take smaller pieces and more of them.  Nodes that do not
+// converge, and steps whose numbers do not fit (disp_scales), are computed in
+// FP64.  Against 113-bit arithmetic (64^3, |phi| <= 4, det e >= 0.48, alpha V <=
+// 0.42 cells) the error is 0.291 units of 2^-53 cells rms and 0.78 at most, that
+// of the FP64 form 0.321 and 1.97 (rounding to the unit alone: 0.289).
+//
+// A block streams planes along i over an 8 x 32 tile; a thread keeps its
+// column's sums of the last planes in registers, so that a plane's 340 nodes
+// are converted once and read back from shared memory 14 times a thread.
+// Bound by instruction issue: 512^3 10.06 -> 3.32 ms; it reads 16 and writes
+// 24 bytes a node (0.8 ms at the copy rate).
+#include "fixed_point.cuh"
+#include "geometry.cuh"
+#include "recon_internal.cuh"
+
+namespace recon {
+
+namespace {
+
+constexpr int kDispBits = 53;
+constexpr long long kDispMax = 1ll << (kDispBits + 7);  // 128 cells
+
+constexpr int DJ = 8, DK = 32, DPJ = DJ + 2, DPK = DK + 2;  // tile, and with its ring
+constexpr int DN = DPJ * DPK;
+constexpr int DPERSM = 3, DBLOCKS = DPERSM * (kRedBlocks / 8);
+
+// alpha V at one node in FP64, rounded to fixed point; values beyond kDispMax
+// cells, which no valid step produces, are held at that bound.
+__device__ __noinline__ void displacement64(const Dims& d, const double* __restrict__ phi,
+                                            const double* __restrict__ dphi, double alpha, int i, int j, int k,
+                                            long long (&out)[3]) {
+    Sym3 e = hessian(d, phi, i, j, k);
+    e.xx += 1.0, e.yy += 1.0, e.zz += 1.0;
+    const double gx = dphi[cell_index(d, i + 1, j, k)] - dphi[cell_index(d, i - 1, j, k)];
+    const double gy = dphi[cell_index(d, i, j + 1, k)] - dphi[cell_index(d, i, j - 1, k)];
+    const double gz = dphi[cell_index(d, i, j, k + 1)] - dphi[cell_index(d, i, j, k - 1)];
+    const double Axx = e.yy * e.zz - e.yz * e.yz, Ayy = e.xx * e.zz - e.xz * e.xz;
+    const double Azz = e.xx * e.yy - e.xy * e.xy, Axy = e.xz * e.yz - e.xy * e.zz;
+    const double Axz = e.xy * e.yz - e.yy * e.xz, Ayz = e.xy * e.xz - e.xx * e.yz;
+    // 1/2 of the central differences, alpha and 2^kDispBits in one factor
+    const double hinv = (0.5 * 9007199254740992.0) * alpha / (e.xx * Axx + e.xy * Axy + e.xz * Axz);
+    auto fix = [](double v) {
+        const long long q = __double2ll_rn(v);  // saturates beyond the int64 range
+        return q > kDispMax ? kDispMax : (q < -kDispMax ? -kDispMax : q);
+    };
+    out[0] = fix((Axx * gx + Axy * gy + Axz * gz) * hinv);
+    out[1] = fix((Axy * gx + Ayy * gy + Ayz * gz) * hinv);
+    out[2] = fix((Axz * gx + Ayz * gy + Azz * gz) * hinv);
+}
+
+// The scales of a step: phi 2^Q, dphi 2^Qd and alpha = 2^-kexp.  ok = false
+// where the fixed-point form does not apply: alpha is no power of two in
+// [2^-40, 1] (a replayed one), or the bound of a field is not finite or leaves
+// phi fewer than 46 fractional bits.
+struct DispScales {
+    int Q, Qd, kexp;
+    bool ok;
+};
+__device__ inline DispScales disp_scales(const double* scal) {
+    DispScales s;
+    const long long a = __double_as_longlong(scal[SC_ALPHA]);
+    s.kexp = 1023 - (int)(a >> 52);
+    s.Q = fixed_bits(scal[SC_PHI_BOUND], 54);
+    s.Qd = fixed_bits(scal[SC_MAX_DPHI], 120);
+    s.ok = (a & 0xfffffffffffffll) == 0 && a > 0 && s.kexp >= 0 && s.kexp <= 40 && s.Q >= 46 && s.Qd > -1000;
+    return s;
+}
+
+// e U = alpha G from the integer sums: h = second differences (xx, yy, zz) at
+// scale 2^Q and four times the mixed ones (xy, xz, yz), g = twice the gradient
+// of dphi at scale 2^Qd.  Returns whether U (scale 2^kDispBits) is within its
+// last place or so.
+__device__ __forceinline__ bool solve_fixed(const DispScales& sc, const long long (&h)[6],
+                                            const long long (&g)[3], long long (&out)[3]) {
+    // FP32: e, its inverse X and the right-hand side
+    int top = 0;  // every sum below 64 at its scale, or the node is not for integers
+#pragma unroll
+    for (int q = 0; q < 6; ++q) top = max(top, abs((int)(h[q] >> 32)));
+    if (top >= 1 << (sc.Q - 26)) return false;
+    const int low = sc.Q - 24;  // 22 .. 30: sums as 32-bit integers at scale 2^24
+    const float ue = pow2f(-24), ug = pow2f(max(31 - sc.Qd - sc.kexp, -126));
+    const float xx = 1.f + (float)(int)(h[0] >> low) * ue, yy = 1.f + (float)(int)(h[1] >> low) * ue,
+                zz = 1.f + (float)(int)(h[2] >> low) * ue;
+    const float xy = (float)(int)(h[3] >> low) * (0.25f * ue), xz = (float)(int)(h[4] >> low) * (0.25f * ue),
+                yz = (float)(int)(h[5] >> low) * (0.25f * ue);
+    float Xxx = yy * zz - yz * yz, Xyy = xx * zz - xz * xz, Xzz = xx * yy - xy * xy;
+    float Xxy = xz * yz - xy * zz, Xxz = xy * yz - yy * xz, Xyz = xy * xz - xx * yz;
+    const float rdet = __fdividef(1.f, xx * Xxx + xy * Xxy + xz * Xxz);
+    Xxx *= rdet, Xyy *= rdet, Xzz *= rdet, Xxy *= rdet, Xxz *= rdet, Xyz *= rdet;
+    const float emax = fmaxf(fmaxf(fabsf(xx), fabsf(yy)), fmaxf(fabsf(zz), fmaxf(fabsf(xy), fmaxf(fabsf(xz), fabsf(yz)))));
+    const float g0 = upper_float(g[0], ug), g1 = upper_float(g[1], ug), g2 = upper_float(g[2], ug);
+    // integers: e at scale 2^54 (Q <= 54)
+    using U64 = unsigned long long;
+    const int up = 54 - sc.Q;
+    const U64 Exx = ((U64)h[0] << up) + (1ull << 54), Eyy = ((U64)h[1] << up) + (1ull << 54),
+              Ezz = ((U64)h[2] << up) + (1ull << 54);
+    auto mixed = [&](long long v) { return (U64)((((long long)((U64)v << up)) + 2) >> 2); };
+    const U64 Exy = mixed(h[3]), Exz = mixed(h[4]), Eyz = mixed(h[5]);
+    float u0, u1, u2, um;  // a piece and its largest magnitude
+    auto piece = [&](float r0, float r1, float r2) {
+        u0 = Xxx * r0 + Xxy * r1 + Xxz * r2;
+        u1 = Xxy * r0 + Xyy * r1 + Xyz * r2;
+        u2 = Xxz * r0 + Xyz * r1 + Xzz * r2;
+        um = fmaxf(fabsf(u0), fmaxf(fabsf(u1), fabsf(u2)));
+    };
+    piece(g0, g1, g2);
+    // The residual of a piece must fit 62 bits: the error of X is about
+    // 2^-22 |e|^2 / det; where that is more, smaller pieces.
+    const float gm = fmaxf(fabsf(g0), fmaxf(fabsf(g1), fabsf(g2)));
+    const float crit = emax * emax * emax * fabsf(rdet) * __fdividef(gm, fmaxf(um, 1e-30f));
+    if (!(um < 32.f && crit < 3e5f)) return false;
+    const int bits = 17 - max(((__float_as_int(crit) >> 23) & 255) - 127 - 9, 0);
+    const float step = pow2f(-bits);
+    // U = D 2^-s in pieces of at most bits + 1 bits, the last at 2^-57
+    auto scale_of = [&] { return min(bits - (((__float_as_int(um) >> 23) & 255) - 127), 57); };
+    int s = scale_of();
+    long long a0 = __float2int_rn(u0 * pow2f(s)), a1 = __float2int_rn(u1 * pow2f(s)), a2 = __float2int_rn(u2 * pow2f(s));
+    U64 D0 = a0, D1 = a1, D2 = a2;
+    float last = um, err = um;
+    if (err >= 7e-18f) {  // 2^-57 cells
+        const int n = 53 + s - sc.Qd - sc.kexp;
+        U64 R0 = shift_fixed(g[0], n), R1 = shift_fixed(g[1], n), R2 = shift_fixed(g[2], n);
+#pragma unroll 1
+        for (int it = 0; it < 7; ++it) {
+            // residual alpha G - e U at scale 2^(54 + s)
+            R0 -= Exx * (U64)a0 + Exy * (U64)a1 + Exz * (U64)a2;
+            R1 -= Exy * (U64)a0 + Eyy * (U64)a1 + Eyz * (U64)a2;
+            R2 -= Exz * (U64)a0 + Eyz * (U64)a1 + Ezz * (U64)a2;
+            const float ur = pow2f(-22 - s);
+            const U64 half = 1ull << 31;
+            piece(upper_float(R0 + half, ur), upper_float(R1 + half, ur), upper_float(R2 + half, ur));
+            const int ns = max(scale_of(), s), m = min(ns - s, 63);
+            s = ns;
+            const float sc2 = pow2f(s);
+            a0 = __float2int_rn(u0 * sc2), a1 = __float2int_rn(u1 * sc2), a2 = __float2int_rn(u2 * sc2);
+            D0 = (D0 << m) + a0, D1 = (D1 << m) + a1, D2 = (D2 << m) + a2;
+            // what remains: the piece's rounding, or X's error as the last two
+            // pieces show it
+            err = um * fmaxf(step, __fdividef(um, last));
+            if (err < 7e-18f) break;
+            if (!(um < 0.25f * last)) return false;
+            last = um;
+            R0 <<= m, R1 <<= m, R2 <<= m;
+        }
+    }
+    const int n = s - kDispBits;  // at most 4; 2^-53 cells
+    auto place = [&](U64 v) { return n > 0 ? ((long long)(v + (1ull << (n - 1)))) >> n : (long long)(v << -n); };
+    out[0] = place(D0), out[1] = place(D1), out[2] = place(D2);
+    return err < 7e-18f;
+}
+
+__global__ void __launch_bounds__(DJ* DK, DPERSM) k_displacement_stream(
+    Dims d, const double* __restrict__ scal, const double* __restrict__ phi, const double* __restrict__ dphi,
+    long long* __restrict__ dx, long long* __restrict__ dy, long long* __restrict__ dz) {
+    __shared__ long long sp[2][DN], sd[2][DN];
+    const DispScales sc = disp_scales(scal);
+    const double alpha = scal[SC_ALPHA];
+    const int t = threadIdx.x, lj = t / DK, lk = t % DK;
+    const int own = (lj + 1) * DPK + lk + 1;
+    const int tiles_k = d.n2 / DK;
+    const long long planes = (long long)tiles_k * (d.n1 / DJ) * d.n0;
+    long long at = planes * blockIdx.x / gridDim.x;
+    const long long end = planes * (blockIdx.x + 1) / gridDim.x;
+    if (!sc.ok) {  // every node in FP64
+        for (; at < end; ++at) {
+            const int col = (int)(at / d.n0), i = (int)(at % d.n0);
+            const int j = (col / tiles_k) * DJ + lj, k = (col % tiles_k) * DK + lk;
+            long long o[3];
+            displacement64(d, phi, dphi, alpha, i, j, k, o);
+            const int c = cell_index(d, i, j, k);
+            dx[c] = o[0], dy[c] = o[1], dz[c] = o[2];
+        }
+        return;
+    }
+    // this thread's nodes of a plane with its ring
+    const int e1 = t + DJ * DK;
+    const bool two = e1 < DN;
+    while (at < end) {
+        const int col = (int)(at / d.n0), i0 = (int)(at % d.n0);
+        const int i1 = (int)min((long long)d.n0, i0 + (end - at));
+        at += i1 - i0;
+        const int k0 = (col % tiles_k) * DK, j0 = (col / tiles_k) * DJ;
+        const int c0 = cell_index(d, 0, j0 - 1 + t / DPK, k0 - 1 + t % DPK);
+        const int c1 = two ? cell_index(d, 0, j0 - 1 + e1 / DPK, k0 - 1 + e1 % DPK) : 0;
+        const int plane = d.n1 * d.n2;
+        double p0, p1 = 0.0, q0, q1 = 0.0;
+        auto load = [&](int i) {
+            const int b = (i & (d.n0 - 1)) * plane;
+            p0 = phi[b + c0], q0 = dphi[b + c0];
+            if (two) p1 = phi[b + c1], q1 = dphi[b + c1];
+        };
+        // sums of the column on planes p - 2, p - 1 (own value, differences in
+        // j and k, own dphi), and plane p - 1's second differences and gradient
+        long long ca = 0, cb = 0, ja = 0, jb = 0, ka = 0, kb = 0, da = 0, db = 0;
+        long long syb = 0, szb = 0, yzb = 0, gyb = 0, gzb = 0;
+        load(i0 - 1);
+        for (int p = i0 - 1; p <= i1; ++p) {
+            const int buf = (p - i0 + 1) & 1;
+            sp[buf][t] = to_fixed(p0, sc.Q), sd[buf][t] = to_fixed(q0, sc.Qd);
+            if (two) sp[buf][e1] = to_fixed(p1, sc.Q), sd[buf][e1] = to_fixed(q1, sc.Qd);
+            if (p < i1) load(p + 1);
+            __syncthreads();  // (the other buffer is read until the next one)
+            const long long *f = sp[buf] + own, *w = sd[buf] + own;
+            const long long c = f[0], jp = f[DPK], jm = f[-DPK], kp = f[1], km = f[-1], dc = w[0];
+            const long long jd = jp - jm, kd = kp - km;
+            if (p > i0) {  // node (p - 1)
+                const long long h[6] = {c + ca - 2 * cb, syb, szb, jd - ja, kd - ka, yzb};
+                const long long g[3] = {dc - da, gyb, gzb};
+                long long o[3];
+                if (!solve_fixed(sc, h, g, o)) displacement64(d, phi, dphi, alpha, p - 1, j0 + lj, k0 + lk, o);
+                const int cell = cell_index(d, p - 1, j0 + lj, k0 + lk);
+                dx[cell] = o[0], dy[cell] = o[1], dz[cell] = o[2];
+            }
+            syb = jp + jm - 2 * c, szb = kp + km - 2 * c;
+            yzb = (f[DPK + 1] - f[DPK - 1]) - (f[-DPK + 1] - f[-DPK - 1]);
+            gyb = w[DPK] - w[-DPK], gzb = w[1] - w[-1];
+            ca = cb, cb = c, ja = jb, jb = jd, ka = kb, kb = kd, da = db, db = dc;
+        }
+        __syncthreads();
+    }
+}
+
+// Any grid, a thread a node, in FP64.
+__global__ void k_displacement_node(Dims d, const double* __restrict__ scal, const double* __restrict__ phi,
+                                    const double* __restrict__ dphi, long long* __restrict__ dx,
+                                    long long* __restrict__ dy, long long* __restrict__ dz) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= d.cells) return;
+    int i, j, k;
+    cell_coords(d, c, i, j, k);
+    long long o[3];
+    displacement64(d, phi, dphi, scal[SC_ALPHA], i, j, k, o);
+    dx[c] = o[0], dy[c] = o[1], dz[c] = o[2];
+}
+
+}  // namespace
+
+void launch_node_displacement(const Dims& d, const double* scal, const double* phi, const double* dphi,
+                              long long* dx, long long* dy, long long* dz, cudaStream_t st) {
+    launch_counter()++;
+    if (d.n2 % DK == 0 && d.n1 % DJ == 0) {
+        k_displacement_stream<<<DBLOCKS, DJ * DK, 0, st>>>(d, scal, phi, dphi, dx, dy, dz);
+        return;
+    }
+    k_displacement_node<<<(d.cells + 255) / 256, 256, 0, st>>>(d, scal, phi, dphi, dx, dy, dz);
+}
+
+}  // namespace recon

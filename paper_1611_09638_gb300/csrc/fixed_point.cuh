@@ -1,0 +1,46 @@
+// fixed_point.cuh -- 64-bit fixed-point forms of the FP64 fields.  GB300
+// issues two FP64 operations a clock and SM against 64 or more integer ones,
+// so stencils of phi and dphi that need more than FP32 run on integers: a
+// value is scaled by a power of two 2^Q, chosen once per field from a bound on
+// its magnitude, and rounded; sums and differences of such values are exact.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace recon {
+
+// x 2^Q rounded to nearest (|x| 2^Q < 2^62), from the bits of x.
+__device__ __forceinline__ long long to_fixed(double x, int Q) {
+    const long long b = __double_as_longlong(x);
+    const int e = (int)(b >> 52) & 0x7ff;
+    // |x| = m 2^(e - 1075); m 2^10 shifted right by t = 10 - (e - 1075 + Q)
+    const unsigned long long m = e ? (((unsigned long long)b << 10) & 0x3ffffffffffffc00ull) | (1ull << 62) : 0ull;
+    const int r = 1085 - Q - e, t = min(max(r, 0), 63);
+    const unsigned long long v = r > 63 ? 0ull : (m + ((1ull << t) >> 1)) >> t;
+    const long long s = b >> 63;
+    return ((long long)v ^ s) - s;
+}
+
+// The largest Q <= most with bound 2^Q <= 2^60, for a bound >= 0; -1000 where
+// there is none to use (not finite, or above 2^90).
+__device__ __forceinline__ int fixed_bits(double bound, int most) {
+    const long long b = __double_as_longlong(bound);
+    const int e = (int)(b >> 52) & 0x7ff;  // bound < 2^(e - 1022)
+    if (b < 0 || e > 1022 + 90) return -1000;
+    return min(most, 60 - (e - 1022));
+}
+
+// v 2^n modulo 2^64 for n >= 0, v 2^n rounded for n < 0.
+__device__ __forceinline__ long long shift_fixed(long long v, int n) {
+    if (n >= 0) return n > 63 ? 0ll : (long long)((unsigned long long)v << n);
+    const int r = min(-n, 63);
+    return (v >> r) + ((v >> (r - 1)) & 1);
+}
+
+// The upper half of v, times unit: an absolute error below one unit besides
+// the rounding.
+__device__ __forceinline__ float upper_float(long long v, float unit) { return (float)(int)(v >> 32) * unit; }
+
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }  // -126 <= e <= 127
+
+}  // namespace recon

@@ -82,6 +82,8 @@ enum Scalar {
     SC_ALPHA,         // step length of the current step
     SC_ADJ_A,         // adjoint sweep: sums used for mean projections
     SC_ADJ_B,
+    SC_MAX_DPHI,      // a bound on max |dphi| of the step
+    SC_PHI_BOUND,     // a bound on max |phi|, grown by every advance
     SC_COUNT
 };
 
@@ -152,7 +154,17 @@ bool launch_coarse_cluster(const CoarseSet& cs, const float* f, float* u, const 
                            int cycles, cudaStream_t st);
 
 // ---- reductions -----------------------------------------------------------
-// op: 0 = sum, 1 = min, 2 = max.  Finishes kRedBlocks partials into slot.
+// op: 0 = sum, 1 = min, 2 = max.  Finishes kRedBlocks partials into slot;
+// finish_reduces does several in one launch.
+struct Finish {
+    const double* partials;
+    int op, slot;
+};
+struct FinishList {
+    int n;
+    Finish f[4];
+};
+void finish_reduces(const FinishList& l, double* scalars, cudaStream_t st);
 void finish_reduce(const double* partials, int op, double* scalars, int slot, cudaStream_t st);
 
 // ---- multigrid (T = float or double) --------------------------------------
@@ -295,10 +307,11 @@ void launch_geometry_source(const Dims& d, const SourceParams& sp, const double*
                             const double* m, double* t, double* e6, double* part_sum,
                             double* part_min, cudaStream_t st);
 // S in three axis passes through tmp2 (2 x cells scratch); out32 (optional)
-// receives an FP32 copy of the result.
+// receives an FP32 copy of the result; part_sum (with out32 and part_max) its
+// sum and largest magnitude, part_sq its sum of squares, or neither.
 void launch_smooth_S(const Dims& d, double s_side, const double* in, const double* shift_scalar,
-                     double* out, float* out32, double* tmp2, double* part_sum, double* part_sq,
-                     cudaStream_t st);
+                     double* out, float* out32, double* tmp2, double* part_sum, double* part_max,
+                     double* part_sq, cudaStream_t st);
 // phi32, dphi32: FP32 copies of phi and dphi used to screen nodes that clear
 // the limiter's floor by a wide margin.
 void launch_limiter(const Dims& d, const LimiterParams& lp, const double* e6, const double* dphi,
@@ -306,9 +319,9 @@ void launch_limiter(const Dims& d, const LimiterParams& lp, const double* e6, co
                     cudaStream_t st);
 void launch_node_velocity(const Dims& d, const double* e6, const double* dphi, double* vx,
                           double* vy, double* vz, cudaStream_t st);
-// The step's node displacements alpha V in fixed point (2^-51 cells), for
-// launch_advance.
-void launch_node_displacement(const Dims& d, const double* e6, const double* dphi, const double* alpha,
+// The step's node displacements alpha V in fixed point (2^-53 cells), for
+// launch_advance; scal: SC_ALPHA, SC_PHI_BOUND and SC_MAX_DPHI are read.
+void launch_node_displacement(const Dims& d, const double* scal, const double* phi, const double* dphi,
                               long long* dx, long long* dy, long long* dz, cudaStream_t st);
 // Tracers move by -alpha V(xi) (the fixed-point displacements CIC-interpolated
 // in integer arithmetic); phi += alpha (dphi - mean), mean = *sum_dphi / cells.
@@ -367,7 +380,8 @@ struct CtlHandles {
     cudaGraphConditionalHandle step, cont, mg, adv, fin, chk;
 };
 
-void launch_ctl_init(Ctl* c, cudaStream_t st);
+// scal: SC_PHI_BOUND starts at 0 (null: the scalars stay as they are)
+void launch_ctl_init(Ctl* c, double* scal, cudaStream_t st);
 void launch_ctl_step_begin(Ctl* c, const double* scal, const CtlArrays& a, double ncells,
                            double tol_out, const CtlHandles& h, cudaStream_t st);
 void launch_ctl_mg_begin(Ctl* c, const CtlArrays& a, int mixed, double tol_in,
@@ -388,8 +402,8 @@ void launch_warm_extrapolate(const Ctl* c, const double* alpha, double* u, doubl
 void launch_ctl_mg_check(Ctl* c, const double* scal, const CtlArrays& a, int per_launch,
                          double tol_in, int max_vcycles, const CtlHandles& h, cudaStream_t st);
 void launch_ctl_select_alpha(Ctl* c, double* scal, const CtlArrays& a, const double* replay,
-                             int kmax_exp, double d_max, double alpha_min, const CtlHandles& h,
-                             cudaStream_t st);
+                             int kmax_exp, double ncells, double d_max, double alpha_min,
+                             const CtlHandles& h, cudaStream_t st);
 void launch_ctl_step_end(Ctl* c, int k_max, const CtlHandles& h, cudaStream_t st);
 void launch_ctl_final(Ctl* c, int want, const CtlHandles& h, cudaStream_t st);
 void launch_ctl_final_mass(Ctl* c, const double* scal, cudaStream_t st);

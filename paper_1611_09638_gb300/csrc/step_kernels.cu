@@ -314,11 +314,12 @@ __global__ void k_geometry_source(Dims d, SourceParams sp, const double* __restr
 __global__ void k_smooth_axis(Dims d, int axis, double ws, const double* __restrict__ in,
                               const double* __restrict__ shift_sum, double* __restrict__ out,
                               float* __restrict__ out32, double* __restrict__ psum,
-                              double* __restrict__ psq) {
+                              double* __restrict__ pmax, double* __restrict__ psq) {
     const double w1 = 1.0 - 2.0 * ws;
     const double shift = shift_sum ? *shift_sum / (double)d.cells : 0.0;
     const int di = axis == 0, dj = axis == 1, dk = axis == 2;
     double s = 0.0, q = 0.0;
+    float mx = 0.f;
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells; c += gridDim.x * blockDim.x) {
         int i, j, k;
         cell_coords(d, c, i, j, k);
@@ -327,8 +328,13 @@ __global__ void k_smooth_axis(Dims d, int axis, double ws, const double* __restr
                              w1 * in[c]) - shift;
         out[c] = v;
         if (out32) out32[c] = (float)v;
+        mx = fmaxf(mx, fabsf((float)v));
         s += v;
         q = fma(v, v, q);
+    }
+    if (pmax) {
+        const double v = block_reduce<OpMax>((double)mx);
+        if (threadIdx.x == 0) pmax[blockIdx.x] = v;
     }
     if (psum) {
         s = block_reduce<OpSum>(s);
@@ -352,8 +358,8 @@ __global__ void k_smooth_axis(Dims d, int axis, double ws, const double* __restr
 //
 // Bound by the FP64 rate (2 lanes a clock and SM).  QUARTER (side weight 1/4,
 // the default): a + 2 b + c per axis and one exact factor 1/64 at the end, 2
-// instructions an axis instead of 3; SUM, SQ: only the sums that are asked
-// for.  512^3: 3.87 -> 2.87 ms (FP64 pipe 72% busy), 32^3 (8 blocks in the
+// instructions an axis instead of 3.  SUM: the FP32 copy, the sum and the
+// largest magnitude (of the FP32 copy); SQ: the sum of squares.  512^3: 3.87 -> 2.87 ms (FP64 pipe 72% busy), 32^3 (8 blocks in the
 // former split): 36.5 -> 9.8 us.
 constexpr int SJ = 8, SK = 32;
 constexpr int kSPerSM = 6, kSBlocks = kSPerSM * (kRedBlocks / 8);
@@ -361,7 +367,7 @@ constexpr int kSPerSM = 6, kSBlocks = kSPerSM * (kRedBlocks / 8);
 template <bool QUARTER, bool SUM, bool SQ>
 __global__ void __launch_bounds__(SJ* SK, kSPerSM) k_smooth_S_stream(
     Dims d, double ws, const double* __restrict__ in, const double* __restrict__ shift_sum,
-    double* __restrict__ out, float* __restrict__ out32, double* __restrict__ part) {
+    double* __restrict__ out, float* __restrict__ out32, double* __restrict__ part, double* __restrict__ pmax) {
     __shared__ double sk[2][SJ + 2][SK];  // planes smoothed along k
     const double w1 = 1.0 - 2.0 * ws;
     const double shift = shift_sum ? *shift_sum * inv_pow2(d.cells) : 0.0;
@@ -391,6 +397,7 @@ __global__ void __launch_bounds__(SJ* SK, kSPerSM) k_smooth_S_stream(
     long long at = planes * blockIdx.x / gridDim.x;
     const long long end = planes * (blockIdx.x + 1) / gridDim.x;
     double acc = 0.0;
+    float mx = 0.f;
     while (at < end) {
         const int col = (int)(at / d.n0), i0 = (int)(at % d.n0);
         const int i1 = (int)min((long long)d.n0, i0 + (end - at));
@@ -417,8 +424,11 @@ __global__ void __launch_bounds__(SJ* SK, kSPerSM) k_smooth_S_stream(
                 const double o = QUARTER ? fma(x, 1.0 / 64.0, -shift) : x - shift;
                 const int e = cell_index(d, p - 1, j0 + lj, k0 + lk);
                 out[e] = o;
-                if (out32) out32[e] = (float)o;
-                if (SUM) acc += o;
+                if (SUM) {
+                    out32[e] = (float)o;
+                    mx = fmaxf(mx, fabsf((float)o));
+                    acc += o;
+                }
                 if (SQ) acc = fma(o, o, acc);
             }
             a2 = a1, a1 = v;
@@ -432,17 +442,24 @@ __global__ void __launch_bounds__(SJ* SK, kSPerSM) k_smooth_S_stream(
             if (blockIdx.x + kSBlocks < kRedBlocks) part[blockIdx.x + kSBlocks] = 0.0;
         }
     }
+    if (SUM) {
+        const double v = block_reduce<OpMax>((double)mx);
+        if (threadIdx.x == 0) {
+            pmax[blockIdx.x] = v;
+            if (blockIdx.x + kSBlocks < kRedBlocks) pmax[blockIdx.x + kSBlocks] = 0.0;
+        }
+    }
 }
 
 template <bool QUARTER>
 void launch_smooth_stream(const Dims& d, double ws, const double* in, const double* shift_sum, double* out,
-                          float* out32, double* part_sum, double* part_sq, cudaStream_t st) {
+                          float* out32, double* part_sum, double* part_max, double* part_sq, cudaStream_t st) {
     if (part_sum)
-        k_smooth_S_stream<QUARTER, true, false><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, part_sum);
+        k_smooth_S_stream<QUARTER, true, false><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, part_sum, part_max);
     else if (part_sq)
-        k_smooth_S_stream<QUARTER, false, true><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, part_sq);
+        k_smooth_S_stream<QUARTER, false, true><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, part_sq, part_max);
     else
-        k_smooth_S_stream<QUARTER, false, false><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, nullptr);
+        k_smooth_S_stream<QUARTER, false, false><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, nullptr, part_max);
 }
 
 template <typename T>
@@ -606,42 +623,6 @@ __global__ void k_node_velocity(Dims d, const double* __restrict__ e6,
     vx[c] = (Axx * gx + Axy * gy + Axz * gz) * hinv;
     vy[c] = (Axy * gx + Ayy * gy + Ayz * gz) * hinv;
     vz[c] = (Axz * gx + Ayz * gy + Azz * gz) * hinv;
-}
-
-// The step's node displacement alpha V = alpha e^-1 G (V as in
-// k_node_velocity) in fixed point with kDispBits fractional bits, for the
-// tracer advance's integer interpolation.  The step limiter bounds it by
-// d_max / lambda_floor (50 cells at the defaults); values beyond kDispMax
-// cells, which no valid step produces, are held at that bound.
-constexpr int kDispBits = 53;
-constexpr long long kDispMax = 1ll << (kDispBits + 7);  // 128 cells
-__global__ void k_node_displacement(Dims d, const double* __restrict__ e6,
-                                    const double* __restrict__ dphi, const double* __restrict__ alpha_p,
-                                    long long* __restrict__ dx, long long* __restrict__ dy,
-                                    long long* __restrict__ dz) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= d.cells) return;
-    int i, j, k;
-    cell_coords(d, c, i, j, k);
-    const size_t n = (size_t)d.cells;
-    Sym3 e;
-    e.xx = e6[c], e.yy = e6[n + c], e.zz = e6[2 * n + c];
-    e.xy = e6[3 * n + c], e.xz = e6[4 * n + c], e.yz = e6[5 * n + c];
-    const double gx = dphi[cell_index(d, i + 1, j, k)] - dphi[cell_index(d, i - 1, j, k)];
-    const double gy = dphi[cell_index(d, i, j + 1, k)] - dphi[cell_index(d, i, j - 1, k)];
-    const double gz = dphi[cell_index(d, i, j, k + 1)] - dphi[cell_index(d, i, j, k - 1)];
-    const double Axx = e.yy * e.zz - e.yz * e.yz, Ayy = e.xx * e.zz - e.xz * e.xz;
-    const double Azz = e.xx * e.yy - e.xy * e.xy, Axy = e.xz * e.yz - e.xy * e.zz;
-    const double Axz = e.xy * e.yz - e.yy * e.xz, Ayz = e.xy * e.xz - e.xx * e.yz;
-    // 1/2 of the central differences, alpha and 2^kDispBits in one factor
-    const double hinv = (0.5 * 9007199254740992.0) * *alpha_p / (e.xx * Axx + e.xy * Axy + e.xz * Axz);
-    auto fix = [](double v) {
-        const long long q = __double2ll_rn(v);  // saturates beyond the int64 range
-        return q > kDispMax ? kDispMax : (q < -kDispMax ? -kDispMax : q);
-    };
-    dx[c] = fix((Axx * gx + Axy * gy + Axz * gz) * hinv);
-    dy[c] = fix((Axy * gx + Ayy * gy + Ayz * gz) * hinv);
-    dz[c] = fix((Axz * gx + Ayz * gy + Azz * gz) * hinv);
 }
 
 // App. A's linear density update (the variant that carries m instead of
@@ -854,19 +835,30 @@ __global__ void k_scale(int cells, const double* __restrict__ in, double s, doub
 }
 
 template <class Op>
-__global__ void k_finish(const double* __restrict__ partials, double* __restrict__ scalars, int slot) {
+__device__ void finish(const double* __restrict__ partials, double* __restrict__ scalars, int slot) {
     double v = Op::id();
     for (int b = threadIdx.x; b < kRedBlocks; b += blockDim.x) v = Op::op(v, partials[b]);
     v = block_reduce<Op>(v);
     if (threadIdx.x == 0) scalars[slot] = v;
 }
 
+// Finishes several reductions, a block each (4.3 us a launch, whatever it holds).
+__global__ void k_finish(FinishList l, double* __restrict__ scalars) {
+    const Finish f = l.f[blockIdx.x];
+    if (f.op == 0) finish<OpSum>(f.partials, scalars, f.slot);
+    else if (f.op == 1) finish<OpMin>(f.partials, scalars, f.slot);
+    else finish<OpMax>(f.partials, scalars, f.slot);
+}
+
 }  // namespace
 
+void finish_reduces(const FinishList& l, double* scalars, cudaStream_t st) {
+    launch_counter()++;
+    k_finish<<<l.n, 1024, 0, st>>>(l, scalars);
+}
+
 void finish_reduce(const double* partials, int op, double* scalars, int slot, cudaStream_t st) {
-    if (op == 0) { launch_counter()++; k_finish<OpSum><<<1, 1024, 0, st>>>(partials, scalars, slot); }
-    else if (op == 1) { launch_counter()++; k_finish<OpMin><<<1, 1024, 0, st>>>(partials, scalars, slot); }
-    else { launch_counter()++; k_finish<OpMax><<<1, 1024, 0, st>>>(partials, scalars, slot); }
+    finish_reduces(FinishList{1, {{partials, op, slot}}}, scalars, st);
 }
 
 void launch_validate_grid(int cells, const double* rho, double* ps, double* pb, cudaStream_t st) {
@@ -930,21 +922,21 @@ void launch_geometry_source(const Dims& d, const SourceParams& sp, const double*
 }
 
 void launch_smooth_S(const Dims& d, double s_side, const double* in, const double* shift_sum,
-                     double* out, float* out32, double* tmp2, double* part_sum, double* part_sq,
-                     cudaStream_t st) {
+                     double* out, float* out32, double* tmp2, double* part_sum, double* part_max,
+                     double* part_sq, cudaStream_t st) {
     if (d.n2 % SK == 0 && d.n1 % SJ == 0 && !(part_sum && part_sq)) {
         launch_counter()++;
         auto launch = s_side == 0.25 ? launch_smooth_stream<true> : launch_smooth_stream<false>;
-        launch(d, s_side, in, shift_sum, out, out32, part_sum, part_sq, st);
+        launch(d, s_side, in, shift_sum, out, out32, part_sum, part_max, part_sq, st);
         return;
     }
     launch_counter() += 3;
     k_smooth_axis<<<kRedBlocks, kRedThreads, 0, st>>>(d, 2, s_side, in, nullptr, tmp2, nullptr,
-                                                      nullptr, nullptr);
+                                                      nullptr, nullptr, nullptr);
     k_smooth_axis<<<kRedBlocks, kRedThreads, 0, st>>>(d, 1, s_side, tmp2, nullptr,
-                                                      tmp2 + d.cells, nullptr, nullptr, nullptr);
+                                                      tmp2 + d.cells, nullptr, nullptr, nullptr, nullptr);
     k_smooth_axis<<<kRedBlocks, kRedThreads, 0, st>>>(d, 0, s_side, tmp2 + d.cells, shift_sum,
-                                                      out, out32, part_sum, part_sq);
+                                                      out, out32, part_sum, part_max, part_sq);
 }
 
 void launch_limiter(const Dims& d, const LimiterParams& lp, const double* e6, const double* dphi,
@@ -958,12 +950,6 @@ void launch_node_velocity(const Dims& d, const double* e6, const double* dphi, d
                           double* vy, double* vz, cudaStream_t st) {
     launch_counter()++;
     k_node_velocity<<<nblocks(d.cells), kThreads, 0, st>>>(d, e6, dphi, vx, vy, vz);
-}
-
-void launch_node_displacement(const Dims& d, const double* e6, const double* dphi, const double* alpha,
-                              long long* dx, long long* dy, long long* dz, cudaStream_t st) {
-    launch_counter()++;
-    k_node_displacement<<<nblocks(d.cells), kThreads, 0, st>>>(d, e6, dphi, alpha, dx, dy, dz);
 }
 
 void launch_advance(const Dims& d, const long long* dx, const long long* dy, const long long* dz,
