@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "librecon.so")
 LIB_CHECKED = os.path.join(HERE, "librecon_checked.so")
-SOURCES = ["recon_api.cu", "mg_kernels.cu", "step_kernels.cu", "displacement.cu", "smoother.cu", "transfer.cu", "control.cu", "adjoint.cu", "noalloc.cu", "coarse_cluster.cu"]
+SOURCES = ["recon_api.cu", "mg_kernels.cu", "step_kernels.cu", "displacement.cu", "screened.cu", "smoother.cu", "transfer.cu", "control.cu", "adjoint.cu", "noalloc.cu", "coarse_cluster.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
          "--expt-relaxed-constexpr"]

@@ -70,7 +70,7 @@ struct Handle {
     // staging of host particle inputs (grown to the largest, kept until destroy)
     void* stage = nullptr;
     size_t stage_bytes = 0;
-    double* e6 = nullptr;  // triad I + Hess phi of the current step, 6 x cells
+    double* e6 = nullptr;  // triad I + Hess phi, 6 x cells (density_update = 1 or checkpoint)
     double* F64 = nullptr;    // face coefficients (a_c + a_{c+e}) / 2 of the finest level, 3 x cells
     double* D64 = nullptr;    // node diagonal: sum of the node's six face coefficients
     float *phi32 = nullptr, *dphi32 = nullptr;  // FP32 copies for the limiter's screen
@@ -461,19 +461,20 @@ void build_hierarchy(Handle* H, std::vector<T*>& c) {
 
 // Mass per current curvilinear cell (tracer CIC deposit, or the carried m
 // of App. A's variant), the operator coefficient a = max(m, a_min) and sum m.
-int deposit_step(Handle* H) {
+// The sum of m is left in part[0]; finish: and finished into SC_SUM_M.
+int deposit_step(Handle* H, bool finish = true) {
     if (H->p.density_update == 1) {
         // the carried mass per cell: only the coefficient and the mass sum
         launch_coef_from_m(H->cells, H->m, H->p.a_min, H->a64, H->mixed ? H->c32[0] : nullptr,
                            H->part[0], H->st);
-        finish_reduce(H->part[0], 0, H->scal, SC_SUM_M, H->st);
+        if (finish) finish_reduce(H->part[0], 0, H->scal, SC_SUM_M, H->st);
         return RECON_OK;
     }
     const double scale = fixed_scale((double)H->cells);
     launch_deposit_tracers(H->d, H->ox, H->oy, H->oz, H->w, scale, H->mfix, H->st);
     launch_mass_coef(H->cells, H->mfix, 1.0 / scale, H->p.a_min, H->m, H->a64,
                      H->mixed ? H->c32[0] : nullptr, H->part[0], H->st);
-    finish_reduce(H->part[0], 0, H->scal, SC_SUM_M, H->st);
+    if (finish) finish_reduce(H->part[0], 0, H->scal, SC_SUM_M, H->st);
     return RECON_OK;
 }
 
@@ -494,11 +495,10 @@ int deposit_step(Handle* H) {
 void step_head(Handle* H, const CtlHandles& h) {
     const recon_params& p = H->p;
     if (H->ckpt) launch_ckpt_state(H->ctl, H->cells, H->phi, H->ox, H->oy, H->oz, H->ckpt, H->st);
-    deposit_step(H);
+    deposit_step(H, false);
     SourceParams sp{p.xi_m, p.v_m, p.climiter};
-    launch_geometry_source(H->d, sp, H->phi, H->m, H->t, H->e6, H->part[0], H->part[1], H->st);
-    finish_reduce(H->part[0], 0, H->scal, SC_SUM_T, H->st);
-    finish_reduce(H->part[1], 1, H->scal, SC_MIN_DET, H->st);
+    launch_source(H->d, sp, H->phi, H->phi32, H->m, H->t, H->part[1], H->st);
+    finish_reduces({2, {{H->part[0], 0, SC_SUM_M}, {H->part[1], 0, SC_SUM_T}}}, H->scal, H->st);
     launch_smooth_S(H->d, p.s_side, H->t, H->scal + SC_SUM_T, H->s, nullptr, H->v3, nullptr, nullptr,
                     H->part[2], H->st);
     finish_reduce(H->part[2], 0, H->scal, SC_SUM_S2, H->st);
@@ -592,7 +592,7 @@ void step_tail(Handle* H, const CtlHandles& h) {
                     H->part[3], nullptr, H->st);
     FinishList fin{2, {{H->part[0], 0, SC_SUM_DPHI}, {H->part[3], 2, SC_MAX_DPHI}}};
     if (!H->replay_d) {
-        launch_limiter(H->d, H->lp, H->e6, H->dphi, H->phi32, H->dphi32, H->part[1], H->part[2],
+        launch_limiter(H->d, H->lp, H->phi, H->dphi, H->phi32, H->dphi32, H->part[1], H->part[2],
                        H->st);
         fin.f[fin.n++] = {H->part[1], 2, SC_MAX_K};
         fin.f[fin.n++] = {H->part[2], 2, SC_MAX_G};
@@ -608,6 +608,7 @@ void advance(Handle* H, const CtlHandles& h) {
     const int n = H->cells;
     const double* alpha = H->scal + SC_ALPHA;
     if (H->p.density_update == 1) {
+        launch_triad(H->d, H->phi, H->e6, H->st);
         launch_mass_literal(H->d, H->e6, H->dphi, alpha, H->m, H->v3m, H->st);
         launch_phi_advance(n, alpha, H->dphi, H->scal + SC_SUM_DPHI, H->phi, H->phi32, H->st);
     } else {
@@ -1127,7 +1128,7 @@ int adjoint(Handle* H, const double* gbar, double* grad) {
         launch_deposit_tracers(d, ox, oy, oz, H->w, scale, H->mfix, st);
         launch_mass_coef(cells, H->mfix, 1.0 / scale, p.a_min, H->m, H->a64,
                          H->mixed ? H->c32[0] : nullptr, H->part[0], st);
-        launch_geometry_source(d, sp, phi_k, H->m, H->t, H->e6, H->part[0], H->part[1], st);
+        launch_triad(d, phi_k, H->e6, st);
         launch_smooth_S(d, p.s_side, pd, nullptr, H->dphi, nullptr, H->v3, nullptr, nullptr, nullptr, st);
         launch_node_velocity(d, H->e6, H->dphi, H->v3, H->v3 + n, H->v3 + 2 * n, st);
         // back through the advance, V = e^-1 G and dphi = S phidot - mean
@@ -1299,7 +1300,8 @@ int recon_create(void** out, const recon_params* p_in, void* cuda_stream) {
     } while (0)
     AL(H->rho, n); AL(H->w, n); AL(H->ox, n); AL(H->oy, n); AL(H->oz, n);
     AL(H->phi, n); AL(H->m, n); AL(H->a64, n); AL(H->t, n); AL(H->s, n);
-    AL(H->phidot, n); AL(H->dphi, n); AL(H->v3, 3 * n); AL(H->mfix, n); AL(H->e6, 6 * n);
+    AL(H->phidot, n); AL(H->dphi, n); AL(H->v3, 3 * n); AL(H->mfix, n);
+    if (p->density_update == 1 || p->checkpoint) AL(H->e6, 6 * n);
     AL(H->F64, 3 * n); AL(H->D64, n); AL(H->phi32, n); AL(H->dphi32, n);
     if (p->warm_start == 2) AL(H->phidot_prev, n);
     if (p->density_update == 1) AL(H->v3m, 6 * n);

@@ -301,11 +301,12 @@ void launch_deposit_tracers(const Dims& d, const double* ox, const double* oy, c
                             cudaStream_t st);
 void launch_mass_coef(int cells, unsigned long long* mfix, double inv_scale, double a_min,
                       double* m, double* a64, float* a32, double* partials, cudaStream_t st);
-// e6 (6 x cells): the triad e = I + Hess phi (xx, yy, zz, xy, xz, yz) of the
-// step, written by the geometry pass and read by the limiter and the advance.
-void launch_geometry_source(const Dims& d, const SourceParams& sp, const double* phi,
-                            const double* m, double* t, double* e6, double* part_sum,
-                            double* part_min, cudaStream_t st);
+// e6 (6 x cells): the triad e = I + Hess phi (xx, yy, zz, xy, xz, yz), for the
+// adjoint and the carried mass of App. A's variant.
+void launch_triad(const Dims& d, const double* phi, double* e6, cudaStream_t st);
+// t = Sigma + C + E from phi (and its FP32 copy) and m, and partial sums of t.
+void launch_source(const Dims& d, const SourceParams& sp, const double* phi, const float* phi32, const double* m,
+                   double* t, double* part_sum, cudaStream_t st);
 // S in three axis passes through tmp2 (2 x cells scratch); out32 (optional)
 // receives an FP32 copy of the result; part_sum (with out32 and part_max) its
 // sum and largest magnitude, part_sq its sum of squares, or neither.
@@ -314,7 +315,7 @@ void launch_smooth_S(const Dims& d, double s_side, const double* in, const doubl
                      double* part_sq, cudaStream_t st);
 // phi32, dphi32: FP32 copies of phi and dphi used to screen nodes that clear
 // the limiter's floor by a wide margin.
-void launch_limiter(const Dims& d, const LimiterParams& lp, const double* e6, const double* dphi,
+void launch_limiter(const Dims& d, const LimiterParams& lp, const double* phi, const double* dphi,
                     const float* phi32, const float* dphi32, double* part_k, double* part_g,
                     cudaStream_t st);
 void launch_node_velocity(const Dims& d, const double* e6, const double* dphi, double* vx,

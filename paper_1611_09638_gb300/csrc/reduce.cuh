@@ -38,4 +38,11 @@ __device__ inline double block_reduce(double v) {
     return v;
 }
 
+// Thread 0 of a block of a grid smaller than `total` blocks: the block's
+// partial, and 0 for the partials that no block has.
+__device__ inline void put_partial(double* part, double v, int total) {
+    part[blockIdx.x] = v;
+    for (int b = blockIdx.x + gridDim.x; b < total; b += gridDim.x) part[b] = 0.0;
+}
+
 }  // namespace recon

@@ -16,12 +16,6 @@ inline int nblocks(long long work) { return (int)((work + kThreads - 1) / kThrea
 
 // ---------------------------------------------------------------- helpers
 
-// lambda_min(M) > floor by Sylvester's criterion on M - floor I.
-__device__ inline bool pd_above(Sym3 M, double floor) {
-    M.xx -= floor, M.yy -= floor, M.zz -= floor;
-    return M.xx > 0.0 && (M.xx * M.yy - M.xy * M.xy) > 0.0 && det3(M) > 0.0;
-}
-
 // 1 / n for a power of two n (< 2^1023), exactly, from the exponent bits
 // (integer work only; x * inv_pow2(n) equals x / n bit for bit).
 __device__ inline double inv_pow2(int n) {
@@ -267,44 +261,6 @@ __global__ void k_mass_coef(int cells, unsigned long long* __restrict__ mfix, do
     if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-// Source of App. A Eq. (elliptic) before smoothing: t = Sigma + C + E with
-// Sigma = 1 - m, C(lambda0) the compression limiter of the triad
-// e = I + Hess phi and E = -2 H(sqrt_g - v_m) |Sigma| the expansion limiter.
-// lambda0 only matters where it is below xi_m (for the soft and step readings
-// C vanishes above it); the Gershgorin bound skips the eigenvalue elsewhere.
-__global__ void k_geometry_source(Dims d, SourceParams sp, const double* __restrict__ phi,
-                                  const double* __restrict__ m, double* __restrict__ t,
-                                  double* __restrict__ e6, double* __restrict__ psum,
-                                  double* __restrict__ pmin) {
-    double s = 0.0, mdet = INFINITY;
-    const size_t n = (size_t)d.cells;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells; c += gridDim.x * blockDim.x) {
-        int i, j, k;
-        cell_coords(d, c, i, j, k);
-        Sym3 e = hessian(d, phi, i, j, k);
-        e.xx += 1.0, e.yy += 1.0, e.zz += 1.0;
-        // the triad is kept for the limiter and the advance of this step
-        e6[c] = e.xx, e6[n + c] = e.yy, e6[2 * n + c] = e.zz;
-        e6[3 * n + c] = e.xy, e6[4 * n + c] = e.xz, e6[5 * n + c] = e.yz;
-        const double g = det3(e);
-        double C = 0.0;
-        const double gersh =
-            fmin(fmin(e.xx - fabs(e.xy) - fabs(e.xz), e.yy - fabs(e.xy) - fabs(e.yz)),
-                 e.zz - fabs(e.xz) - fabs(e.yz));
-        if (sp.climiter == 1 || gersh < sp.xi_m) C = climit(sp.climiter, sp.xi_m, min_eig_sym3(e));
-        const double Sigma = 1.0 - m[c];
-        const double E = g - sp.v_m > 0.0 ? -2.0 * fabs(Sigma) : 0.0;
-        const double v = Sigma + C + E;
-        t[c] = v;
-        s += v;
-        mdet = fmin(mdet, g);
-    }
-    s = block_reduce<OpSum>(s);
-    if (threadIdx.x == 0) psum[blockIdx.x] = s;
-    mdet = block_reduce<OpMin>(mdet);
-    if (threadIdx.x == 0) pmin[blockIdx.x] = mdet;
-}
-
 // One axis of the smoothing operator S (a weighted mean over the 3x3x3
 // neighbourhood, separable into (w, 1-2w, w) along each axis): out =
 // w in[-1] + (1-2w) in[0] + w in[+1] along `axis`, minus (*shift_sum / cells)
@@ -437,17 +393,11 @@ __global__ void __launch_bounds__(SJ* SK, kSPerSM) k_smooth_S_stream(
     }
     if (SUM || SQ) {
         acc = block_reduce<OpSum>(acc);
-        if (threadIdx.x == 0) {
-            part[blockIdx.x] = acc;
-            if (blockIdx.x + kSBlocks < kRedBlocks) part[blockIdx.x + kSBlocks] = 0.0;
-        }
+        if (threadIdx.x == 0) put_partial(part, acc, kRedBlocks);
     }
     if (SUM) {
         const double v = block_reduce<OpMax>((double)mx);
-        if (threadIdx.x == 0) {
-            pmax[blockIdx.x] = v;
-            if (blockIdx.x + kSBlocks < kRedBlocks) pmax[blockIdx.x + kSBlocks] = 0.0;
-        }
+        if (threadIdx.x == 0) put_partial(pmax, v, kRedBlocks);
     }
 }
 
@@ -462,143 +412,8 @@ void launch_smooth_stream(const Dims& d, double ws, const double* in, const doub
         k_smooth_S_stream<QUARTER, false, false><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, nullptr, part_max);
 }
 
-template <typename T>
-struct Hess3 {
-    T xx, yy, zz, xy, xz, yz;
-};
-
-// Hessian in FP32 of an FP32 copy, and the largest |value| it read.
-__device__ inline Hess3<float> hessian32(const Dims& d, const float* __restrict__ f, int i, int j,
-                                         int k, float& vmax) {
-    float v[19];
-    v[0] = f[cell_index(d, i, j, k)];
-    v[1] = f[cell_index(d, i + 1, j, k)], v[2] = f[cell_index(d, i - 1, j, k)];
-    v[3] = f[cell_index(d, i, j + 1, k)], v[4] = f[cell_index(d, i, j - 1, k)];
-    v[5] = f[cell_index(d, i, j, k + 1)], v[6] = f[cell_index(d, i, j, k - 1)];
-    v[7] = f[cell_index(d, i + 1, j + 1, k)], v[8] = f[cell_index(d, i + 1, j - 1, k)];
-    v[9] = f[cell_index(d, i - 1, j + 1, k)], v[10] = f[cell_index(d, i - 1, j - 1, k)];
-    v[11] = f[cell_index(d, i + 1, j, k + 1)], v[12] = f[cell_index(d, i + 1, j, k - 1)];
-    v[13] = f[cell_index(d, i - 1, j, k + 1)], v[14] = f[cell_index(d, i - 1, j, k - 1)];
-    v[15] = f[cell_index(d, i, j + 1, k + 1)], v[16] = f[cell_index(d, i, j + 1, k - 1)];
-    v[17] = f[cell_index(d, i, j - 1, k + 1)], v[18] = f[cell_index(d, i, j - 1, k - 1)];
-    vmax = 0.0f;
-#pragma unroll
-    for (int q = 0; q < 19; ++q) vmax = fmaxf(vmax, fabsf(v[q]));
-    Hess3<float> H;
-    H.xx = v[1] - 2.0f * v[0] + v[2];
-    H.yy = v[3] - 2.0f * v[0] + v[4];
-    H.zz = v[5] - 2.0f * v[0] + v[6];
-    H.xy = 0.25f * (v[7] - v[8] - v[9] + v[10]);
-    H.xz = 0.25f * (v[11] - v[12] - v[13] + v[14]);
-    H.yz = 0.25f * (v[15] - v[16] - v[17] + v[18]);
-    return H;
-}
-
-// Sylvester's test of N = M - floor I in FP32 with a bound on its error:
-// returns +1 when N is certainly positive definite, -1 when it certainly is
-// not, 0 when FP32 cannot tell.  eps bounds the error of every entry of M;
-// the minors' bounds add the propagated entry errors and the FP32 roundings
-// of their own evaluation (u = 2^-24).
-__device__ inline int sylvester32(float xx, float yy, float zz, float xy, float xz, float yz,
-                                  float floor, float eps) {
-    constexpr float u = 5.96046448e-8f;
-    xx -= floor, yy -= floor, zz -= floor;
-    const float big = fmaxf(fmaxf(fabsf(xx), fabsf(yy)), fmaxf(fabsf(zz),
-                            fmaxf(fabsf(xy), fmaxf(fabsf(xz), fabsf(yz)))));
-    const float en = eps + 2.0f * u * (big + floor);  // entries of N
-    const float m1 = xx;
-    const float m2 = xx * yy - xy * xy;
-    const float m3 = xx * (yy * zz - yz * yz) - xy * (xy * zz - yz * xz) + xz * (xy * yz - yy * xz);
-    const float e1 = en;
-    const float e2 = 4.0f * en * big + en * en + 8.0f * u * big * big;
-    const float e3 = 9.0f * en * big * big + 3.0f * en * en * big + en * en * en + 72.0f * u * big * big * big;
-    if (m1 < -e1 || m2 < -e2 || m3 < -e3) return -1;
-    if (m1 > e1 && m2 > e2 && m3 > e3) return 1;
-    return 0;
-}
-
-// Step limiter, per node: the smallest k in [0, kmax] with
-// lambda_min(e + 2^-k Hess dphi) > floor (kmax + 1 if none), e = I + Hess phi
-// the FP64 triad stored by k_geometry_source, and max_a |central grad_a
-// dphi|.  Both are max-reduced over the grid.
-// Each alpha is first tested in FP32 on Hessians of FP32 copies of phi and
-// dphi, with a bound on every rounding involved (an entry of a Hessian
-// combines at most four stencil values of magnitude <= vmax; the FP32 copies
-// and at most four operations each round by 2^-24 relative, so 32 u vmax
-// bounds its error with room to spare).  Only when FP32 cannot certify the answer does the node
-// take the FP64 test (Sylvester's criterion on the FP64 triad); where FP32
-// certifies it, the FP64 test gives the same answer, so every decision is the
-// FP64 one while most nodes issue no FP64 arithmetic beyond the move limit.
-__global__ void k_limiter(Dims d, LimiterParams lp, const double* __restrict__ e6,
-                          const double* __restrict__ dphi, const float* __restrict__ phi32,
-                          const float* __restrict__ dphi32, double* __restrict__ pk,
-                          double* __restrict__ pg) {
-    constexpr float u = 5.96046448e-8f;
-    double kk = 0.0;
-    unsigned long long gbits = 0ull;  // max |G| as the bits of a non-negative double
-    const size_t n = (size_t)d.cells;
-    const float floor32 = (float)lp.lambda_floor;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells; c += gridDim.x * blockDim.x) {
-        int i, j, k;
-        cell_coords(d, c, i, j, k);
-        // move limit: central differences of dphi in FP64 (the max is taken on
-        // the bit patterns, 0.5 is applied once per block)
-        const double gx = dphi[cell_index(d, i + 1, j, k)] - dphi[cell_index(d, i - 1, j, k)];
-        const double gy = dphi[cell_index(d, i, j + 1, k)] - dphi[cell_index(d, i, j - 1, k)];
-        const double gz = dphi[cell_index(d, i, j, k + 1)] - dphi[cell_index(d, i, j, k - 1)];
-        const unsigned long long mask = 0x7fffffffffffffffull;
-        gbits = max(gbits, (unsigned long long)__double_as_longlong(gx) & mask);
-        gbits = max(gbits, (unsigned long long)__double_as_longlong(gy) & mask);
-        gbits = max(gbits, (unsigned long long)__double_as_longlong(gz) & mask);
-        float vm0, vm1;
-        const Hess3<float> A = hessian32(d, phi32, i, j, k, vm0);
-        const Hess3<float> B = hessian32(d, dphi32, i, j, k, vm1);
-        bool have64 = false;
-        Sym3 e, H1;
-        int kn = lp.kmax + 1;
-        float al = 1.0f;
-        for (int q = 0; q <= lp.kmax; ++q, al *= 0.5f) {
-            const float mxx = 1.0f + A.xx + al * B.xx, myy = 1.0f + A.yy + al * B.yy;
-            const float mzz = 1.0f + A.zz + al * B.zz, mxy = A.xy + al * B.xy;
-            const float mxz = A.xz + al * B.xz, myz = A.yz + al * B.yz;
-            const float big = fmaxf(fmaxf(fabsf(mxx), fabsf(myy)),
-                                    fmaxf(fabsf(mzz), fmaxf(fabsf(mxy), fmaxf(fabsf(mxz), fabsf(myz)))));
-            // inputs and Hessian arithmetic (|entry| <= 4 vmax), then the two
-            // additions forming M
-            const float eps = 32.0f * u * (vm0 + al * vm1) + 4.0f * u * (big + 1.0f);
-            const int v = sylvester32(mxx, myy, mzz, mxy, mxz, myz, floor32, eps);
-            bool pass;
-            if (v != 0) {
-                pass = v > 0;
-            } else {
-                if (!have64) {
-                    e.xx = e6[c], e.yy = e6[n + c], e.zz = e6[2 * n + c];
-                    e.xy = e6[3 * n + c], e.xz = e6[4 * n + c], e.yz = e6[5 * n + c];
-                    H1 = hessian(d, dphi, i, j, k);
-                    have64 = true;
-                }
-                const double al64 = ldexp(1.0, -q);
-                Sym3 M;
-                M.xx = e.xx + al64 * H1.xx, M.yy = e.yy + al64 * H1.yy, M.zz = e.zz + al64 * H1.zz;
-                M.xy = e.xy + al64 * H1.xy, M.xz = e.xz + al64 * H1.xz, M.yz = e.yz + al64 * H1.yz;
-                pass = pd_above(M, lp.lambda_floor);
-            }
-            if (pass) {
-                kn = q;
-                break;
-            }
-        }
-        kk = fmax(kk, (double)kn);
-    }
-    kk = block_reduce<OpMax>(kk);
-    if (threadIdx.x == 0) pk[blockIdx.x] = kk;
-    double gm = 0.5 * __longlong_as_double((long long)gbits);
-    gm = block_reduce<OpMax>(gm);
-    if (threadIdx.x == 0) pg[blockIdx.x] = gm;
-}
-
 // V = e^-1 G at every node: e = I + Hess phi (before the step; stored by
-// k_geometry_source), G the central-difference gradient of dphi; e^-1 from
+// launch_triad), G the central-difference gradient of dphi; e^-1 from
 // the adjugate of the symmetric e.
 __global__ void k_node_velocity(Dims d, const double* __restrict__ e6,
                                 const double* __restrict__ dphi, double* __restrict__ vx,
@@ -842,7 +657,7 @@ __device__ void finish(const double* __restrict__ partials, double* __restrict__
     if (threadIdx.x == 0) scalars[slot] = v;
 }
 
-// Finishes several reductions, a block each (4.3 us a launch, whatever it holds).
+// Finishes several reductions, a block each.
 __global__ void k_finish(FinishList l, double* __restrict__ scalars) {
     const Finish f = l.f[blockIdx.x];
     if (f.op == 0) finish<OpSum>(f.partials, scalars, f.slot);
@@ -854,7 +669,7 @@ __global__ void k_finish(FinishList l, double* __restrict__ scalars) {
 
 void finish_reduces(const FinishList& l, double* scalars, cudaStream_t st) {
     launch_counter()++;
-    k_finish<<<l.n, 1024, 0, st>>>(l, scalars);
+    k_finish<<<l.n, 256, 0, st>>>(l, scalars);
 }
 
 void finish_reduce(const double* partials, int op, double* scalars, int slot, cudaStream_t st) {
@@ -914,13 +729,6 @@ void launch_mass_coef(int cells, unsigned long long* mfix, double inv_scale, dou
                                                     partials);
 }
 
-void launch_geometry_source(const Dims& d, const SourceParams& sp, const double* phi,
-                            const double* m, double* t, double* e6, double* part_sum,
-                            double* part_min, cudaStream_t st) {
-    launch_counter()++;
-    k_geometry_source<<<kRedBlocks, kRedThreads, 0, st>>>(d, sp, phi, m, t, e6, part_sum, part_min);
-}
-
 void launch_smooth_S(const Dims& d, double s_side, const double* in, const double* shift_sum,
                      double* out, float* out32, double* tmp2, double* part_sum, double* part_max,
                      double* part_sq, cudaStream_t st) {
@@ -937,13 +745,6 @@ void launch_smooth_S(const Dims& d, double s_side, const double* in, const doubl
                                                       tmp2 + d.cells, nullptr, nullptr, nullptr, nullptr);
     k_smooth_axis<<<kRedBlocks, kRedThreads, 0, st>>>(d, 0, s_side, tmp2 + d.cells, shift_sum,
                                                       out, out32, part_sum, part_max, part_sq);
-}
-
-void launch_limiter(const Dims& d, const LimiterParams& lp, const double* e6, const double* dphi,
-                    const float* phi32, const float* dphi32, double* part_k, double* part_g,
-                    cudaStream_t st) {
-    launch_counter()++;
-    k_limiter<<<kRedBlocks, kRedThreads, 0, st>>>(d, lp, e6, dphi, phi32, dphi32, part_k, part_g);
 }
 
 void launch_node_velocity(const Dims& d, const double* e6, const double* dphi, double* vx,

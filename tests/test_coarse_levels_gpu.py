@@ -92,3 +92,23 @@ def test_node_displacements_match_the_oracle(shape, alpha):
         phi, m = R.field("phi").cpu().numpy(), R.field("mass").cpu().numpy()
     assert np.linalg.norm(phi - ref.phi) <= 1e-9 * np.linalg.norm(ref.phi)
     assert np.abs(m - ref.m).max() <= 1e-9
+
+
+@pytest.mark.parametrize("climiter", [0, 1, 2])
+@pytest.mark.parametrize("shape", [(8, 8, 8), (8, 8, 32), (16, 8, 64), (32, 16, 32)])
+def test_source_and_limiter_match_the_oracle(shape, climiter):
+    """The screened source and limiter on strongly deformed maps where both
+    limiters act (v_m = 1.5, xi_m = 0.5), every reading of C: the step lengths
+    exactly and phi within the FP64 bar."""
+    r = np.random.default_rng(sum(shape) + climiter)
+    k = np.meshgrid(*[np.arange(n) * 2 * np.pi / n for n in shape], indexing="ij")
+    rho = np.exp(1.2 * np.sin(k[0] + 1) * np.cos(k[1]) + 0.8 * np.cos(k[2] + k[0]) + 0.3 * r.standard_normal(shape))
+    kw = dict(climiter=climiter, v_m=1.5, xi_m=0.5)
+    ref = O.solve(O.OracleParams(n=shape, k_max=6, tol_in=1e-12, max_vcycles=100, **kw), rho)
+    with Recon(shape, k_max=6, tol_in=1e-12, max_vcycles=100, **kw) as R:
+        R.deposit_grid(torch.from_numpy(rho).cuda())
+        st = R.solve()
+        phi = R.field("phi").cpu().numpy()
+    assert st.status == ref.status
+    np.testing.assert_array_equal(st.alpha, ref.alpha)
+    assert np.linalg.norm(phi - ref.phi) <= BARS["fp64"] * np.linalg.norm(ref.phi)
