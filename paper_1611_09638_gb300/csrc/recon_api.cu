@@ -134,6 +134,7 @@ struct Handle {
     cudaStream_t gst[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // capture streams
     cudaGraphExec_t solve_exec = nullptr;
     GraphCounts gn{};
+    int stats_kernels = 0;  // kernels of the end-of-solve statistics
 
     bool have_density = false, solved = false;
     double rho_sum = 0.0;
@@ -944,9 +945,6 @@ int build_solve_graph(Handle* H) {
     return RECON_OK;
 }
 
-// Kernels of the end-of-solve statistics (geometry, delta_r, 3 reductions).
-constexpr int kStatsKernels = 5;
-
 // Launches the whole solve (graph mode) and, with stats, the end-of-solve
 // statistics and the readback of the control block and the per-step
 // records; nothing waits for the device.
@@ -959,11 +957,8 @@ int solve_launch(Handle* H, bool want_stats) {
     CK(cudaGraphLaunch(H->solve_exec, H->st));
     CK(cudaEventRecord(H->ev1, H->st));
     if (want_stats) {
-        launch_geometry_out(H->d, H->phi, nullptr, nullptr, H->part[0], H->part[1], H->st);
-        finish_reduce(H->part[0], 1, H->scal, SC_MIN_DET, H->st);
-        finish_reduce(H->part[1], 1, H->scal, SC_MIN_LAM, H->st);
-        launch_delta_r(H->d, H->phi, H->t, H->part[2], H->st);
-        finish_reduce(H->part[2], 2, H->scal, SC_MAX_DR, H->st);
+        H->stats_kernels =
+            launch_extrema(H->d, H->phi, H->phi32, H->t, H->part[0], H->part[1], H->part[2], H->scal, H->st);
         CK(cudaMemcpyAsync(H->hscal, H->scal, SC_COUNT * sizeof(double), cudaMemcpyDeviceToHost, H->st));
     }
     CK(cudaMemcpyAsync(H->hctl, H->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, H->st));
@@ -1022,7 +1017,7 @@ int solve_finish(Handle* H, recon_stats* stats) {
     if (stats) {
         float ms = 0.f;
         cudaEventElapsedTime(&ms, H->ev0, H->ev1);
-        fill_stats(H, stats, ms, kk + kStatsKernels, true);
+        fill_stats(H, stats, ms, kk + H->stats_kernels, true);
         stats->smooth_ms = 0.0;
         stats->smooth_sweeps = 0;
         stats->smooth_bytes = 4.0 * (H->mixed ? sizeof(float) : sizeof(double)) * (double)H->cells;
@@ -1052,11 +1047,7 @@ int solve(Handle* H, recon_stats* stats) {
     if (stats) {
         float ms = 0.f;
         cudaEventElapsedTime(&ms, H->ev0, H->ev1);
-        launch_geometry_out(H->d, H->phi, nullptr, nullptr, H->part[0], H->part[1], H->st);
-        finish_reduce(H->part[0], 1, H->scal, SC_MIN_DET, H->st);
-        finish_reduce(H->part[1], 1, H->scal, SC_MIN_LAM, H->st);
-        launch_delta_r(H->d, H->phi, H->t, H->part[2], H->st);
-        finish_reduce(H->part[2], 2, H->scal, SC_MAX_DR, H->st);
+        launch_extrema(H->d, H->phi, H->phi32, H->t, H->part[0], H->part[1], H->part[2], H->scal, H->st);
         CK(cudaMemcpyAsync(H->hscal, H->scal, SC_COUNT * sizeof(double), cudaMemcpyDeviceToHost, H->st));
         CK(cudaMemcpyAsync(H->hctl, H->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, H->st));
         const size_t km = (size_t)std::max(H->p.k_max, 1);

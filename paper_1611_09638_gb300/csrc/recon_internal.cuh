@@ -70,13 +70,13 @@ enum Scalar {
     SC_SUM_RHO = 0,   // sum of the deposited density
     SC_BAD,           // nonzero if an input was NaN/Inf/negative (as double)
     SC_SUM_T,         // sum of t = Sigma + C + E
-    SC_MIN_DET,       // min det(I + Hess phi)
     SC_SUM_S2,        // sum of s^2
     SC_SUM_M,         // sum of m
     SC_RES2,          // sum of residual^2
     SC_SUM_DPHI,      // sum of S(phidot)
     SC_MAX_K,         // max over nodes of the per-node limiter exponent
     SC_MAX_G,         // max |grad dphi|
+    SC_MIN_DET,       // min det(I + Hess phi)
     SC_MIN_LAM,       // min lambda0
     SC_MAX_DR,        // max delta_r
     SC_ALPHA,         // step length of the current step
@@ -344,6 +344,10 @@ void launch_delta_r(const Dims& d, const double* phi, double* out, double* part_
 void launch_mesh_x(const Dims& d, const double* phi, double h, double* out, cudaStream_t st);
 void launch_geometry_out(const Dims& d, const double* phi, double* det, double* lam,
                          double* part_min_det, double* part_min_lam, cudaStream_t st);
+// min det, min lambda0 and max delta_r of phi into scal (SC_MIN_DET,
+// SC_MIN_LAM, SC_MAX_DR); scratch: cells doubles.  Returns the kernels launched.
+int launch_extrema(const Dims& d, const double* phi, const float* phi32, double* scratch, double* part_det,
+                   double* part_lam, double* part_dr, double* scal, cudaStream_t st);
 void launch_scale(int cells, const double* in, double s, double* out, cudaStream_t st);
 
 // ---- device-side control of the iteration (control.cu) -----------------

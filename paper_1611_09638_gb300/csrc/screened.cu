@@ -370,6 +370,136 @@ __global__ void k_limiter_node(Dims d, LimiterParams lp, const double* __restric
     if (threadIdx.x == 0) pg[blockIdx.x] = gm;
 }
 
+// The outputs of one node in FP64.  Not inlined, so that the fields and the
+// closing statistics come from the same instructions.
+__device__ __noinline__ double det64(const Sym3& e) { return det3(e); }
+__device__ __noinline__ double lambda64(const Sym3& e) { return min_eig_sym3(e); }
+__device__ __noinline__ Sym3 triad64(const Dims& d, const double* __restrict__ phi, int i, int j, int k) {
+    Sym3 e = hessian(d, phi, i, j, k);
+    e.xx += 1.0, e.yy += 1.0, e.zz += 1.0;
+    return e;
+}
+// delta_r = -lap f with the 7-point Laplacian.
+__device__ __noinline__ double delta_r_at(const Dims& d, const double* __restrict__ f, int i, int j, int k) {
+    const double p = f[cell_index(d, i, j, k)];
+    return -((f[cell_index(d, i + 1, j, k)] - 2.0 * p + f[cell_index(d, i - 1, j, k)]) +
+             (f[cell_index(d, i, j + 1, k)] - 2.0 * p + f[cell_index(d, i, j - 1, k)]) +
+             (f[cell_index(d, i, j, k + 1)] - 2.0 * p + f[cell_index(d, i, j, k - 1)]));
+}
+
+
+__global__ void k_delta_r(Dims d, const double* __restrict__ phi, double* __restrict__ out,
+                          double* __restrict__ pmax) {
+    double mx = -INFINITY;
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells; c += gridDim.x * blockDim.x) {
+        int i, j, k;
+        cell_coords(d, c, i, j, k);
+        const double v = delta_r_at(d, phi, i, j, k);
+        out[c] = v;
+        mx = fmax(mx, v);
+    }
+    mx = block_reduce<OpMax>(mx);
+    if (threadIdx.x == 0) pmax[blockIdx.x] = mx;
+}
+
+__global__ void k_geometry_out(Dims d, const double* __restrict__ phi, double* __restrict__ det,
+                               double* __restrict__ lam, double* __restrict__ pdet,
+                               double* __restrict__ plam) {
+    double md = INFINITY, ml = INFINITY;
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells; c += gridDim.x * blockDim.x) {
+        int i, j, k;
+        cell_coords(d, c, i, j, k);
+        const Sym3 e = triad64(d, phi, i, j, k);
+        const double g = det64(e);
+        if (det) det[c] = g;
+        md = fmin(md, g);
+        // lambda0 >= the Gershgorin bound, so without a per-node output the
+        // eigenvalue is needed only where that bound is below the running min
+        const double gersh =
+            fmin(fmin(e.xx - fabs(e.xy) - fabs(e.xz), e.yy - fabs(e.xy) - fabs(e.yz)),
+                 e.zz - fabs(e.xz) - fabs(e.yz));
+        if (lam || gersh < ml) {
+            const double l = lambda64(e);
+            if (lam) lam[c] = l;
+            ml = fmin(ml, l);
+        }
+    }
+    md = block_reduce<OpMin>(md);
+    if (threadIdx.x == 0) pdet[blockIdx.x] = md;
+    ml = block_reduce<OpMin>(ml);
+    if (threadIdx.x == 0) plam[blockIdx.x] = ml;
+}
+
+// The solve's closing statistics: min det e, min lambda0 and max delta_r, each
+// the FP64 value of the node that attains it.  The first pass (EXACT = false)
+// bounds them from FP32 values (the smallest upper bounds, the largest lower
+// one), the second evaluates in FP64 the nodes that the bounds leave open.
+// lambda0 in FP32 comes from the closed form: Weyl's theorem bounds what the
+// entries' errors do to it, and the angle's error, at most the square root of
+// the rounding of the determinant that it is taken from, is covered by 2^-8 p.
+// 512^3: 26 -> 2.0 ms for all three (FP64 at every node, 23 of them for det and
+// lambda0).
+template <bool EXACT>
+__global__ void __launch_bounds__(GJ* GK, GPERSM) k_extrema_stream(Dims d, const double* __restrict__ phi,
+                                                                   const float* __restrict__ phi32,
+                                                                   const double* __restrict__ bounds,
+                                                                   double* __restrict__ pdet,
+                                                                   double* __restrict__ plam,
+                                                                   double* __restrict__ pdr) {
+    __shared__ float buf[2][1][GN];
+    const int lj = threadIdx.x / GK, lk = threadIdx.x % GK;
+    const int own = (lj + 1) * GPK + lk + 1;
+    const float bd = EXACT ? __double2float_ru(bounds[0]) : 0.f, bl = EXACT ? __double2float_ru(bounds[1]) : 0.f,
+                br = EXACT ? __double2float_rd(bounds[2]) : 0.f;
+    Column32 col{};
+    float fd = INFINITY, fl = INFINITY, fr = -INFINITY;
+    double md = INFINITY, ml = INFINITY, mr = -INFINITY;
+    const float* const fields[1] = {phi32};
+    stream_planes<1>(
+        d, fields, buf, [&] { col = Column32{}; },
+        [&](int p, bool done, int j0, int k0, int w) {
+            float gy, gz;
+            const Hess32 h = col.feed(buf[w][0] + own, gy, gz);
+            if (!done) return;
+            const float xx = 1.f + h.xx, yy = 1.f + h.yy, zz = 1.f + h.zz;
+            const float big = fmaxf(fmaxf(fmaxf(fabsf(xx), fabsf(yy)), fabsf(zz)),
+                                    fmaxf(fabsf(h.xy), fmaxf(fabsf(h.xz), fabsf(h.yz))));
+            const float eps = 32.0f * kU * h.vmax + 4.0f * kU * (big + 1.0f);
+            const float det = xx * (yy * zz - h.yz * h.yz) - h.xy * (h.xy * zz - h.yz * h.xz) +
+                              h.xz * (h.xy * h.yz - yy * h.xz);
+            const float ed = 9.0f * eps * big * big + 3.0f * eps * eps * big + eps * eps * eps +
+                             72.0f * kU * big * big * big;
+            const float q = (xx + yy + zz) * (1.f / 3.f);
+            const float b1 = xx - q, b2 = yy - q, b3 = zz - q;
+            const float p2 = b1 * b1 + b2 * b2 + b3 * b3 + 2.f * (h.xy * h.xy + h.xz * h.xz + h.yz * h.yz);
+            const float pp = sqrtf(p2 * (1.f / 6.f)), ip = 1.f / fmaxf(pp, 1e-30f);
+            const float r = 0.5f * ip * ip * ip * (b1 * (b2 * b3 - h.yz * h.yz) - h.xy * (h.xy * b3 - h.yz * h.xz) +
+                                                  h.xz * (h.xy * h.yz - b2 * h.xz));
+            const float lam = q + 2.f * pp * cosf(acosf(fminf(1.f, fmaxf(-1.f, r))) * (1.f / 3.f) + 2.0943951f);
+            const float el = 3.f * eps + 0.00390625f * pp + 16.f * kU * big;
+            const float dr = -(h.xx + h.yy + h.zz), er = 3.f * eps + 8.f * kU * (big + 1.f);
+            if (!EXACT) {
+                fd = fminf(fd, det + ed), fl = fminf(fl, lam + el), fr = fmaxf(fr, dr - er);
+            } else {
+                const bool od = !(det - ed > bd), ol = !(lam - el > bl), orr = !(dr + er < br);
+                if (od || ol || orr) {
+                    const int i = p - 1, j = j0 + lj, k = k0 + lk;
+                    const Sym3 e = triad64(d, phi, i, j, k);
+                    md = fmin(md, det64(e));
+                    if (ol) ml = fmin(ml, lambda64(e));
+                    if (orr) mr = fmax(mr, delta_r_at(d, phi, i, j, k));
+                }
+            }
+        });
+    md = block_reduce<OpMin>(EXACT ? md : (double)fd);
+    ml = block_reduce<OpMin>(EXACT ? ml : (double)fl);
+    mr = block_reduce<OpMax>(EXACT ? mr : (double)fr);
+    if (threadIdx.x == 0)
+        for (int b = blockIdx.x, first = 1; b < kRedBlocks; b += gridDim.x, first = 0) {
+            pdet[b] = first ? md : INFINITY, plam[b] = first ? ml : INFINITY, pdr[b] = first ? mr : -INFINITY;
+        }
+}
+
 // The triad e = I + Hess phi (6 x cells: xx, yy, zz, xy, xz, yz), for the
 // adjoint and App. A's density update.
 __global__ void k_triad(Dims d, const double* __restrict__ phi, double* __restrict__ e6) {
@@ -407,6 +537,36 @@ void launch_limiter(const Dims& d, const LimiterParams& lp, const double* phi, c
         return;
     }
     k_limiter_node<<<kRedBlocks, kRedThreads, 0, st>>>(d, lp, phi, dphi, part_k, part_g);
+}
+
+void launch_delta_r(const Dims& d, const double* phi, double* out, double* part_max,
+                    cudaStream_t st) {
+    launch_counter()++;
+    k_delta_r<<<kRedBlocks, kRedThreads, 0, st>>>(d, phi, out, part_max);
+}
+
+void launch_geometry_out(const Dims& d, const double* phi, double* det, double* lam,
+                         double* part_min_det, double* part_min_lam, cudaStream_t st) {
+    launch_counter()++;
+    k_geometry_out<<<kRedBlocks, kRedThreads, 0, st>>>(d, phi, det, lam, part_min_det, part_min_lam);
+}
+
+int launch_extrema(const Dims& d, const double* phi, const float* phi32, double* scratch, double* part_det,
+                   double* part_lam, double* part_dr, double* scal, cudaStream_t st) {
+    const FinishList fin{3, {{part_det, 1, SC_MIN_DET}, {part_lam, 1, SC_MIN_LAM}, {part_dr, 2, SC_MAX_DR}}};
+    if (tiles(d)) {
+        static_assert(SC_MIN_LAM == SC_MIN_DET + 1 && SC_MAX_DR == SC_MIN_DET + 2, "the bounds are adjacent");
+        launch_counter() += 2;
+        k_extrema_stream<false><<<GBLOCKS, GJ * GK, 0, st>>>(d, phi, phi32, nullptr, part_det, part_lam, part_dr);
+        finish_reduces(fin, scal, st);
+        k_extrema_stream<true><<<GBLOCKS, GJ * GK, 0, st>>>(d, phi, phi32, scal + SC_MIN_DET, part_det, part_lam,
+                                                            part_dr);
+    } else {
+        launch_geometry_out(d, phi, nullptr, nullptr, part_det, part_lam, st);
+        launch_delta_r(d, phi, scratch, part_dr, st);
+    }
+    finish_reduces(fin, scal, st);
+    return tiles(d) ? 4 : 3;
 }
 
 void launch_triad(const Dims& d, const double* phi, double* e6, cudaStream_t st) {

@@ -588,23 +588,6 @@ __global__ void k_advance(Dims d, const long long* __restrict__ dx, const long l
     phi32[c] = (float)pn;
 }
 
-__global__ void k_delta_r(Dims d, const double* __restrict__ phi, double* __restrict__ out,
-                          double* __restrict__ pmax) {
-    double mx = -INFINITY;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells; c += gridDim.x * blockDim.x) {
-        int i, j, k;
-        cell_coords(d, c, i, j, k);
-        const double p = phi[c];
-        const double lap = (phi[cell_index(d, i + 1, j, k)] - 2.0 * p + phi[cell_index(d, i - 1, j, k)]) +
-                           (phi[cell_index(d, i, j + 1, k)] - 2.0 * p + phi[cell_index(d, i, j - 1, k)]) +
-                           (phi[cell_index(d, i, j, k + 1)] - 2.0 * p + phi[cell_index(d, i, j, k - 1)]);
-        out[c] = -lap;
-        mx = fmax(mx, -lap);
-    }
-    mx = block_reduce<OpMax>(mx);
-    if (threadIdx.x == 0) pmax[blockIdx.x] = mx;
-}
-
 __global__ void k_mesh_x(Dims d, const double* __restrict__ phi, double h, double* __restrict__ out) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= d.cells) return;
@@ -613,35 +596,6 @@ __global__ void k_mesh_x(Dims d, const double* __restrict__ phi, double h, doubl
     out[3 * c + 0] = ((double)i + 0.5 * (phi[cell_index(d, i + 1, j, k)] - phi[cell_index(d, i - 1, j, k)])) * h;
     out[3 * c + 1] = ((double)j + 0.5 * (phi[cell_index(d, i, j + 1, k)] - phi[cell_index(d, i, j - 1, k)])) * h;
     out[3 * c + 2] = ((double)k + 0.5 * (phi[cell_index(d, i, j, k + 1)] - phi[cell_index(d, i, j, k - 1)])) * h;
-}
-
-__global__ void k_geometry_out(Dims d, const double* __restrict__ phi, double* __restrict__ det,
-                               double* __restrict__ lam, double* __restrict__ pdet,
-                               double* __restrict__ plam) {
-    double md = INFINITY, ml = INFINITY;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells; c += gridDim.x * blockDim.x) {
-        int i, j, k;
-        cell_coords(d, c, i, j, k);
-        Sym3 e = hessian(d, phi, i, j, k);
-        e.xx += 1.0, e.yy += 1.0, e.zz += 1.0;
-        const double g = det3(e);
-        if (det) det[c] = g;
-        md = fmin(md, g);
-        // lambda0 >= the Gershgorin bound, so without a per-node output the
-        // eigenvalue is needed only where that bound is below the running min
-        const double gersh =
-            fmin(fmin(e.xx - fabs(e.xy) - fabs(e.xz), e.yy - fabs(e.xy) - fabs(e.yz)),
-                 e.zz - fabs(e.xz) - fabs(e.yz));
-        if (lam || gersh < ml) {
-            const double l = min_eig_sym3(e);
-            if (lam) lam[c] = l;
-            ml = fmin(ml, l);
-        }
-    }
-    md = block_reduce<OpMin>(md);
-    if (threadIdx.x == 0) pdet[blockIdx.x] = md;
-    ml = block_reduce<OpMin>(ml);
-    if (threadIdx.x == 0) plam[blockIdx.x] = ml;
 }
 
 __global__ void k_scale(int cells, const double* __restrict__ in, double s, double* __restrict__ out) {
@@ -780,21 +734,9 @@ void launch_phi_advance(int cells, const double* alpha, const double* dphi,
     k_phi_advance<<<nblocks(cells), kThreads, 0, st>>>(cells, alpha, dphi, sum_dphi, phi, phi32);
 }
 
-void launch_delta_r(const Dims& d, const double* phi, double* out, double* part_max,
-                    cudaStream_t st) {
-    launch_counter()++;
-    k_delta_r<<<kRedBlocks, kRedThreads, 0, st>>>(d, phi, out, part_max);
-}
-
 void launch_mesh_x(const Dims& d, const double* phi, double h, double* out, cudaStream_t st) {
     launch_counter()++;
     k_mesh_x<<<nblocks(d.cells), kThreads, 0, st>>>(d, phi, h, out);
-}
-
-void launch_geometry_out(const Dims& d, const double* phi, double* det, double* lam,
-                         double* part_min_det, double* part_min_lam, cudaStream_t st) {
-    launch_counter()++;
-    k_geometry_out<<<kRedBlocks, kRedThreads, 0, st>>>(d, phi, det, lam, part_min_det, part_min_lam);
 }
 
 void launch_scale(int cells, const double* in, double s, double* out, cudaStream_t st) {

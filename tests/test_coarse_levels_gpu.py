@@ -112,3 +112,17 @@ def test_source_and_limiter_match_the_oracle(shape, climiter):
     assert st.status == ref.status
     np.testing.assert_array_equal(st.alpha, ref.alpha)
     assert np.linalg.norm(phi - ref.phi) <= BARS["fp64"] * np.linalg.norm(ref.phi)
+
+
+@pytest.mark.parametrize("shape", [(8, 8, 8), (8, 8, 32), (64, 32, 32), (16, 64, 64)])
+def test_closing_statistics_are_those_of_the_fields(shape):
+    """min det, min lambda0 and max delta_r of a solve's record are the extrema
+    of the fields, to the last bit (the same FP64 arithmetic at the node that
+    attains each)."""
+    rho = _rough(shape, 3 * sum(shape))
+    with Recon(shape, precision="mixed", k_max=5) as R:
+        R.deposit_grid(torch.from_numpy(rho).cuda())
+        st = R.solve()
+        assert st.min_det == R.field("det").min().item()
+        assert st.min_lambda0 == R.field("lambda0").min().item()
+        assert st.max_delta_r == R.field("delta_r").max().item()
