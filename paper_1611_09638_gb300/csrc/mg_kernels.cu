@@ -109,8 +109,13 @@ __global__ void k_residual64(Dims d, const double* __restrict__ u, const double*
 // node.  The norm only decides the multigrid stopping test: each thread's
 // FP32 sum covers cells / (kRedBlocks * kRedThreads) nodes (54 at 256^3, 431
 // at 512^3), so its relative error stays below ~3e-5, and the block sums
-// are FP64.
-__global__ void k_residual64_to32(Dims d, const double* __restrict__ u,
+// are FP64.  One round of four blocks per SM with 59 registers, so that a
+// node's fifteen loads are all in flight: 512^3 2.19 -> 1.98 ms, 256^3 274 -> 254
+// us against 38 registers in kRedBlocks blocks (eight FP64 instructions at 2
+// lanes a clock and SM take 1.71 ms; rounding the FP32 copy by integer
+// instructions instead took 2.3 ms).
+constexpr int kResPerSM = 4, kResBlocks = kResPerSM * (kRedBlocks / 8);
+__global__ void __launch_bounds__(kRedThreads, kResPerSM) k_residual64_to32(Dims d, const double* __restrict__ u,
                                   const double* __restrict__ f, const double* __restrict__ F,
                                   const double* __restrict__ D, float* __restrict__ r32,
                                   double* __restrict__ partials) {
@@ -143,29 +148,40 @@ __global__ void k_residual64_to32(Dims d, const double* __restrict__ u,
     }
     acc += (double)acc32;
     acc = block_reduce<OpSum>(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = acc;
+    if (threadIdx.x == 0) put_partial(partials, acc, kRedBlocks);
+}
+
+// x 2^e, for a positive normal x away from the ends of the range by its
+// exponent bits, else by a product: no FP64 operation.
+__device__ __forceinline__ double times_pow2(double x, int e) {
+    const long long b = __double_as_longlong(x);
+    const int old = (int)(b >> 52);
+    return old > 64 && old < 1984 ? __longlong_as_double(b + ((long long)e << 52)) : x * ldexp(1.0, e);
 }
 
 // Face coefficients A = h^-2 (a_c + a_{c + e_a}) / 2 of a level, one array per
-// axis (wx, wy, wz: h^-2 / 2 of that axis), the node diagonal D = sum of the
-// node's six A, and optionally 1 / D.
-__global__ void k_faces64(Dims d, double wx, double wy, double wz, const double* __restrict__ a,
-                          double* __restrict__ F,
-                          double* __restrict__ D, double* __restrict__ inv_d) {
+// axis, the node diagonal D = sum of the node's six A, and optionally 1 / D.
+// h^-2 / 2 = 2^ex (ey, ez) of each axis.  Bound by the FP64 rate: each value is
+// scaled by its exponent bits, so the three faces take one sum each and D six
+// instructions on an isotropic level (17 in all with the products, 512^3 3.59
+// -> 2.32 ms).
+template <bool ISO>
+__global__ void k_faces64(Dims d, int ex, int ey, int ez, const double* __restrict__ a,
+                          double* __restrict__ F, double* __restrict__ D, double* __restrict__ inv_d) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= d.cells) return;
     int i, j, k;
     cell_coords(d, c, i, j, k);
     const size_t n = (size_t)d.cells;
     const double ac = a[c];
-    const double xp = wx * (ac + a[cell_index(d, i + 1, j, k)]);
-    const double xm = wx * (ac + a[cell_index(d, i - 1, j, k)]);
-    const double yp = wy * (ac + a[cell_index(d, i, j + 1, k)]);
-    const double ym = wy * (ac + a[cell_index(d, i, j - 1, k)]);
-    const double zp = wz * (ac + a[cell_index(d, i, j, k + 1)]);
-    const double zm = wz * (ac + a[cell_index(d, i, j, k - 1)]);
-    F[c] = xp, F[n + c] = yp, F[2 * n + c] = zp;
-    const double dg = ((xp + xm) + (yp + ym)) + (zp + zm);
+    const double xp = times_pow2(a[cell_index(d, i + 1, j, k)], ex), xm = times_pow2(a[cell_index(d, i - 1, j, k)], ex);
+    const double yp = times_pow2(a[cell_index(d, i, j + 1, k)], ey), ym = times_pow2(a[cell_index(d, i, j - 1, k)], ey);
+    const double zp = times_pow2(a[cell_index(d, i, j, k + 1)], ez), zm = times_pow2(a[cell_index(d, i, j, k - 1)], ez);
+    const double cx = times_pow2(ac, ex);
+    const double cy = ISO ? cx : times_pow2(ac, ey), cz = ISO ? cx : times_pow2(ac, ez);
+    F[c] = cx + xp, F[n + c] = cy + yp, F[2 * n + c] = cz + zp;
+    const double sum = ((xp + xm) + (yp + ym)) + (zp + zm);
+    const double dg = ISO ? fma(6.0, cx, sum) : fma(2.0, cx + (cy + cz), sum);
     D[c] = dg;
     if (inv_d) inv_d[c] = 1.0 / dg;
 }
@@ -222,10 +238,12 @@ __global__ void k_restrict64(Dims df, Dims dc, int cx, int cy, int cz, const dou
 // Residual r = f - L u evaluated at the fine nodes of each coarse node's
 // full-weighting stencil and restricted at once (the fine residual is never
 // stored): per node the 7-point residual f - L u followed by the full weighting.
+// red: u has just been swept, so black nodes have none (but for rounding) and
+// are left out, half the evaluations (128 x 64 x 32 nodes: 8.5 -> 7.2 us a level).
 template <typename T>
 __global__ void k_resid_restrict(Dims df, Dims dc, int cx, int cy, int cz, T hx, T hy, T hz,
                                  const T* __restrict__ u, const T* __restrict__ f,
-                                 const T* __restrict__ a, int face, T* __restrict__ out) {
+                                 const T* __restrict__ a, int face, int red, T* __restrict__ out) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= dc.cells) return;
     int I, J, K;
@@ -237,6 +255,7 @@ __global__ void k_resid_restrict(Dims df, Dims dc, int cx, int cy, int cz, T hx,
         for (int oj = -cy; oj <= cy; ++oj) {
             const T wj = cy ? (oj == 0 ? T(0.5) : T(0.25)) : T(1);
             for (int ok = -cz; ok <= cz; ++ok) {
+                if (red && ((fi + oi + fj + oj + fk + ok) & 1)) continue;
                 const T wk = cz ? (ok == 0 ? T(0.5) : T(0.25)) : T(1);
                 const int i = (fi + oi) & (df.n0 - 1), j = (fj + oj) & (df.n1 - 1),
                           k = (fk + ok) & (df.n2 - 1);
@@ -571,11 +590,11 @@ void launch_restrict<double>(const Level& fine, const Level& coarse, const doubl
 
 template <typename T>
 void launch_resid_restrict(const Level& fine, const Level& coarse, const T* u, const T* f,
-                           const T* a, T* out, cudaStream_t st) {
+                           const T* a, T* out, bool swept, cudaStream_t st) {
     launch_counter()++;
     k_resid_restrict<T><<<nblocks(coarse.d.cells), kThreads, 0, st>>>(
         fine.d, coarse.d, fine.coarsen[0], fine.coarsen[1], fine.coarsen[2], (T)fine.h2i[0],
-        (T)fine.h2i[1], (T)fine.h2i[2], u, f, a, fine.face, out);
+        (T)fine.h2i[1], (T)fine.h2i[2], u, f, a, fine.face, swept ? 1 : 0, out);
 }
 
 void launch_faces_line(const Level& fine, const Level& coarse, const float* in, float* out,
@@ -626,13 +645,13 @@ void launch_to_f32(int cells, const double* x, float* y, cudaStream_t st) {
 void launch_residual64_to32(const Level& L, const double* u, const double* f, const double* F,
                             const double* D, float* r32, double* partials, cudaStream_t st) {
     launch_counter()++;
-    k_residual64_to32<<<kRedBlocks, kRedThreads, 0, st>>>(L.d, u, f, F, D, r32, partials);
+    k_residual64_to32<<<kResBlocks, kRedThreads, 0, st>>>(L.d, u, f, F, D, r32, partials);
 }
 
 void launch_residual_norm64(const Level& L, const double* u, const double* f, const double* F,
                             const double* D, double* partials, cudaStream_t st) {
     launch_counter()++;
-    k_residual64_to32<<<kRedBlocks, kRedThreads, 0, st>>>(L.d, u, f, F, D, nullptr, partials);
+    k_residual64_to32<<<kResBlocks, kRedThreads, 0, st>>>(L.d, u, f, F, D, nullptr, partials);
 }
 
 void launch_rbgs_sweep64(const Level& L, double* u, const double* f, const double* F,
@@ -653,8 +672,9 @@ void launch_residual64(const Level& L, const double* u, const double* f, const d
 void launch_faces64(const Level& L, const double* a, double* F, double* D, double* inv_d,
                     cudaStream_t st) {
     launch_counter()++;
-    k_faces64<<<nblocks(L.d.cells), kThreads, 0, st>>>(L.d, 0.5 * L.h2i[0], 0.5 * L.h2i[1], 0.5 * L.h2i[2], a, F,
-                                                       D, inv_d);
+    const int ex = ilogb(0.5 * L.h2i[0]), ey = ilogb(0.5 * L.h2i[1]), ez = ilogb(0.5 * L.h2i[2]);
+    auto fn = ex == ey && ey == ez ? k_faces64<true> : k_faces64<false>;
+    fn<<<nblocks(L.d.cells), kThreads, 0, st>>>(L.d, ex, ey, ez, a, F, D, inv_d);
 }
 
 void launch_correct(int cells, double* u, const float* e, cudaStream_t st) {
@@ -664,7 +684,7 @@ void launch_correct(int cells, double* u, const float* e, cudaStream_t st) {
 
 template void launch_rbgs_sweep<float>(const Level&, float*, const float*, const float*, cudaStream_t);
 template void launch_resid_restrict<float>(const Level&, const Level&, const float*, const float*,
-                                           const float*, float*, cudaStream_t);
+                                           const float*, float*, bool, cudaStream_t);
 template void launch_coarse_invert<float>(const Level&, const float*, double*, cudaStream_t);
 template void launch_coarse_invert<double>(const Level&, const double*, double*, cudaStream_t);
 template void launch_coarse_solve<float>(const double*, const float*, float*, cudaStream_t);

@@ -374,7 +374,8 @@ bool vcycle(Handle* H, MG<T>& g, int l, T* u, const T* f, bool zero_u,
     bool streamed = false;
     if constexpr (sizeof(T) == sizeof(float))
         streamed = launch_resid_restrict_stream(L, H->lv[l + 1], cur, f, g.c[l], g.f[l + 1], H->st);
-    if (!streamed) launch_resid_restrict<T>(L, H->lv[l + 1], cur, f, g.c[l], g.f[l + 1], H->st);
+    if (!streamed)
+        launch_resid_restrict<T>(L, H->lv[l + 1], cur, f, g.c[l], g.f[l + 1], H->p.nu1 > 0, H->st);
     vcycle<T>(H, g, l + 1, g.u[l + 1], g.f[l + 1], true);
     int nu2 = H->p.nu2;
     bool folded = false, corrected = false;

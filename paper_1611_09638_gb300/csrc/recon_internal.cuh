@@ -234,10 +234,11 @@ void launch_faces_line(const Level& fine, const Level& coarse, const float* in, 
                        cudaStream_t st);
 // y = (float) x, elementwise
 void launch_to_f32(int cells, const double* x, float* y, cudaStream_t st);
-// full-weighting restriction of the residual f - L u, without storing it
+// full-weighting restriction of the residual f - L u, without storing it;
+// swept: u comes from a red-black sweep, so only red nodes have one
 template <typename T>
 void launch_resid_restrict(const Level& fine, const Level& coarse, const T* u, const T* f,
-                           const T* a, T* out, cudaStream_t st);
+                           const T* a, T* out, bool swept, cudaStream_t st);
 template <typename T>
 void launch_prolong_add(const Level& fine, const Level& coarse, const T* uc, T* u, cudaStream_t st);
 // Coarsest (4x4x4) level: the 64 x 64 matrix of the mean-free solution, once
