@@ -144,8 +144,8 @@ extern "C" int recon_deposit_cic_noalloc(int n0, int n1, int n2, double cell, co
         cudaGetLastError();
         return recon::set_last_error(RECON_E_CUDA, cudaGetErrorString(e));
     }
-    recon::launch_deposit_particles(d, np, pos, mass, 1.0 / cell, scale, S->acc, st);
-    recon::launch_fix_to_double((int)cells, S->acc, 1.0 / scale, rho, st);
+    recon::launch_deposit_particles(d, np, pos, mass, 1.0 / cell, scale, nullptr, nullptr, S->acc, st);
+    recon::launch_fix_to_double((int)cells, S->acc, scale, nullptr, rho, st);
     e = cudaGetLastError();
     if (e != cudaSuccess) return recon::set_last_error(RECON_E_CUDA, cudaGetErrorString(e));
     return RECON_OK;

@@ -1415,6 +1415,7 @@ int recon_create(void** out, const recon_params* p_in, void* cuda_stream) {
     }
     std::memset(H->hctl, 0, sizeof(Ctl));
     cudaError_t e = cudaMemsetAsync(H->mfix, 0, n * sizeof(unsigned long long), H->st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(H->scal, 0, SC_COUNT * sizeof(double), H->st);
     if (e == cudaSuccess && H->replay_d)
         e = cudaMemcpyAsync(H->replay_d, H->replay.data(), H->replay.size() * sizeof(double),
                             cudaMemcpyHostToDevice, H->st);
@@ -1475,31 +1476,34 @@ int recon_deposit(void* hp, int mode, const double* data, const double* mass, in
                 dmass = (const double*)q;
             }
         }
-        launch_validate_particles(np, dpos, dmass, H->part[0], H->part[1], H->st);
-        finish_reduce(H->part[0], 0, H->scal, SC_SUM_RHO, H->st);
-        finish_reduce(H->part[1], 2, H->scal, SC_BAD, H->st);
-        int rc = sync_scalars(H);
-        if (rc == RECON_OK && H->hscal[SC_BAD] != 0.0)
-            rc = fail(RECON_E_NONFINITE, "particle positions or masses are not finite / negative");
-        if (rc == RECON_OK && !(H->hscal[SC_SUM_RHO] > 0.0))
-            rc = fail(RECON_E_INVALID, "total particle mass is zero");
-        if (rc == RECON_OK) {
-            const double scale = fixed_scale(H->hscal[SC_SUM_RHO]);
-            launch_deposit_particles(H->d, np, dpos, dmass, 1.0 / H->h, scale, H->mfix, H->st);
-            launch_fix_to_double(n, H->mfix, 1.0 / scale, H->rho, H->st);
-            launch_validate_grid(n, H->rho, H->part[0], H->part[1], H->st);
+        // The whole deposit is enqueued before the inputs' checks are read back
+        // (every index is masked into the grid, whatever a position holds): with
+        // unit masses the total is known and the deposit checks the positions
+        // itself; with masses their sum and checks come first and set the scale
+        // on the device.
+        const double* total = nullptr;
+        double scale = fixed_scale((double)np);
+        if (dmass) {
+            launch_validate_particles(np, dpos, dmass, H->part[0], H->part[1], H->st);
+            finish_reduces({2, {{H->part[0], 0, SC_MASS}, {H->part[1], 2, SC_BAD_PARTICLE}}}, H->scal, H->st);
+            total = H->scal + SC_MASS;
         }
-        if (rc) {
-            cudaStreamSynchronize(H->st);
-            return rc;
-        }
+        launch_deposit_particles(H->d, np, dpos, dmass, 1.0 / H->h, scale, total,
+                                 dmass ? nullptr : H->scal + SC_BAD_PARTICLE, H->mfix, H->st);
+        launch_fix_validate(n, H->mfix, scale, total, H->rho, H->part[0], H->part[1], H->st);
     } else {
         return fail(RECON_E_INVALID, "unknown deposit mode %d", mode);
     }
-    finish_reduce(H->part[0], 0, H->scal, SC_SUM_RHO, H->st);
-    finish_reduce(H->part[1], 2, H->scal, SC_BAD, H->st);
+    finish_reduces({2, {{H->part[0], 0, SC_SUM_RHO}, {H->part[1], 2, SC_BAD}}}, H->scal, H->st);
     int rc = sync_scalars(H);
     if (rc) return rc;
+    if (mode == RECON_PARTICLES) {
+        if (H->hscal[SC_BAD_PARTICLE] != 0.0) {
+            CK(cudaMemsetAsync(H->scal + SC_BAD_PARTICLE, 0, sizeof(double), H->st));
+            return fail(RECON_E_NONFINITE, "particle positions or masses are not finite / negative");
+        }
+        if (mass && !(H->hscal[SC_MASS] > 0.0)) return fail(RECON_E_INVALID, "total particle mass is zero");
+    }
     if (H->hscal[SC_BAD] != 0.0) return fail(RECON_E_NONFINITE, "density has NaN/Inf or negative values");
     if (!(H->hscal[SC_SUM_RHO] > 0.0)) return fail(RECON_E_INVALID, "total density is zero");
     H->rho_sum = H->hscal[SC_SUM_RHO];

@@ -83,6 +83,8 @@ enum Scalar {
     SC_ADJ_A,         // adjoint sweep: sums used for mean projections
     SC_ADJ_B,
     SC_MAX_DPHI,      // a bound on max |dphi| of the step
+    SC_MASS,          // total mass of the deposited particles
+    SC_BAD_PARTICLE,  // nonzero if a particle was NaN/Inf or negative; 0 between deposits
     SC_PHI_BOUND,     // a bound on max |phi|, grown by every advance
     SC_COUNT
 };
@@ -291,8 +293,14 @@ void launch_validate_grid(int cells, const double* rho, double* partials_sum, do
 void launch_validate_particles(int64_t np, const double* pos, const double* mass,
                                double* partials_sum, double* partials_bad, cudaStream_t st);
 void launch_deposit_particles(const Dims& d, int64_t np, const double* pos, const double* mass,
-                              double inv_h, double scale, unsigned long long* mfix, cudaStream_t st);
-void launch_fix_to_double(int cells, unsigned long long* mfix, double inv_scale, double* out,
+                              double inv_h, double scale, const double* total, double* bad,
+                              unsigned long long* mfix, cudaStream_t st);
+// m = mfix / scale (mfix is cleared), with the sum of m and the checks of
+// launch_validate_grid.  total: the device sum of the masses that sets the
+// scale, or null (then `scale` does).
+void launch_fix_validate(int cells, unsigned long long* mfix, double scale, const double* total, double* out,
+                         double* ps, double* pb, cudaStream_t st);
+void launch_fix_to_double(int cells, unsigned long long* mfix, double scale, const double* total, double* out,
                           cudaStream_t st);
 void launch_init_tracers(int cells, const double* rho, const double* sum_rho, double* w,
                          double* ox, double* oy, double* oz, double* phi, float* phi32,

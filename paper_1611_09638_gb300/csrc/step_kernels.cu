@@ -3,6 +3,7 @@
 // the map x = xi + grad phi, the limited source of Eq. (elliptic), the
 // smoothing operator S, the step limiter, the mesh advance and the outputs.
 #include "checked.cuh"
+#include "fixed_point.cuh"
 #include "geometry.cuh"
 #include "recon_internal.cuh"
 #include "reduce.cuh"
@@ -43,9 +44,11 @@ constexpr int kFracBits = 52;
 
 // The fixed-point position of a tracer along one axis: the offset from its
 // home node rounded to 2^-kFracBits of a cell (|off| < 2^11), as the lower
-// node and the fraction f in [0, 2^kFracBits).
+// node and the fraction f in [0, 2^kFracBits).  Below 2^10 cells the rounding is
+// integer work.
 __device__ inline void fixed_axis(int home, double off, int& i0, unsigned long long& f) {
-    const long long q = __double2ll_rn(off * 4503599627370496.0);  // off 2^52
+    const bool near = ((int)(__double_as_longlong(off) >> 52) & 0x7ff) < 1023 + 10;
+    const long long q = near ? to_fixed(off, kFracBits) : __double2ll_rn(off * 4503599627370496.0);
     i0 = home + (int)(q >> kFracBits);                              // floor
     f = (unsigned long long)q & ((1ull << kFracBits) - 1);
 }
@@ -117,34 +120,100 @@ __global__ void k_validate_particles(int64_t np, const double* __restrict__ pos,
     if (threadIdx.x == 0) pb[blockIdx.x] = bad;
 }
 
-__global__ void k_deposit_particles(Dims d, int64_t np, const double* __restrict__ pos,
-                                    const double* __restrict__ mass, double inv_h, double scale,
-                                    unsigned long long* __restrict__ mfix) {
-    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= np) return;
-    // the position wrapped into [0, n) grid units, then as fixed_axis does
-    // for an offset from node 0 (the same integer charges as the tracers')
-    // (x * inv_pow2(n) is x / n exactly: n is a power of two)
-    auto wrap = [](double x, int n) { return x - (double)n * floor(x * inv_pow2(n)); };
-    CicCharges q;
-    unsigned long long fx, fy, fz;
-    fixed_axis(0, wrap(pos[3 * p] * inv_h, d.n0), q.i0, fx);
-    fixed_axis(0, wrap(pos[3 * p + 1] * inv_h, d.n1), q.j0, fy);
-    fixed_axis(0, wrap(pos[3 * p + 2] * inv_h, d.n2), q.k0, fz);
-    const double m = mass ? mass[p] : 1.0;
-    split_charges((unsigned long long)__double2ll_rn(m * scale), fx, fy, fz, q);
-    for (int di = 0; di < 2; ++di)
-        for (int dj = 0; dj < 2; ++dj)
-            for (int dk = 0; dk < 2; ++dk)
-                atomicAdd(&mfix[cell_index(d, q.i0 + di, q.j0 + dj, q.k0 + dk)], q.c[di][dj][dk]);
+// The scale of the fixed point for a total mass known on the device (total;
+// what fixed_scale gives on the host), or the given one.
+__device__ inline double deposit_scale(const double* __restrict__ total, double scale) {
+    if (!total) return scale;
+    const int e = (int)(__double_as_longlong(*total) >> 52) - 1022;  // total < 2^e
+    return __longlong_as_double((long long)(1023 + 61 - min(max(e, 1), 1000)) << 52);
 }
 
-__global__ void k_fix_to_double(int cells, unsigned long long* __restrict__ mfix, double inv_scale,
-                                double* __restrict__ out) {
+// bad: null, or set to 1 where a position is not finite (unit masses: such a
+// deposit needs no pass over the particles before it).
+__global__ void k_deposit_particles(Dims d, int64_t np, const double* __restrict__ pos,
+                                    const double* __restrict__ mass, double inv_h, double given,
+                                    const double* __restrict__ total, double* __restrict__ bad,
+                                    unsigned long long* __restrict__ mfix) {
+    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (bad) {
+        const bool off = p < np && !(isfinite(pos[3 * p]) && isfinite(pos[3 * p + 1]) && isfinite(pos[3 * p + 2]));
+        if (off) *bad = 1.0;
+    }
+    const double scale = deposit_scale(total, given);
+    // the position as an offset from node 0 (the same integer charges as the
+    // tracers'; cell_index wraps it), first wrapped into [0, n) grid units where
+    // it is 2^10 cells away or more (x * inv_pow2(n) is x / n exactly)
+    auto wrap = [](double x, int n) {
+        return fabs(x) < 1024.0 ? x : x - (double)n * floor(x * inv_pow2(n));
+    };
+    CicCharges q{};
+    if (p < np) {
+        unsigned long long fx, fy, fz;
+        fixed_axis(0, wrap(pos[3 * p] * inv_h, d.n0), q.i0, fx);
+        fixed_axis(0, wrap(pos[3 * p + 1] * inv_h, d.n1), q.j0, fy);
+        fixed_axis(0, wrap(pos[3 * p + 2] * inv_h, d.n2), q.k0, fz);
+        const double m = mass ? mass[p] : 1.0;
+        split_charges((unsigned long long)__double2ll_rn(m * scale), fx, fy, fz, q);
+    }
+    // Two lanes add one particle's pair of cells along k, so that an atomic
+    // instruction of particles in no order touches half as many sectors, which
+    // bound it: 20 million in random order on 256^3 1.43 -> 1.19 ms, one a cell of
+    // 512^3 in order 6.6 -> 3.0 ms (4.2 of that with the FP64 wrap and scalings
+    // left out).
+    const int lane = threadIdx.x & 31, dk = lane & 1;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const int src = (lane >> 1) + 16 * s;
+        const int i0 = __shfl_sync(0xffffffffu, q.i0, src), j0 = __shfl_sync(0xffffffffu, q.j0, src);
+        const int k = __shfl_sync(0xffffffffu, q.k0, src) + dk;
+#pragma unroll
+        for (int di = 0; di < 2; ++di)
+#pragma unroll
+            for (int dj = 0; dj < 2; ++dj) {
+                const unsigned long long a = __shfl_sync(0xffffffffu, q.c[di][dj][0], src);
+                const unsigned long long b = __shfl_sync(0xffffffffu, q.c[di][dj][1], src);
+                const unsigned long long v = dk ? b : a;
+                if (v) atomicAdd(&mfix[cell_index(d, i0 + di, j0 + dj, k)], v);
+            }
+    }
+}
+
+// 1 / 2^n of a power of two by its exponent bits.
+__device__ inline double inv_of_pow2(double x) {
+    return __longlong_as_double((2046ll << 52) - __double_as_longlong(x));
+}
+
+__global__ void k_fix_to_double(int cells, unsigned long long* __restrict__ mfix, double given,
+                                const double* __restrict__ total, double* __restrict__ out) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= cells) return;
+    const double inv_scale = inv_of_pow2(deposit_scale(total, given));
     out[c] = (double)(long long)mfix[c] * inv_scale;
     mfix[c] = 0ull;
+}
+
+// The same with the sum of the density and the checks of k_validate_grid, for
+// grids of at most 2^20 cells: one launch instead of two (64^3: 2.5 us of a 69 us
+// deposit); on larger grids the two passes are faster (256^3: 116 us against
+// 181).
+__global__ void k_fix_validate(int cells, unsigned long long* __restrict__ mfix, double given,
+                               const double* __restrict__ total, double* __restrict__ out, double* ps, double* pb) {
+    double s = 0.0, bad = 0.0;
+    const double inv_scale = inv_of_pow2(deposit_scale(total, given));
+    const int stride = gridDim.x * blockDim.x;
+    auto one = [&](int c, long long q) {
+        const double v = (double)q * inv_scale;
+        mfix[c] = 0ull;
+        out[c] = v;
+        if (q < 0) bad = 1.0;
+        else s += v;
+    };
+    int c = blockIdx.x * blockDim.x + threadIdx.x;
+    for (; c < cells; c += stride) one(c, (long long)mfix[c]);
+    s = block_reduce<OpSum>(s);
+    if (threadIdx.x == 0) ps[blockIdx.x] = s;
+    bad = block_reduce<OpMax>(bad);
+    if (threadIdx.x == 0) pb[blockIdx.x] = bad;
 }
 
 __global__ void k_init_tracers(int cells, const double* __restrict__ rho,
@@ -153,8 +222,11 @@ __global__ void k_init_tracers(int cells, const double* __restrict__ rho,
                                double* __restrict__ oy, double* __restrict__ oz,
                                double* __restrict__ phi, float* __restrict__ phi32) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ double inv;  // (a division in every thread bound this kernel: 512^3 3.54 -> 1.00 ms)
+    if (threadIdx.x == 0) inv = 1.0 / (*sum_rho / (double)cells);
+    __syncthreads();
     if (c >= cells) return;
-    const double inv_rho_bar = 1.0 / (*sum_rho / (double)cells);
+    const double inv_rho_bar = inv;
     w[c] = rho[c] * inv_rho_bar;
     ox[c] = 0.0, oy[c] = 0.0, oz[c] = 0.0;
     phi[c] = 0.0;
@@ -642,17 +714,29 @@ void launch_validate_particles(int64_t np, const double* pos, const double* mass
 }
 
 void launch_deposit_particles(const Dims& d, int64_t np, const double* pos, const double* mass,
-                              double inv_h, double scale, unsigned long long* mfix, cudaStream_t st) {
+                              double inv_h, double scale, const double* total, double* bad,
+                              unsigned long long* mfix, cudaStream_t st) {
     if (np <= 0) return;
     launch_counter()++;
     k_deposit_particles<<<(unsigned)((np + kThreads - 1) / kThreads), kThreads, 0, st>>>(
-        d, np, pos, mass, inv_h, scale, mfix);
+        d, np, pos, mass, inv_h, scale, total, bad, mfix);
 }
 
-void launch_fix_to_double(int cells, unsigned long long* mfix, double inv_scale, double* out,
+void launch_fix_validate(int cells, unsigned long long* mfix, double scale, const double* total, double* out,
+                         double* ps, double* pb, cudaStream_t st) {
+    if (cells > 1 << 20) {
+        launch_fix_to_double(cells, mfix, scale, total, out, st);
+        launch_validate_grid(cells, out, ps, pb, st);
+        return;
+    }
+    launch_counter()++;
+    k_fix_validate<<<kRedBlocks, kRedThreads, 0, st>>>(cells, mfix, scale, total, out, ps, pb);
+}
+
+void launch_fix_to_double(int cells, unsigned long long* mfix, double scale, const double* total, double* out,
                           cudaStream_t st) {
     launch_counter()++;
-    k_fix_to_double<<<nblocks(cells), kThreads, 0, st>>>(cells, mfix, inv_scale, out);
+    k_fix_to_double<<<nblocks(cells), kThreads, 0, st>>>(cells, mfix, scale, total, out);
 }
 
 void launch_init_tracers(int cells, const double* rho, const double* sum_rho, double* w,

@@ -126,3 +126,46 @@ def test_closing_statistics_are_those_of_the_fields(shape):
         assert st.min_det == R.field("det").min().item()
         assert st.min_lambda0 == R.field("lambda0").min().item()
         assert st.max_delta_r == R.field("delta_r").max().item()
+
+
+def test_particle_errors_leave_the_next_deposit_exact():
+    """The deposit is enqueued before its inputs' checks are read back: every
+    rejected catalogue (not finite, negative, without mass) reports its status
+    and leaves the accumulators clear, so that the next deposit on the handle
+    is that of a fresh one, bit for bit, with and without masses."""
+    from paper_1611_09638_gb300 import ReconError, _abi
+
+    n, box, count = 16, 50.0, 3001
+    r = np.random.default_rng(5)
+    pos = torch.from_numpy(r.uniform(-box, 2 * box, (count, 3))).cuda()
+    mass = torch.from_numpy(r.uniform(0.1, 3.0, count)).cuda()
+
+    def with_value(t, value, at):
+        t = t.clone()
+        t.view(-1)[at] = value
+        return t
+
+    with Recon((n, n, n), box=box) as fresh:
+        fresh.deposit_particles(pos)
+        unit = fresh.field("density").clone()
+        fresh.deposit_particles(pos, mass)
+        heavy = fresh.field("density").clone()
+    assert abs(unit.sum().item() - count) <= 1e-9 * count
+    assert abs(heavy.sum().item() - mass.sum().item()) <= 1e-9 * mass.sum().item()
+    cases = [((with_value(pos, float("nan"), 7), None), _abi.RECON_E_NONFINITE),
+             ((with_value(pos, float("inf"), 3 * count - 1), None), _abi.RECON_E_NONFINITE),
+             ((with_value(pos, float("-inf"), 0), mass), _abi.RECON_E_NONFINITE),
+             ((pos, with_value(mass, -1.0, 5)), _abi.RECON_E_NONFINITE),
+             ((pos, with_value(mass, float("nan"), count - 1)), _abi.RECON_E_NONFINITE),
+             ((pos, torch.zeros_like(mass)), _abi.RECON_E_INVALID)]
+    with Recon((n, n, n), box=box) as R:
+        for (p, m), status in cases:
+            with pytest.raises(ReconError) as e:
+                R.deposit_particles(p, m)
+            assert e.value.status == status
+            with pytest.raises(ReconError):
+                R.field("density")
+            R.deposit_particles(pos)
+            assert torch.equal(R.field("density"), unit)
+            R.deposit_particles(pos, mass)
+            assert torch.equal(R.field("density"), heavy)
