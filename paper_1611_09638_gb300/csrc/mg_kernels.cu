@@ -691,161 +691,203 @@ template void launch_coarse_solve<float>(const double*, const float*, float*, cu
 
 }  // namespace recon
 
-// ---------------------------------------------------------------------------
-// The coarse end of the V-cycle in one block: every level from l0 (at most
-// kCoarseMaxCells nodes) down to the 4^3 level is smoothed, restricted, solved
-// and prolonged in shared memory, with the same per-node arithmetic as the
-// kernels above, so a V-cycle launches one kernel for all of these levels.
+// The coarse end of the FP32 V-cycle in one block: every level from l0 (at most
+// 4096 nodes) down to the 4^3 level is smoothed, restricted, solved and prolonged
+// in shared memory, so a V-cycle launches one kernel for all of these levels.
+//
+// Each level's face coefficients and 1 / diagonal are formed once, as it is
+// loaded; a node of a colour phase then takes 14 shared values and no division.
+// Consecutive threads take consecutive k of alternating planes (the parity gives
+// the colour), which fall into distinct banks.  As in coarse_cluster.cu the
+// residual is evaluated at red nodes only after a sweep, and the prolongation
+// added at black nodes only before one.  The spacing factors come as FP32 from
+// the host: an FP64 conversion in each of 1024 threads takes the SM 512 cycles.
+// 32 x 16 x 8 and below: 33.6 -> 24.4 us a V(1, 1).
 
 namespace recon {
 
 namespace {
 
-template <typename T>
-__device__ inline void sm_sweep_colour(const Dims& d, T hx, T hy, T hz, int colour, T* u,
-                                       const T* f, const T* a) {
-    const int half = d.cells >> 1, hs2 = d.s2 - 1;
-    for (int t = threadIdx.x; t < half; t += blockDim.x) {
-        const int kk = t & ((1 << hs2) - 1);
-        const int j = (t >> hs2) & (d.n1 - 1);
-        const int i = t >> (d.s1 + hs2);
-        const int k = 2 * kk + ((i + j + colour) & 1);
-        const int c = cell_index(d, i, j, k);
-        Stencil7<T> s = stencil7<T>(d, hx, hy, hz, i, j, k, c, u, a);
-        u[c] = (s.off - f[c]) / s.diag;
-    }
-}
+constexpr int kVcT = 1024;
 
-template <typename T>
-__device__ inline void sm_sweeps(const Dims& d, T hx, T hy, T hz, int nu, T* u, const T* f,
-                                 const T* a) {
-    for (int s = 0; s < nu; ++s)
-        for (int colour = 0; colour < 2; ++colour) {
-            sm_sweep_colour<T>(d, hx, hy, hz, colour, u, f, a);
+struct CoarseSet32 {
+    int nlev, nu1, nu2;
+    Dims d[kCoarseMaxLevels];
+    int coarsen[kCoarseMaxLevels][3];
+    float w[kCoarseMaxLevels][3];  // h^-2 / 2 per axis
+    const float* a[kCoarseMaxLevels];
+};
+
+__global__ void __launch_bounds__(kVcT) k_coarse_vcycle(const __grid_constant__ CoarseSet32 cs,
+                                                        const float* __restrict__ f_top,
+                                                        float* __restrict__ u_top,
+                                                        const double* __restrict__ minv_g, int zero_u) {
+    extern __shared__ double sm_vc[];
+    double* minv = sm_vc;            // the 4^3 matrix, then its right-hand side in FP64
+    double* f64 = minv + kNc * kNc;
+    float* base = reinterpret_cast<float*>(f64 + kNc);
+    // arrays of level l: gx, gy, gz (the face between a node and its +1
+    // neighbour), 1 / diagonal, u, f, r (a until the faces are formed)
+    auto arrays = [&](int l) {
+        float* q = base;
+        for (int m = 0; m < l; ++m) q += 7 * cs.d[m].cells;
+        return q;
+    };
+    const int t0 = threadIdx.x, last = cs.nlev - 1;
+    for (int e = t0; e < kNc * kNc; e += kVcT) minv[e] = minv_g[e];
+    for (int l = 0; l < last; ++l) {
+        float* r = arrays(l) + 6 * cs.d[l].cells;
+        for (int c = t0; c < cs.d[l].cells; c += kVcT) r[c] = cs.a[l][c];
+    }
+    {
+        const int n = cs.d[0].cells;
+        float *u = arrays(0) + 4 * n, *f = u + n;
+        for (int c = t0; c < n; c += kVcT) {
+            f[c] = f_top[c];
+            u[c] = zero_u ? 0.f : u_top[c];
+        }
+    }
+    __syncthreads();
+    for (int l = 0; l < last; ++l) {
+        const Dims d = cs.d[l];
+        float* g = arrays(l);
+        const float* a = g + 6 * d.cells;
+        for (int c = t0; c < d.cells; c += kVcT) {
+            int i, j, k;
+            cell_coords(d, c, i, j, k);
+            g[c] = cs.w[l][0] * (a[c] + a[cell_index(d, i + 1, j, k)]);
+            g[d.cells + c] = cs.w[l][1] * (a[c] + a[cell_index(d, i, j + 1, k)]);
+            g[2 * d.cells + c] = cs.w[l][2] * (a[c] + a[cell_index(d, i, j, k + 1)]);
+        }
+    }
+    __syncthreads();
+    auto diag = [&](const Dims& d, const float* g, int i, int j, int k, int c) {
+        return (g[c] + g[cell_index(d, i - 1, j, k)]) +
+               (g[d.cells + c] + g[d.cells + cell_index(d, i, j - 1, k)]) +
+               (g[2 * d.cells + c] + g[2 * d.cells + cell_index(d, i, j, k - 1)]);
+    };
+    for (int l = 0; l < last; ++l) {
+        const Dims d = cs.d[l];
+        float* g = arrays(l);
+        for (int c = t0; c < d.cells; c += kVcT) {
+            int i, j, k;
+            cell_coords(d, c, i, j, k);
+            g[3 * d.cells + c] = 1.f / diag(d, g, i, j, k, c);
+        }
+    }
+    __syncthreads();
+    auto off = [&](const Dims& d, const float* g, const float* u, int i, int j, int k, int c) {
+        const int xm = cell_index(d, i - 1, j, k), ym = cell_index(d, i, j - 1, k), zm = cell_index(d, i, j, k - 1);
+        return (g[c] * u[cell_index(d, i + 1, j, k)] + g[xm] * u[xm]) +
+               (g[d.cells + c] * u[cell_index(d, i, j + 1, k)] + g[d.cells + ym] * u[ym]) +
+               (g[2 * d.cells + c] * u[cell_index(d, i, j, k + 1)] + g[2 * d.cells + zm] * u[zm]);
+    };
+    // the t-th node of a colour
+    auto node = [&](const Dims& d, int t, int colour, int& i, int& j, int& k) {
+        k = t & (d.n2 - 1), j = (t >> d.s2) & (d.n1 - 1);
+        i = 2 * (t >> (d.s1 + d.s2)) + ((j + k + colour) & 1);
+        return cell_index(d, i, j, k);
+    };
+    auto sweeps = [&](int l, int nu, bool zero) {
+        const Dims d = cs.d[l];
+        float *g = arrays(l), *u = g + 4 * d.cells;
+        const float *rd = g + 3 * d.cells, *f = u + d.cells;
+        for (int s = 0; s < 2 * nu; ++s) {
+            for (int t = t0; t < d.cells >> 1; t += kVcT) {
+                int i, j, k;
+                const int c = node(d, t, s & 1, i, j, k);
+                u[c] = ((zero && s == 0 ? 0.f : off(d, g, u, i, j, k, c)) - f[c]) * rd[c];
+            }
             __syncthreads();
         }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(1024) k_coarse_vcycle(CoarseSet cs, const T* __restrict__ f_top,
-                                                        T* __restrict__ u_top,
-                                                        const double* __restrict__ minv_g,
-                                                        int zero_u) {
-    extern __shared__ unsigned char smem_raw[];
-    T* base = reinterpret_cast<T*>(smem_raw);
-    T *u[kCoarseMaxLevels], *f[kCoarseMaxLevels], *a[kCoarseMaxLevels], *r[kCoarseMaxLevels];
-    {
-        T* q = base;
-        for (int l = 0; l < cs.nlev; ++l) {
-            const int n = cs.lv[l].d.cells;
-            u[l] = q, f[l] = q + n, a[l] = q + 2 * n, r[l] = q + 3 * n;
-            q += 4 * n;
-        }
-    }
-    for (int l = 0; l < cs.nlev; ++l) {
-        const T* ag = reinterpret_cast<const T*>(cs.a[l]);
-        for (int c = threadIdx.x; c < cs.lv[l].d.cells; c += blockDim.x) a[l][c] = ag[c];
-    }
-    for (int c = threadIdx.x; c < cs.lv[0].d.cells; c += blockDim.x) {
-        f[0][c] = f_top[c];
-        u[0][c] = zero_u ? T(0) : u_top[c];
-    }
-    // the 4^3 inverse in shared memory, after the levels (8-byte aligned: 4 arrays of whole levels)
-    double* minv = reinterpret_cast<double*>(u[cs.nlev - 1] + 4 * cs.lv[cs.nlev - 1].d.cells);
-    for (int e = threadIdx.x; e < kNc * kNc; e += blockDim.x) minv[e] = minv_g[e];
-    __syncthreads();
-    const int last = cs.nlev - 1;
-    // down
+    };
     for (int l = 0; l < last; ++l) {
-        const Level& L = cs.lv[l];
-        const T hx = (T)L.h2i[0], hy = (T)L.h2i[1], hz = (T)L.h2i[2];
-        sm_sweeps<T>(L.d, hx, hy, hz, cs.nu1, u[l], f[l], a[l]);
-        for (int c = threadIdx.x; c < L.d.cells; c += blockDim.x) {
-            int i, j, k;
-            cell_coords(L.d, c, i, j, k);
-            Stencil7<T> s = stencil7<T>(L.d, hx, hy, hz, i, j, k, c, u[l], a[l]);
-            r[l][c] = f[l][c] - (s.off - s.diag * u[l][c]);
-        }
+        const Dims d = cs.d[l], dc = cs.d[l + 1];
+        float *g = arrays(l), *u = g + 4 * d.cells, *r = g + 6 * d.cells;
+        const float* f = g + 5 * d.cells;
+        sweeps(l, cs.nu1, l > 0 || zero_u);
+        for (int colour = cs.nu1 ? 0 : 1; colour >= 0; --colour)
+            for (int t = t0; t < d.cells >> 1; t += kVcT) {
+                int i, j, k;
+                const int c = node(d, t, colour, i, j, k);
+                r[c] = f[c] - (off(d, g, u, i, j, k, c) - diag(d, g, i, j, k, c) * u[c]);
+            }
         __syncthreads();
-        const Dims& dc = cs.lv[l + 1].d;
-        const int cx = L.coarsen[0], cy = L.coarsen[1], cz = L.coarsen[2];
-        for (int c = threadIdx.x; c < dc.cells; c += blockDim.x) {
+        const int cx = cs.coarsen[l][0], cy = cs.coarsen[l][1], cz = cs.coarsen[l][2];
+        float* gc = arrays(l + 1);
+        for (int c = t0; c < dc.cells; c += kVcT) {
             int I, J, K;
             cell_coords(dc, c, I, J, K);
             const int fi = cx ? 2 * I : I, fj = cy ? 2 * J : J, fk = cz ? 2 * K : K;
-            T acc = T(0);
-            for (int oi = -cx; oi <= cx; ++oi) {
-                const T wi = cx ? (oi == 0 ? T(0.5) : T(0.25)) : T(1);
+            float acc = 0.f;
+            for (int oi = -cx; oi <= cx; ++oi)
                 for (int oj = -cy; oj <= cy; ++oj) {
-                    const T wj = cy ? (oj == 0 ? T(0.5) : T(0.25)) : T(1);
+                    const float wij = (cx ? (oi ? 0.25f : 0.5f) : 1.f) * (cy ? (oj ? 0.25f : 0.5f) : 1.f);
                     for (int ok = -cz; ok <= cz; ++ok) {
-                        const T wk = cz ? (ok == 0 ? T(0.5) : T(0.25)) : T(1);
-                        acc += wi * wj * wk * r[l][cell_index(L.d, fi + oi, fj + oj, fk + ok)];
+                        if (cs.nu1 && ((fi + oi + fj + oj + fk + ok) & 1)) continue;  // black: none
+                        acc += wij * (cz ? (ok ? 0.25f : 0.5f) : 1.f) * r[cell_index(d, fi + oi, fj + oj, fk + ok)];
                     }
                 }
-            }
-            f[l + 1][c] = acc;
-            u[l + 1][c] = T(0);
+            if (l + 1 == last) f64[c] = (double)acc;
+            else gc[5 * dc.cells + c] = acc;
+            gc[4 * dc.cells + c] = 0.f;
         }
         __syncthreads();
     }
-    // coarsest: u = M^-1 [f; 0]
-    if (threadIdx.x < kNc) {
+    if (t0 < 4 * kNc) {  // 4^3: u = M f in FP64, four threads a row
         double acc = 0.0;
-        for (int c = 0; c < kNc; ++c) acc += minv[threadIdx.x * kNc + c] * (double)f[last][c];
-        u[last][threadIdx.x] = (T)acc;
+        for (int c = t0 & 3; c < kNc; c += 4) acc = fma(minv[(t0 >> 2) * kNc + c], f64[c], acc);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        if ((t0 & 3) == 0) arrays(last)[4 * kNc + (t0 >> 2)] = (float)acc;
     }
     __syncthreads();
-    // up
     for (int l = last - 1; l >= 0; --l) {
-        const Level& L = cs.lv[l];
-        const Dims& dc = cs.lv[l + 1].d;
-        const int cx = L.coarsen[0], cy = L.coarsen[1], cz = L.coarsen[2];
-        for (int c = threadIdx.x; c < L.d.cells; c += blockDim.x) {
-            int i, j, k;
-            cell_coords(L.d, c, i, j, k);
-            int ii[2], jj[2], kk[2];
-            T wi[2], wj[2], wk[2];
-            int ni, nj, nk;
-            if (!cx) { ii[0] = i; wi[0] = T(1); ni = 1; }
-            else if (!(i & 1)) { ii[0] = i >> 1; wi[0] = T(1); ni = 1; }
-            else { ii[0] = i >> 1; ii[1] = (i >> 1) + 1; wi[0] = wi[1] = T(0.5); ni = 2; }
-            if (!cy) { jj[0] = j; wj[0] = T(1); nj = 1; }
-            else if (!(j & 1)) { jj[0] = j >> 1; wj[0] = T(1); nj = 1; }
-            else { jj[0] = j >> 1; jj[1] = (j >> 1) + 1; wj[0] = wj[1] = T(0.5); nj = 2; }
-            if (!cz) { kk[0] = k; wk[0] = T(1); nk = 1; }
-            else if (!(k & 1)) { kk[0] = k >> 1; wk[0] = T(1); nk = 1; }
-            else { kk[0] = k >> 1; kk[1] = (k >> 1) + 1; wk[0] = wk[1] = T(0.5); nk = 2; }
-            T acc = T(0);
-            for (int p = 0; p < ni; ++p)
-                for (int q = 0; q < nj; ++q)
-                    for (int rr = 0; rr < nk; ++rr)
-                        acc += wi[p] * wj[q] * wk[rr] * u[l + 1][cell_index(dc, ii[p], jj[q], kk[rr])];
-            u[l][c] += acc;
-        }
+        const Dims d = cs.d[l], dc = cs.d[l + 1];
+        float* u = arrays(l) + 4 * d.cells;
+        const float* uc = arrays(l + 1) + 4 * dc.cells;
+        const int cx = cs.coarsen[l][0], cy = cs.coarsen[l][1], cz = cs.coarsen[l][2];
+        for (int colour = cs.nu2 ? 1 : 0; colour < 2; ++colour)
+            for (int t = t0; t < d.cells >> 1; t += kVcT) {
+                int i, j, k;
+                const int c = node(d, t, colour, i, j, k);
+                const int oi = cx & i, oj = cy & j, ok = cz & k;  // odd along a coarsened axis
+                const int I = cx ? i >> 1 : i, J = cy ? j >> 1 : j, K = cz ? k >> 1 : k;
+                // the two values of each axis, equal ones where it is even
+                auto row = [&](int II, int JJ) { return uc[cell_index(dc, II, JJ, K)] + uc[cell_index(dc, II, JJ, K + ok)]; };
+                u[c] += 0.125f * ((row(I, J) + row(I, J + oj)) + (row(I + oi, J) + row(I + oi, J + oj)));
+            }
         __syncthreads();
-        sm_sweeps<T>(L.d, (T)L.h2i[0], (T)L.h2i[1], (T)L.h2i[2], cs.nu2, u[l], f[l], a[l]);
+        sweeps(l, cs.nu2, false);
     }
-    for (int c = threadIdx.x; c < cs.lv[0].d.cells; c += blockDim.x) u_top[c] = u[0][c];
+    const float* u = arrays(0) + 4 * cs.d[0].cells;
+    for (int c = t0; c < cs.d[0].cells; c += kVcT) u_top[c] = u[c];
 }
 
 }  // namespace
 
-template <typename T>
-bool launch_coarse_vcycle(const CoarseSet& cs, const T* f_top, T* u_top, const double* minv,
+size_t coarse_vcycle_smem(size_t cells) {
+    return 7 * cells * sizeof(float) + (kNc + 1) * kNc * sizeof(double);
+}
+
+bool launch_coarse_vcycle(const CoarseSet& cs, const float* f_top, float* u_top, const double* minv,
                           bool zero_u, cudaStream_t st) {
     size_t cells = 0;
     for (int l = 0; l < cs.nlev; ++l) cells += cs.lv[l].d.cells;
-    const size_t sm = 4 * cells * sizeof(T) + kNc * kNc * sizeof(double);
+    const size_t sm = coarse_vcycle_smem(cells);
     if (cs.nlev < 1 || cs.nlev > kCoarseMaxLevels || sm > kCoarseMaxSmem) return false;
-    allow_smem((const void*)k_coarse_vcycle<T>, (int)kCoarseMaxSmem);
+    CoarseSet32 s{};
+    s.nlev = cs.nlev, s.nu1 = cs.nu1, s.nu2 = cs.nu2;
+    for (int l = 0; l < cs.nlev; ++l) {
+        s.d[l] = cs.lv[l].d, s.a[l] = (const float*)cs.a[l];
+        for (int x = 0; x < 3; ++x) s.coarsen[l][x] = cs.lv[l].coarsen[x], s.w[l][x] = (float)(0.5 * cs.lv[l].h2i[x]);
+    }
+    allow_smem((const void*)k_coarse_vcycle, (int)kCoarseMaxSmem);
     launch_counter()++;
-    k_coarse_vcycle<T><<<1, 1024, sm, st>>>(cs, f_top, u_top, minv, zero_u ? 1 : 0);
+    k_coarse_vcycle<<<1, kVcT, sm, st>>>(s, f_top, u_top, minv, zero_u ? 1 : 0);
     return true;
 }
 
-template bool launch_coarse_vcycle<float>(const CoarseSet&, const float*, float*, const double*,
-                                          bool, cudaStream_t);
 // The same for FP64 levels (at most kCoarse64Cells nodes on the first), from
 // their stored faces and diagonals: 8 FP64 instructions a node and colour.
 // One block holds a level of 8^3 nodes (a node a thread and phase); above

@@ -363,7 +363,7 @@ bool vcycle(Handle* H, MG<T>& g, int l, T* u, const T* f, bool zero_u,
     const int last = (int)H->lv.size() - 1;
     const Level& L = H->lv[l];
     if (l == H->lc && launch_coarse_cluster(H->cc, f, u, H->minv, zero_u, 1, H->st)) return false;
-    if (l == H->l0 && launch_coarse_vcycle<T>(H->cs, f, u, H->minv, zero_u, H->st)) return false;
+    if (l == H->l0 && launch_coarse_vcycle(H->cs, f, u, H->minv, zero_u, H->st)) return false;
     if (l == last) {
         launch_coarse_solve<T>(H->minv, f, u, H->st);
         return false;
@@ -1366,12 +1366,15 @@ int recon_create(void** out, const recon_params* p_in, void* cuda_stream) {
     }
     // the levels from the first one of at most 16^3 nodes (8^3 in FP64) down
     // run in one block
-    for (int l = 0; l < nl; ++l)
+    for (int l = 0; l < nl; ++l) {
+        size_t below = 0;
+        for (int q = l; q < nl; ++q) below += H->lv[q].d.cells;
         if (H->lv[l].d.cells <= (H->mixed ? 4096 : kCoarse64Cells) && nl - l <= kCoarseMaxLevels &&
-            !H->lv[l].face) {
+            (!H->mixed || coarse_vcycle_smem(below) <= kCoarseMaxSmem) && !H->lv[l].face) {
             H->l0 = l;
             break;
         }
+    }
     // a 32^3 level with 16^3, 8^3 and 4^3 below it runs in one cluster launch
     if (H->mixed && nl >= 4) {
         CoarseSet& cc = H->cc;

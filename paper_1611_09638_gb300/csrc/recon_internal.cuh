@@ -263,8 +263,10 @@ void launch_coarse_vcycle64(const CoarseSet64& cs, const double* f_top, double* 
 // V-cycle of the FP32 levels in cs in one block: L u = f on the first of them,
 // u updated in place (zero_u: u = 0 on entry, not read); returns false,
 // launching nothing, if they do not fit.
-template <typename T>
-bool launch_coarse_vcycle(const CoarseSet& cs, const T* f_top, T* u_top, const double* minv,
+// Shared memory of that block for levels of `cells` nodes in all; at most
+// kCoarseMaxSmem.
+size_t coarse_vcycle_smem(size_t cells);
+bool launch_coarse_vcycle(const CoarseSet& cs, const float* f_top, float* u_top, const double* minv,
                           bool zero_u, cudaStream_t st);
 // An FP64 level: face coefficients F (3 x cells: A = h^-2 (a_c + a_{c+e}) / 2
 // for the +x, +y, +z face of each node), the node diagonal D = sum of its six

@@ -41,6 +41,21 @@ def test_coarse_levels_match_the_oracle(shape, precision):
 
 
 @pytest.mark.parametrize("nu", [(1, 1), (2, 1), (0, 2), (2, 0)])
+@pytest.mark.parametrize("shape", [(32, 16, 8), (64, 32, 16)])
+def test_single_block_schedules_match_the_oracle(shape, nu):
+    """The coarse levels of anisotropic grids in one block, alone and below
+    other levels, under every form of the schedule."""
+    rho = _rough(shape, 11 * sum(shape))
+    ref = O.solve(O.OracleParams(n=shape, k_max=1), rho)
+    with Recon(shape, precision="mixed", k_max=1, replay_alpha=ref.alpha, nu1=nu[0], nu2=nu[1]) as R:
+        R.deposit_grid(torch.from_numpy(rho).cuda())
+        st = R.solve()
+        phi = R.field("phi").cpu().numpy()
+    assert st.steps == 1 and st.relres[0] <= 1e-8
+    assert np.linalg.norm(phi - ref.phi) <= BARS["mixed"] * np.linalg.norm(ref.phi)
+
+
+@pytest.mark.parametrize("nu", [(1, 1), (2, 1), (0, 2), (2, 0)])
 @pytest.mark.parametrize("n,faces", [(32, 0), (64, 0), (64, 1)])
 def test_cluster_schedules_match_the_oracle(n, faces, nu):
     """The cluster's V-cycle under every form of its schedule (no sweep before
