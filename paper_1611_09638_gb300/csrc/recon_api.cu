@@ -1191,7 +1191,6 @@ static int bounds_status() {
     int id = bounds_fail_smoother();
     if (!id) id = bounds_fail_transfer();
     if (!id) id = bounds_fail_cluster();
-    if (!id) id = bounds_fail_steps();
     if (id) return fail(RECON_E_CUDA, "index bounds check %d failed (RECON_CHECKED build)", id);
     return RECON_OK;
 }
