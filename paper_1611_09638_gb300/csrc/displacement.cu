@@ -18,7 +18,7 @@
 // 0.42 cells) the error is 0.291 units of 2^-53 cells rms and 0.78 at most, that
 // of the FP64 form 0.321 and 1.97 (rounding to the unit alone: 0.289).
 //
-// A block streams planes along i over an 8 x 32 tile; a thread keeps its
+// A block streams planes along i over an 8 x 32 (or 16 x 16) tile; a thread keeps its
 // column's sums of the last planes in registers, so that a plane's 340 nodes
 // are converted once and read back from shared memory 14 times a thread.
 // Bound by instruction issue: 512^3 10.06 -> 3.32 ms; it reads 16 and writes
@@ -34,8 +34,7 @@ namespace {
 constexpr int kDispBits = 53;
 constexpr long long kDispMax = 1ll << (kDispBits + 7);  // 128 cells
 
-constexpr int DJ = 8, DK = 32, DPJ = DJ + 2, DPK = DK + 2;  // tile, and with its ring
-constexpr int DN = DPJ * DPK;
+constexpr int DT = 256;  // nodes of a tile, DK of them along k
 constexpr int DPERSM = 3, DBLOCKS = DPERSM * (kRedBlocks / 8);
 
 // alpha V at one node in FP64, rounded to fixed point; values beyond kDispMax
@@ -163,9 +162,12 @@ __device__ __forceinline__ bool solve_fixed(const DispScales& sc, const long lon
     return err < 7e-18f;
 }
 
-__global__ void __launch_bounds__(DJ* DK, DPERSM) k_displacement_stream(
+template <int DK>
+__global__ void __launch_bounds__(DT, DPERSM) k_displacement_stream(
     Dims d, const double* __restrict__ scal, const double* __restrict__ phi, const double* __restrict__ dphi,
     long long* __restrict__ dx, long long* __restrict__ dy, long long* __restrict__ dz) {
+    constexpr int DJ = DT / DK, DPK = DK + 2, DN = (DJ + 2) * DPK;  // rows, and with the ring
+    static_assert(DN <= 2 * DT, "two values a thread and field");
     __shared__ long long sp[2][DN], sd[2][DN];
     const DispScales sc = disp_scales(scal);
     const double alpha = scal[SC_ALPHA];
@@ -187,7 +189,7 @@ __global__ void __launch_bounds__(DJ* DK, DPERSM) k_displacement_stream(
         return;
     }
     // this thread's nodes of a plane with its ring
-    const int e1 = t + DJ * DK;
+    const int e1 = t + DT;
     const bool two = e1 < DN;
     while (at < end) {
         const int col = (int)(at / d.n0), i0 = (int)(at % d.n0);
@@ -252,8 +254,12 @@ __global__ void k_displacement_node(Dims d, const double* __restrict__ scal, con
 void launch_node_displacement(const Dims& d, const double* scal, const double* phi, const double* dphi,
                               long long* dx, long long* dy, long long* dz, cudaStream_t st) {
     launch_counter()++;
-    if (d.n2 % DK == 0 && d.n1 % DJ == 0) {
-        k_displacement_stream<<<DBLOCKS, DJ * DK, 0, st>>>(d, scal, phi, dphi, dx, dy, dz);
+    if (d.n2 % 32 == 0 && d.n1 % 8 == 0) {
+        k_displacement_stream<32><<<DBLOCKS, DT, 0, st>>>(d, scal, phi, dphi, dx, dy, dz);
+        return;
+    }
+    if (d.n2 % 16 == 0 && d.n1 % 16 == 0) {
+        k_displacement_stream<16><<<DBLOCKS, DT, 0, st>>>(d, scal, phi, dphi, dx, dy, dz);
         return;
     }
     k_displacement_node<<<(d.cells + 255) / 256, 256, 0, st>>>(d, scal, phi, dphi, dx, dy, dz);

@@ -5,7 +5,7 @@
 // values with a bound on their error settle the question, and the result is
 // the FP64 one.
 //
-// Both stream planes of an 8 x 32 tile along i: a plane's FP32 values (with a
+// Both stream planes of an 8 x 32 (or 16 x 16) tile along i: a plane's FP32 values (with a
 // one-node ring) go through shared memory once, and a thread keeps its
 // column's sums of the last two planes in registers.  A node that FP32 does not
 // settle is put on its warp's list, and a full list of 32 runs the FP64 form
@@ -24,7 +24,13 @@ namespace recon {
 
 namespace {
 
-constexpr int GJ = 8, GK = 32, GPK = GK + 2, GN = (GJ + 2) * GPK;
+// A tile of 256 nodes of the (j, k) plane, GK of them along k (32, or 16 on
+// grids whose last axis is no multiple of 32), and with its one-node ring.
+constexpr int GT = 256;
+template <int GK>
+struct Tile {
+    static constexpr int J = GT / GK, PK = GK + 2, N = (J + 2) * PK;
+};
 constexpr int GPERSM = 3, GBLOCKS = GPERSM * (kRedBlocks / 8);
 constexpr float kU = 5.96046448e-8f;  // 2^-24
 
@@ -42,6 +48,7 @@ struct Hess32 {
 // Hessian at the node one plane back.  An entry combines at most four stencil
 // values of magnitude <= vmax; the FP32 copies and at most four operations
 // each round by 2^-24 relative, so 32 u vmax bounds its error with room.
+template <int GPK>
 struct Column32 {
     float ca, cb, ja, jb, ka, kb, va, vb, syb, szb, yzb, gyb, gzb, gx;
     // f: the node in the plane (its ring around it); gives the Hessian and
@@ -90,15 +97,17 @@ __device__ __forceinline__ int sylvester32(float xx, float yy, float zz, float x
 // every plane from the one before a piece to the one after it, with the
 // piece's first plane and column origin, from NF fields staged in shared
 // memory.
-template <int NF, typename Begin, typename Plane>
+template <int GK, int NF, typename Begin, typename Plane>
 __device__ __forceinline__ void stream_planes(const Dims& d, const float* const (&field)[NF],
-                                              float (&buf)[2][NF][GN], Begin&& begin, Plane&& plane) {
+                                              float (&buf)[2][NF][Tile<GK>::N], Begin&& begin, Plane&& plane) {
+    constexpr int GJ = Tile<GK>::J, GPK = Tile<GK>::PK, GN = Tile<GK>::N;
+    static_assert(GN <= 2 * GT, "two values a thread and field");
     const int t = threadIdx.x;
     const int tiles_k = d.n2 / GK;
     const long long planes = (long long)tiles_k * (d.n1 / GJ) * d.n0;
     long long at = planes * blockIdx.x / gridDim.x;
     const long long end = planes * (blockIdx.x + 1) / gridDim.x;
-    const int e1 = t + GJ * GK;
+    const int e1 = t + GT;
     const bool two = e1 < GN;
     while (at < end) {
         const int col = (int)(at / d.n0), i0 = (int)(at % d.n0);
@@ -180,19 +189,21 @@ __device__ __noinline__ double source64(const Dims& d, const SourceParams& sp, c
 // C = E = 0 where FP32 certifies that every eigenvalue of e exceeds xi_m
 // (Sylvester's criterion) and, e being positive definite then, that its trace
 // stays below 3 v_m^(1/3) (det e <= (tr e / 3)^3).
-__global__ void __launch_bounds__(GJ* GK, GPERSM) k_source_stream(Dims d, SourceParams sp, float trace_max,
+template <int GK>
+__global__ void __launch_bounds__(GT, GPERSM) k_source_stream(Dims d, SourceParams sp, float trace_max,
                                                                   const double* __restrict__ phi,
                                                                   const float* __restrict__ phi32,
                                                                   const double* __restrict__ m,
                                                                   double* __restrict__ t,
                                                                   double* __restrict__ psum) {
-    __shared__ float buf[2][1][GN];
-    __shared__ int list[GJ][64];
+    constexpr int GPK = Tile<GK>::PK;
+    __shared__ float buf[2][1][Tile<GK>::N];
+    __shared__ int list[GT / 32][64];
     const int lj = threadIdx.x / GK, lk = threadIdx.x % GK;
     const int own = (lj + 1) * GPK + lk + 1;
     const float xi = (float)sp.xi_m * (1.f + 4.f * kU);  // not below xi_m
-    WarpList todo{list[lj], 0};
-    Column32 col{};
+    WarpList todo{list[threadIdx.x / 32], 0};
+    Column32<GPK> col{};
     double s = 0.0;
     auto exact = [&] {
         const int c = todo.take();
@@ -203,8 +214,8 @@ __global__ void __launch_bounds__(GJ* GK, GPERSM) k_source_stream(Dims d, Source
         }
     };
     const float* const fields[1] = {phi32};
-    stream_planes<1>(
-        d, fields, buf, [&] { col = Column32{}; },
+    stream_planes<GK, 1>(
+        d, fields, buf, [&] { col = Column32<GPK>{}; },
         [&](int p, bool done, int j0, int k0, int w) {
             float gy, gz;
             const int c = done ? cell_index(d, p - 1, j0 + lj, k0 + lk) : 0;
@@ -276,20 +287,22 @@ __device__ inline double gradient64(const Dims& d, const double* __restrict__ dp
 // verdict on the way is open (then the FP64 form does).  The gradient's maximum is FP64 too: a node
 // is evaluated only where FP32 does not show it to be below the largest value
 // its warp has found.
-__global__ void __launch_bounds__(GJ* GK, GPERSM) k_limiter_stream(Dims d, LimiterParams lp,
+template <int GK>
+__global__ void __launch_bounds__(GT, GPERSM) k_limiter_stream(Dims d, LimiterParams lp,
                                                                    const double* __restrict__ phi,
                                                                    const double* __restrict__ dphi,
                                                                    const float* __restrict__ phi32,
                                                                    const float* __restrict__ dphi32,
                                                                    double* __restrict__ pk,
                                                                    double* __restrict__ pg) {
-    __shared__ float buf[2][2][GN];
-    __shared__ int list[GJ][64];
+    constexpr int GPK = Tile<GK>::PK;
+    __shared__ float buf[2][2][Tile<GK>::N];
+    __shared__ int list[GT / 32][64];
     const int lj = threadIdx.x / GK, lk = threadIdx.x % GK;
     const int own = (lj + 1) * GPK + lk + 1;
     const float floor32 = (float)lp.lambda_floor;
-    WarpList todo{list[lj], 0};
-    Column32 A{}, B{};
+    WarpList todo{list[threadIdx.x / 32], 0};
+    Column32<GPK> A{}, B{};
     int kk = 0;            // the warp's largest k so far, and 2^-kk
     float al = 1.f;
     double gm = 0.0;       // this lane's largest |2 G|
@@ -301,8 +314,8 @@ __global__ void __launch_bounds__(GJ* GK, GPERSM) k_limiter_stream(Dims d, Limit
         al = kk < 126 ? __int_as_float((127 - kk) << 23) : 0.f;
     };
     const float* const fields[2] = {phi32, dphi32};
-    stream_planes<2>(
-        d, fields, buf, [&] { A = Column32{}, B = Column32{}; },
+    stream_planes<GK, 2>(
+        d, fields, buf, [&] { A = Column32<GPK>{}, B = Column32<GPK>{}; },
         [&](int p, bool done, int j0, int k0, int w) {
             float gy, gz, ay, az;
             const Hess32 a = A.feed(buf[w][0] + own, ay, az);
@@ -439,24 +452,25 @@ __global__ void k_geometry_out(Dims d, const double* __restrict__ phi, double* _
 // the rounding of the determinant that it is taken from, is covered by 2^-8 p.
 // 512^3: 26 -> 2.0 ms for all three (FP64 at every node, 23 of them for det and
 // lambda0).
-template <bool EXACT>
-__global__ void __launch_bounds__(GJ* GK, GPERSM) k_extrema_stream(Dims d, const double* __restrict__ phi,
+template <int GK, bool EXACT>
+__global__ void __launch_bounds__(GT, GPERSM) k_extrema_stream(Dims d, const double* __restrict__ phi,
                                                                    const float* __restrict__ phi32,
                                                                    const double* __restrict__ bounds,
                                                                    double* __restrict__ pdet,
                                                                    double* __restrict__ plam,
                                                                    double* __restrict__ pdr) {
-    __shared__ float buf[2][1][GN];
+    constexpr int GPK = Tile<GK>::PK;
+    __shared__ float buf[2][1][Tile<GK>::N];
     const int lj = threadIdx.x / GK, lk = threadIdx.x % GK;
     const int own = (lj + 1) * GPK + lk + 1;
     const float bd = EXACT ? __double2float_ru(bounds[0]) : 0.f, bl = EXACT ? __double2float_ru(bounds[1]) : 0.f,
                 br = EXACT ? __double2float_rd(bounds[2]) : 0.f;
-    Column32 col{};
+    Column32<GPK> col{};
     float fd = INFINITY, fl = INFINITY, fr = -INFINITY;
     double md = INFINITY, ml = INFINITY, mr = -INFINITY;
     const float* const fields[1] = {phi32};
-    stream_planes<1>(
-        d, fields, buf, [&] { col = Column32{}; },
+    stream_planes<GK, 1>(
+        d, fields, buf, [&] { col = Column32<GPK>{}; },
         [&](int p, bool done, int j0, int k0, int w) {
             float gy, gz;
             const Hess32 h = col.feed(buf[w][0] + own, gy, gz);
@@ -513,16 +527,20 @@ __global__ void k_triad(Dims d, const double* __restrict__ phi, double* __restri
     e6[3 * n + c] = e.xy, e6[4 * n + c] = e.xz, e6[5 * n + c] = e.yz;
 }
 
-bool tiles(const Dims& d) { return d.n2 % GK == 0 && d.n1 % GJ == 0; }
+// The tile's nodes along k on this grid (0: none fits).
+int tile_k(const Dims& d) {
+    return d.n2 % 32 == 0 && d.n1 % 8 == 0 ? 32 : d.n2 % 16 == 0 && d.n1 % 16 == 0 ? 16 : 0;
+}
 
 }  // namespace
 
 void launch_source(const Dims& d, const SourceParams& sp, const double* phi, const float* phi32, const double* m,
                    double* t, double* part_sum, cudaStream_t st) {
     launch_counter()++;
-    if (tiles(d)) {
+    if (const int tk = tile_k(d)) {
         const float trace_max = (float)(3.0 * cbrt(sp.v_m) * (1.0 - 1e-5));
-        k_source_stream<<<GBLOCKS, GJ * GK, 0, st>>>(d, sp, trace_max, phi, phi32, m, t, part_sum);
+        auto fn = tk == 32 ? k_source_stream<32> : k_source_stream<16>;
+        fn<<<GBLOCKS, GT, 0, st>>>(d, sp, trace_max, phi, phi32, m, t, part_sum);
         return;
     }
     k_source_node<<<kRedBlocks, kRedThreads, 0, st>>>(d, sp, phi, m, t, part_sum);
@@ -532,8 +550,9 @@ void launch_limiter(const Dims& d, const LimiterParams& lp, const double* phi, c
                     const float* phi32, const float* dphi32, double* part_k, double* part_g,
                     cudaStream_t st) {
     launch_counter()++;
-    if (tiles(d)) {
-        k_limiter_stream<<<GBLOCKS, GJ * GK, 0, st>>>(d, lp, phi, dphi, phi32, dphi32, part_k, part_g);
+    if (const int tk = tile_k(d)) {
+        auto fn = tk == 32 ? k_limiter_stream<32> : k_limiter_stream<16>;
+        fn<<<GBLOCKS, GT, 0, st>>>(d, lp, phi, dphi, phi32, dphi32, part_k, part_g);
         return;
     }
     k_limiter_node<<<kRedBlocks, kRedThreads, 0, st>>>(d, lp, phi, dphi, part_k, part_g);
@@ -554,19 +573,22 @@ void launch_geometry_out(const Dims& d, const double* phi, double* det, double* 
 int launch_extrema(const Dims& d, const double* phi, const float* phi32, double* scratch, double* part_det,
                    double* part_lam, double* part_dr, double* scal, cudaStream_t st) {
     const FinishList fin{3, {{part_det, 1, SC_MIN_DET}, {part_lam, 1, SC_MIN_LAM}, {part_dr, 2, SC_MAX_DR}}};
-    if (tiles(d)) {
+    const int tk = tile_k(d);
+    if (tk) {
         static_assert(SC_MIN_LAM == SC_MIN_DET + 1 && SC_MAX_DR == SC_MIN_DET + 2, "the bounds are adjacent");
         launch_counter() += 2;
-        k_extrema_stream<false><<<GBLOCKS, GJ * GK, 0, st>>>(d, phi, phi32, nullptr, part_det, part_lam, part_dr);
+        auto bound = tk == 32 ? k_extrema_stream<32, false> : k_extrema_stream<16, false>;
+        auto exact = tk == 32 ? k_extrema_stream<32, true> : k_extrema_stream<16, true>;
+        bound<<<GBLOCKS, GT, 0, st>>>(d, phi, phi32, nullptr, part_det, part_lam, part_dr);
         finish_reduces(fin, scal, st);
-        k_extrema_stream<true><<<GBLOCKS, GJ * GK, 0, st>>>(d, phi, phi32, scal + SC_MIN_DET, part_det, part_lam,
+        exact<<<GBLOCKS, GT, 0, st>>>(d, phi, phi32, scal + SC_MIN_DET, part_det, part_lam,
                                                             part_dr);
     } else {
         launch_geometry_out(d, phi, nullptr, nullptr, part_det, part_lam, st);
         launch_delta_r(d, phi, scratch, part_dr, st);
     }
     finish_reduces(fin, scal, st);
-    return tiles(d) ? 4 : 3;
+    return tk ? 4 : 3;
 }
 
 void launch_triad(const Dims& d, const double* phi, double* e6, cudaStream_t st) {

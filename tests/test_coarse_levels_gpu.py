@@ -88,7 +88,7 @@ def test_smoothing_forms_match_the_oracle(shape, s_side):
 
 
 @pytest.mark.parametrize("alpha", [0.125, 0.1])
-@pytest.mark.parametrize("shape", [(8, 8, 8), (8, 8, 32), (16, 8, 64), (8, 16, 16), (64, 32, 32)])
+@pytest.mark.parametrize("shape", [(8, 8, 8), (8, 8, 32), (16, 8, 64), (8, 16, 16), (32, 64, 16), (64, 32, 32)])
 def test_node_displacements_match_the_oracle(shape, alpha):
     """The tracers' displacements in fixed point and in FP64 (grids that do not
     fill the tile, step lengths that are no power of two): four steps with
@@ -110,7 +110,7 @@ def test_node_displacements_match_the_oracle(shape, alpha):
 
 
 @pytest.mark.parametrize("climiter", [0, 1, 2])
-@pytest.mark.parametrize("shape", [(8, 8, 8), (8, 8, 32), (16, 8, 64), (32, 16, 32)])
+@pytest.mark.parametrize("shape", [(8, 8, 8), (8, 8, 32), (16, 8, 64), (32, 16, 32), (32, 32, 16), (8, 16, 16)])
 def test_source_and_limiter_match_the_oracle(shape, climiter):
     """The screened source and limiter on strongly deformed maps where both
     limiters act (v_m = 1.5, xi_m = 0.5), every reading of C: the step lengths
@@ -129,7 +129,7 @@ def test_source_and_limiter_match_the_oracle(shape, climiter):
     assert np.linalg.norm(phi - ref.phi) <= BARS["fp64"] * np.linalg.norm(ref.phi)
 
 
-@pytest.mark.parametrize("shape", [(8, 8, 8), (8, 8, 32), (64, 32, 32), (16, 64, 64)])
+@pytest.mark.parametrize("shape", [(8, 8, 8), (8, 8, 32), (64, 32, 32), (16, 64, 64), (16, 32, 16)])
 def test_closing_statistics_are_those_of_the_fields(shape):
     """min det, min lambda0 and max delta_r of a solve's record are the extrema
     of the fields, to the last bit (the same FP64 arithmetic at the node that
