@@ -649,7 +649,7 @@ def _config(a, W):
     return {"workload": W.name, "grid": [n, n, n], "box_mpc_h": W.box,
             "displacement": "2LPT" if W.order == 2 else "ZA", "seed": W.seed,
             "k_max": a.k_max, "tol_in": 1e-8, "tol_out": 1e-3,
-            "l2": f"inputs larger than L2 (working set ~{n ** 3 * 235 / 1e9:.1f} GB per solve)",
+            "l2": f"inputs larger than L2 (working set ~{n ** 3 * 190 / 1e9:.1f} GB per solve)",
             "parallelism": f"replicas x{_dist()[1]}"}
 
 
