@@ -1,0 +1,113 @@
+// displacement_solve.cuh -- the node's system of the tracer displacement,
+// e U = alpha G in 64-bit fixed point (displacement.cu).  Integer and FP32 work
+// only, so that it also compiles for the host.
+#pragma once
+
+#include "fixed_point.cuh"
+
+namespace recon {
+
+constexpr int kDispBits = 53;  // fraction bits of a displacement, in cells
+
+// The scales of a step: phi 2^Q, dphi 2^Qd and alpha = 2^-kexp.  ok = false
+// where the fixed-point form does not apply: alpha is no power of two in
+// [2^-40, 1] (a replayed one), or the bound of a field is not finite or leaves
+// phi fewer than 46 fractional bits.
+struct DispScales {
+    int Q, Qd, kexp;
+    bool ok;
+};
+// e U = alpha G from the integer sums: h = second differences (xx, yy, zz) at
+// scale 2^Q and four times the mixed ones (xy, xz, yz), g = twice the gradient
+// of dphi at scale 2^Qd.  Returns whether U (scale 2^kDispBits) is within its
+// last place or so.
+__device__ __forceinline__ bool solve_fixed(const DispScales& sc, const long long (&h)[6],
+                                            const long long (&g)[3], long long (&out)[3]) {
+    // FP32: e, its inverse X and the right-hand side
+    int top = 0;  // every sum below 64 at its scale, or the node is not for integers
+#pragma unroll
+    for (int q = 0; q < 6; ++q) top = max(top, abs((int)(h[q] >> 32)));
+    if (top >= 1 << (sc.Q - 26)) return false;
+    const int low = sc.Q - 24;  // 22 .. 30: sums as 32-bit integers at scale 2^24
+    const float ue = pow2f(-24);
+    const float xx = 1.f + (float)(int)(h[0] >> low) * ue, yy = 1.f + (float)(int)(h[1] >> low) * ue,
+                zz = 1.f + (float)(int)(h[2] >> low) * ue;
+    const float xy = (float)(int)(h[3] >> low) * (0.25f * ue), xz = (float)(int)(h[4] >> low) * (0.25f * ue),
+                yz = (float)(int)(h[5] >> low) * (0.25f * ue);
+    float Xxx = yy * zz - yz * yz, Xyy = xx * zz - xz * xz, Xzz = xx * yy - xy * xy;
+    float Xxy = xz * yz - xy * zz, Xxz = xy * yz - yy * xz, Xyz = xy * xz - xx * yz;
+    const float rdet = __fdividef(1.f, xx * Xxx + xy * Xxy + xz * Xxz);
+    Xxx *= rdet, Xyy *= rdet, Xzz *= rdet, Xxy *= rdet, Xxz *= rdet, Xyz *= rdet;
+    const float emax = fmaxf(fmaxf(fabsf(xx), fabsf(yy)), fmaxf(fabsf(zz), fmaxf(fabsf(xy), fmaxf(fabsf(xz), fabsf(yz)))));
+    // the gradient brought to 62 bits first: most nodes' is far below the field's
+    // largest, which set its scale
+    using U64 = unsigned long long;
+    const U64 any = (U64)(g[0] ^ (g[0] >> 63)) | (U64)(g[1] ^ (g[1] >> 63)) | (U64)(g[2] ^ (g[2] >> 63));
+    const int sh = max(__clzll((long long)any) - 2, 0);
+    const float ug = pow2f(max(31 - sc.Qd - sc.kexp - sh, -126));
+    auto upper = [&](long long v) { return upper_float((long long)((U64)v << sh), ug); };
+    const float g0 = upper(g[0]), g1 = upper(g[1]), g2 = upper(g[2]);
+    // integers: e at scale 2^54 (Q <= 54)
+    const int up = 54 - sc.Q;
+    const U64 Exx = ((U64)h[0] << up) + (1ull << 54), Eyy = ((U64)h[1] << up) + (1ull << 54),
+              Ezz = ((U64)h[2] << up) + (1ull << 54);
+    auto mixed = [&](long long v) { return (U64)((((long long)((U64)v << up)) + 2) >> 2); };
+    const U64 Exy = mixed(h[3]), Exz = mixed(h[4]), Eyz = mixed(h[5]);
+    float u0, u1, u2, um;  // a piece and its largest magnitude
+    auto piece = [&](float r0, float r1, float r2) {
+        u0 = Xxx * r0 + Xxy * r1 + Xxz * r2;
+        u1 = Xxy * r0 + Xyy * r1 + Xyz * r2;
+        u2 = Xxz * r0 + Xyz * r1 + Xzz * r2;
+        um = fmaxf(fabsf(u0), fmaxf(fabsf(u1), fabsf(u2)));
+    };
+    piece(g0, g1, g2);
+    // The residual of a piece must fit 62 bits: the error of X is about
+    // 2^-22 |e|^2 / det; where that is more, smaller pieces.
+    const float gm = fmaxf(fabsf(g0), fmaxf(fabsf(g1), fabsf(g2)));
+    const float crit = emax * emax * emax * fabsf(rdet) * __fdividef(gm, fmaxf(um, 1e-30f));
+    if (!(um < 32.f && crit < 3e5f)) return false;
+    const int bits = 17 - max(((__float_as_int(crit) >> 23) & 255) - 127 - 9, 0);
+    // U = D 2^-s in pieces of at most bits + 1 bits, the last at 2^-57
+    auto scale_of = [&] { return min(bits - (((__float_as_int(um) >> 23) & 255) - 127), 57); };
+    int s = scale_of();
+    long long a0 = __float2int_rn(u0 * pow2f(s)), a1 = __float2int_rn(u1 * pow2f(s)), a2 = __float2int_rn(u2 * pow2f(s));
+    U64 D0 = a0, D1 = a1, D2 = a2;
+    float last = um, err = um;
+    constexpr float done = 7e-18f;  // 2^-57 cells
+    if (err >= done) {
+        const float xmax = fmaxf(fmaxf(fmaxf(fabsf(Xxx), fabsf(Xyy)), fmaxf(fabsf(Xzz), fabsf(Xxy))), fmaxf(fabsf(Xxz), fabsf(Xyz)));
+        const int n = 53 + s - sc.Qd - sc.kexp;
+        U64 R0 = shift_fixed(g[0], n), R1 = shift_fixed(g[1], n), R2 = shift_fixed(g[2], n);
+#pragma unroll 1
+        for (int it = 0; it < 7; ++it) {
+            // residual alpha G - e U at scale 2^(54 + s)
+            R0 -= Exx * (U64)a0 + Exy * (U64)a1 + Exz * (U64)a2;
+            R1 -= Exy * (U64)a0 + Eyy * (U64)a1 + Eyz * (U64)a2;
+            R2 -= Exz * (U64)a0 + Eyz * (U64)a1 + Ezz * (U64)a2;
+            const float ur = pow2f(-22 - s);
+            const U64 half = 1ull << 31;
+            piece(upper_float(R0 + half, ur), upper_float(R1 + half, ur), upper_float(R2 + half, ur));
+            // (22 bits at most: what the upper halves show of the residual)
+            const int ns = min(max(scale_of(), s), s + 22), m = ns - s;
+            s = ns;
+            const float sc2 = pow2f(s);
+            a0 = __float2int_rn(u0 * sc2), a1 = __float2int_rn(u1 * sc2), a2 = __float2int_rn(u2 * sc2);
+            D0 = (D0 << m) + a0, D1 = (D1 << m) + a1, D2 = (D2 << m) + a2;
+            // what remains: the piece's rounding, the residual's (half a unit
+            // of its upper half each, through X), or X's error as the last two
+            // pieces show it
+            err = fmaxf(fmaxf(pow2f(-1 - s), 1.5f * xmax * ur), um * __fdividef(um, last));
+            if (err < done) break;
+            if (!(um < 0.25f * last)) return false;
+            last = fmaxf(um, 6.f * xmax * ur);
+            R0 <<= m, R1 <<= m, R2 <<= m;
+        }
+    }
+    // 2^-53 cells; the pieces end at 2^-57 (at 2^-56 with err at its bound)
+    const int n = s - kDispBits;
+    auto place = [&](U64 v) { return n > 0 ? ((long long)(v + (1ull << (n - 1)))) >> n : (long long)(v << -n); };
+    out[0] = place(D0), out[1] = place(D1), out[2] = place(D2);
+    return err < done;
+}
+
+}  // namespace recon
