@@ -42,7 +42,7 @@ struct CicCharges {
 constexpr int kFracBits = 52;
 
 // The fixed-point position of a tracer along one axis: the offset from its
-// home node rounded to 2^-kFracBits of a cell (|off| < 2^11), as the lower
+// home node rounded to 2^-kFracBits of a cell (-2^11 <= off < 2^11), as the lower
 // node and the fraction f in [0, 2^kFracBits).  Below 2^10 cells the rounding is
 // integer work.
 __device__ inline void fixed_axis(int home, double off, int& i0, unsigned long long& f) {
@@ -141,9 +141,12 @@ __global__ void k_deposit_particles(Dims d, int64_t np, const double* __restrict
     const double scale = deposit_scale(total, given);
     // the position as an offset from node 0 (the same integer charges as the
     // tracers'; cell_index wraps it), first wrapped into [0, n) grid units where
-    // it is 2^10 cells away or more (x * inv_pow2(n) is x / n exactly)
+    // it is 2^10 cells away or more (x * inv_pow2(n) is x / n exactly), and from
+    // there into [-2^11, 2^11), which is what fixed_axis holds (n <= 4096)
     auto wrap = [](double x, int n) {
-        return fabs(x) < 1024.0 ? x : x - (double)n * floor(x * inv_pow2(n));
+        if (fabs(x) < 1024.0) return x;
+        const double y = x - (double)n * floor(x * inv_pow2(n));
+        return y < 2048.0 ? y : y - (double)n;
     };
     CicCharges q{};
     if (p < np) {
