@@ -124,7 +124,7 @@ __global__ void k_validate_particles(int64_t np, const double* __restrict__ pos,
 __device__ inline double deposit_scale(const double* __restrict__ total, double scale) {
     if (!total) return scale;
     const int e = (int)(__double_as_longlong(*total) >> 52) - 1022;  // total < 2^e
-    return __longlong_as_double((long long)(1023 + 61 - min(max(e, 1), 1000)) << 52);
+    return __longlong_as_double((long long)(1023 + 61 - min(max(e, 1), 1024)) << 52);
 }
 
 // bad: null, or set to 1 where a position is not finite (unit masses: such a

@@ -34,3 +34,18 @@ def test_positions_along_the_longest_axes(shape):
         R.deposit_particles(torch.from_numpy(pos).cuda())
         rho = R.field("density").cpu().numpy()
     assert np.abs(rho - ref).max() <= 2 * charges * 2.0 ** -46
+
+
+@pytest.mark.parametrize("exponent", [900, 985, 1000, 1009])
+def test_masses_up_to_the_end_of_the_range(exponent):
+    """The fixed point's unit follows the total mass by powers of two, so masses
+    times 2^exponent (a total of up to 2^1023) give the density times that, bit
+    for bit."""
+    r = np.random.default_rng(exponent)
+    pos = torch.from_numpy(r.uniform(0, 16, (5000, 3))).cuda()
+    mass = torch.from_numpy(r.uniform(0.5, 1.5, 5000)).cuda()
+    with Recon((16, 16, 16)) as R:
+        R.deposit_particles(pos, mass)
+        rho = R.field("density").clone()
+        R.deposit_particles(pos, mass * 2.0 ** exponent)
+        assert torch.equal(R.field("density"), rho * 2.0 ** exponent)
