@@ -16,6 +16,7 @@
 //
 // 512^3: the source 11.9 -> 1.08 ms (it formed and stored e in FP64), the
 // limiter 5.35 -> 1.12 ms; both are bound by instruction issue.
+#include "eigen32.cuh"
 #include "geometry.cuh"
 #include "recon_internal.cuh"
 #include "reduce.cuh"
@@ -32,7 +33,6 @@ struct Tile {
     static constexpr int J = GT / GK, PK = GK + 2, N = (J + 2) * PK;
 };
 constexpr int GPERSM = 3, GBLOCKS = GPERSM * (kRedBlocks / 8);
-constexpr float kU = 5.96046448e-8f;  // 2^-24
 
 // lambda_min(M) > floor by Sylvester's criterion on M - floor I.
 __device__ inline bool pd_above(Sym3 M, double floor) {
@@ -447,9 +447,6 @@ __global__ void k_geometry_out(Dims d, const double* __restrict__ phi, double* _
 // the FP64 value of the node that attains it.  The first pass (EXACT = false)
 // bounds them from FP32 values (the smallest upper bounds, the largest lower
 // one), the second evaluates in FP64 the nodes that the bounds leave open.
-// lambda0 in FP32 comes from the closed form: Weyl's theorem bounds what the
-// entries' errors do to it, and the angle's error, at most the square root of
-// the rounding of the determinant that it is taken from, is covered by 2^-8 p.
 // 512^3: 26 -> 2.0 ms for all three (FP64 at every node, 23 of them for det and
 // lambda0).
 template <int GK, bool EXACT>
@@ -483,14 +480,8 @@ __global__ void __launch_bounds__(GT, GPERSM) k_extrema_stream(Dims d, const dou
                               h.xz * (h.xy * h.yz - yy * h.xz);
             const float ed = 9.0f * eps * big * big + 3.0f * eps * eps * big + eps * eps * eps +
                              72.0f * kU * big * big * big;
-            const float q = (xx + yy + zz) * (1.f / 3.f);
-            const float b1 = xx - q, b2 = yy - q, b3 = zz - q;
-            const float p2 = b1 * b1 + b2 * b2 + b3 * b3 + 2.f * (h.xy * h.xy + h.xz * h.xz + h.yz * h.yz);
-            const float pp = sqrtf(p2 * (1.f / 6.f)), ip = 1.f / fmaxf(pp, 1e-30f);
-            const float r = 0.5f * ip * ip * ip * (b1 * (b2 * b3 - h.yz * h.yz) - h.xy * (h.xy * b3 - h.yz * h.xz) +
-                                                  h.xz * (h.xy * h.yz - b2 * h.xz));
-            const float lam = q + 2.f * pp * cosf(acosf(fminf(1.f, fmaxf(-1.f, r))) * (1.f / 3.f) + 2.0943951f);
-            const float el = 3.f * eps + 0.00390625f * pp + 16.f * kU * big;
+            float el;
+            const float lam = lambda32(h.xx, h.yy, h.zz, h.xy, h.xz, h.yz, big, eps, el);
             const float dr = -(h.xx + h.yy + h.zz), er = 3.f * eps + 8.f * kU * (big + 1.f);
             if (!EXACT) {
                 fd = fminf(fd, det + ed), fl = fminf(fl, lam + el), fr = fmaxf(fr, dr - er);
