@@ -17,8 +17,7 @@ __device__ inline void set_cond(const CtlHandles& h, cudaGraphConditionalHandle 
     if (h.active) cudaGraphSetConditional(c, v ? 1u : 0u);
 }
 
-__global__ void k_ctl_init(Ctl* c, double* scal) {
-    if (scal) scal[SC_PHI_BOUND] = 0.0;
+__global__ void k_ctl_init(Ctl* c) {
     c->k = 0, c->status = RECON_NOT_CONVERGED, c->vtot = 0, c->ncyc = 0;
     c->final_deposit = 1;
     c->n_step = c->n_cont = c->n_mg = c->n_adv = c->n_fin = 0;
@@ -156,8 +155,7 @@ __global__ void k_warm_extrapolate(const Ctl* __restrict__ c, const double* __re
 // max |alpha grad dphi| > d_max; below alpha_min the iteration stops with the
 // current map (RECON_STALLED).  With a replay array alpha_k is taken from it.
 __global__ void k_ctl_select_alpha(Ctl* c, double* scal, CtlArrays a, const double* replay,
-                                   int kmax_exp, double ncells, double d_max, double alpha_min,
-                                   CtlHandles h) {
+                                   int kmax_exp, double d_max, double alpha_min, CtlHandles h) {
     const int k = c->k;
     double alpha;
     if (replay) {
@@ -177,10 +175,6 @@ __global__ void k_ctl_select_alpha(Ctl* c, double* scal, CtlArrays a, const doub
     }
     c->alpha = alpha;
     scal[SC_ALPHA] = alpha;
-    // max |phi| after the advance is at most that plus alpha max |dphi - mean|
-    // (SC_MAX_DPHI is of an FP32 copy; the factors cover every rounding)
-    scal[SC_PHI_BOUND] = (scal[SC_PHI_BOUND] + fabs(alpha) * (scal[SC_MAX_DPHI] * (1.0 + 1e-6) +
-                                                               fabs(scal[SC_SUM_DPHI]) / ncells)) * (1.0 + 1e-12);
     a.alpha[k] = alpha;
     c->go_adv = 1;
     set_cond(h, h.adv, 1);
@@ -210,9 +204,9 @@ __global__ void k_ctl_final_mass(Ctl* c, const double* scal) {
 
 }  // namespace
 
-void launch_ctl_init(Ctl* c, double* scal, cudaStream_t st) {
+void launch_ctl_init(Ctl* c, cudaStream_t st) {
     launch_counter()++;
-    k_ctl_init<<<1, 1, 0, st>>>(c, scal);
+    k_ctl_init<<<1, 1, 0, st>>>(c);
 }
 void launch_ctl_step_begin(Ctl* c, const double* scal, const CtlArrays& a, double ncells,
                            double tol_out, const CtlHandles& h, cudaStream_t st) {
@@ -253,10 +247,10 @@ void launch_zero_if_fresh(const Ctl* c, float* u, int cells, cudaStream_t st) {
 }
 
 void launch_ctl_select_alpha(Ctl* c, double* scal, const CtlArrays& a, const double* replay,
-                             int kmax_exp, double ncells, double d_max, double alpha_min,
-                             const CtlHandles& h, cudaStream_t st) {
+                             int kmax_exp, double d_max, double alpha_min, const CtlHandles& h,
+                             cudaStream_t st) {
     launch_counter()++;
-    k_ctl_select_alpha<<<1, 1, 0, st>>>(c, scal, a, replay, kmax_exp, ncells, d_max, alpha_min, h);
+    k_ctl_select_alpha<<<1, 1, 0, st>>>(c, scal, a, replay, kmax_exp, d_max, alpha_min, h);
 }
 void launch_ctl_step_end(Ctl* c, int k_max, const CtlHandles& h, cudaStream_t st) {
     launch_counter()++;

@@ -6,7 +6,9 @@
 // In FP64 a node takes some 70 instructions (the Hessian, six cofactors, a
 // division, three products), 10 ms at 512^3 with the Hessian read back from
 // memory.  Here only FP32 and integer instructions run: phi and dphi are
-// brought to 64-bit fixed point as a plane is loaded, Hessian and gradient are
+// brought to 64-bit fixed point as a plane is loaded (phi to 2^-54 whatever its
+// size, modulo 2^64: the source's pass over the same phi shows that every
+// second difference fits; dphi to 2^-Qd from the limiter's largest gradient), Hessian and gradient are
 // exact integer sums, and e U = alpha G is solved by iterative refinement: X ~
 // e^-1 in FP32 gives a first U, and each further piece comes from the exact
 // residual alpha G - e U, formed modulo 2^64 (its leading bits cancel, so the
@@ -14,9 +16,11 @@
 // three residuals leave an error below the 2^-53 cells of the result; badly
 // conditioned nodes take smaller pieces and more of them.  Nodes that do not
 // converge, and steps whose numbers do not fit (disp_scales), are computed in
-// FP64.  Against 113-bit arithmetic (64^3, |phi| <= 4, det e >= 0.48, alpha V <=
-// 0.42 cells) the error is 0.291 units of 2^-53 cells rms and 0.78 at most, that
-// of the FP64 form 0.321 and 1.97 (rounding to the unit alone: 0.289).
+// FP64.  Against exact rational arithmetic (smooth fields with |phi| up to 4, 60
+// and 166 cells^2, alpha V up to half a cell) the error is 0.29 units of 2^-53 cells rms and
+// 0.57 at most, also at the nodes of the large fields where phi is small; that
+// of the FP64 form 0.29, 0.61 and 4.9 rms (0.29, 0.44 and 0.33 where |phi| < 6),
+// 148 at most (rounding to the unit alone: 0.289).
 //
 // A block streams planes along i over an 8 x 32 (or 16 x 16) tile; a thread keeps its
 // column's sums of the last planes in registers, so that a plane's 340 nodes
@@ -60,25 +64,15 @@ __device__ __noinline__ void displacement64(const Dims& d, const double* __restr
     out[2] = fix((Axz * gx + Ayz * gy + Azz * gz) * hinv);
 }
 
-__device__ inline DispScales disp_scales(const double* scal) {
-    DispScales s;
-    const long long a = __double_as_longlong(scal[SC_ALPHA]);
-    s.kexp = 1023 - (int)(a >> 52);
-    s.Q = fixed_bits(scal[SC_PHI_BOUND], 54);
-    s.Qd = fixed_bits(scal[SC_MAX_DPHI], 120);
-    s.ok = (a & 0xfffffffffffffll) == 0 && a > 0 && s.kexp >= 0 && s.kexp <= 40 && s.Q >= 46 && s.Qd > -1000;
-    return s;
-}
-
 template <int DK>
 __global__ void __launch_bounds__(DT, DPERSM) k_displacement_stream(
     Dims d, const double* __restrict__ scal, const double* __restrict__ phi, const double* __restrict__ dphi,
     long long* __restrict__ dx, long long* __restrict__ dy, long long* __restrict__ dz) {
     constexpr int DJ = DT / DK, DPK = DK + 2, DN = (DJ + 2) * DPK;  // rows, and with the ring
     static_assert(DN <= 2 * DT, "two values a thread and field");
-    __shared__ long long sp[2][DN], sd[2][DN];
-    const DispScales sc = disp_scales(scal);
+    __shared__ U64 sp[2][DN], sd[2][DN];
     const double alpha = scal[SC_ALPHA];
+    const DispScales sc = disp_scales(alpha, scal[SC_MAX_G], scal[SC_SUM_DPHI], scal[SC_WIDE] != 0.0);
     const int t = threadIdx.x, lj = t / DK, lk = t % DK;
     const int own = (lj + 1) * DPK + lk + 1;
     const int tiles_k = d.n2 / DK;
@@ -113,32 +107,22 @@ __global__ void __launch_bounds__(DT, DPERSM) k_displacement_stream(
             p0 = phi[b + c0], q0 = dphi[b + c0];
             if (two) p1 = phi[b + c1], q1 = dphi[b + c1];
         };
-        // sums of the column on planes p - 2, p - 1 (own value, differences in
-        // j and k, own dphi), and plane p - 1's second differences and gradient
-        long long ca = 0, cb = 0, ja = 0, jb = 0, ka = 0, kb = 0, da = 0, db = 0;
-        long long syb = 0, szb = 0, yzb = 0, gyb = 0, gzb = 0;
+        DispColumn sums{};
         load(i0 - 1);
         for (int p = i0 - 1; p <= i1; ++p) {
             const int buf = (p - i0 + 1) & 1;
-            sp[buf][t] = to_fixed(p0, sc.Q), sd[buf][t] = to_fixed(q0, sc.Qd);
-            if (two) sp[buf][e1] = to_fixed(p1, sc.Q), sd[buf][e1] = to_fixed(q1, sc.Qd);
+            sp[buf][t] = to_fixed_mod(p0, kPhiBits), sd[buf][t] = to_fixed_mod(q0, sc.Qd);
+            if (two) sp[buf][e1] = to_fixed_mod(p1, kPhiBits), sd[buf][e1] = to_fixed_mod(q1, sc.Qd);
             if (p < i1) load(p + 1);
             __syncthreads();  // (the other buffer is read until the next one)
-            const long long *f = sp[buf] + own, *w = sd[buf] + own;
-            const long long c = f[0], jp = f[DPK], jm = f[-DPK], kp = f[1], km = f[-1], dc = w[0];
-            const long long jd = jp - jm, kd = kp - km;
+            long long h[6], g[3];
+            sums.feed(sp[buf] + own, sd[buf] + own, DPK, h, g);
             if (p > i0) {  // node (p - 1)
-                const long long h[6] = {c + ca - 2 * cb, syb, szb, jd - ja, kd - ka, yzb};
-                const long long g[3] = {dc - da, gyb, gzb};
                 long long o[3];
                 if (!solve_fixed(sc, h, g, o)) displacement64(d, phi, dphi, alpha, p - 1, j0 + lj, k0 + lk, o);
                 const int cell = cell_index(d, p - 1, j0 + lj, k0 + lk);
                 dx[cell] = o[0], dy[cell] = o[1], dz[cell] = o[2];
             }
-            syb = jp + jm - 2 * c, szb = kp + km - 2 * c;
-            yzb = (f[DPK + 1] - f[DPK - 1]) - (f[-DPK + 1] - f[-DPK - 1]);
-            gyb = w[DPK] - w[-DPK], gzb = w[1] - w[-1];
-            ca = cb, cb = c, ja = jb, jb = jd, ka = kb, kb = kd, da = db, db = dc;
         }
         __syncthreads();
     }

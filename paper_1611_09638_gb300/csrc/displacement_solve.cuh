@@ -9,17 +9,55 @@ namespace recon {
 
 constexpr int kDispBits = 53;  // fraction bits of a displacement, in cells
 
-// The scales of a step: phi 2^Q, dphi 2^Qd and alpha = 2^-kexp.  ok = false
-// where the fixed-point form does not apply: alpha is no power of two in
-// [2^-40, 1] (a replayed one), or the bound of a field is not finite or leaves
-// phi fewer than 46 fractional bits.
+using U64 = unsigned long long;
+
+// phi's scale: 2^kPhiBits, modulo 2^64.
+constexpr int kPhiBits = 54;
+
+// The scales of a step: dphi 2^Qd and alpha = 2^-kexp.  ok = false where the
+// fixed-point form does not apply: alpha is no power of two in [2^-40, 1] (a
+// replayed one), some second difference of phi may not be known from its value
+// modulo 2^10 cells (wide), or dphi is not finite (sum_dphi) or beyond 2^90.
+// max_g: the largest central difference of dphi.  It, and not dphi's own size,
+// sets Qd, since only differences of dphi are used.
 struct DispScales {
-    int Q, Qd, kexp;
+    int Qd, kexp;
     bool ok;
 };
+__device__ __forceinline__ DispScales disp_scales(double alpha, double max_g, double sum_dphi, bool wide) {
+    DispScales s;
+    const long long a = __double_as_longlong(alpha), g = __double_as_longlong(max_g);
+    const int e = (int)(g >> 52) & 0x7ff, es = (int)(__double_as_longlong(sum_dphi) >> 52) & 0x7ff;
+    s.kexp = 1023 - (int)(a >> 52);
+    s.Qd = min(120, 1083 - e);  // max_g < 2^(e - 1022), twice that below 2^62
+    s.ok = (a & 0xfffffffffffffll) == 0 && a > 0 && s.kexp >= 0 && s.kexp <= 40 && !wide && es < 0x7ff &&
+           g >= 0 && e <= 1022 + 90;
+    return s;
+}
+
+// A column's sums over the planes it is fed: the second differences of phi and
+// twice the gradient of dphi at the node one plane back, both modulo 2^64.
+struct DispColumn {
+    U64 ca, cb, ja, jb, ka, kb, da, db;      // planes p - 2, p - 1: own value, differences in j and k, own dphi
+    U64 syb, szb, yzb, gyb, gzb;             // plane p - 1's second differences and gradient
+    // f, w: the node's phi and dphi in the plane, rows of `row` values apart;
+    // h (xx, yy, zz and four times xy, xz, yz) and g are those of the node before
+    __device__ __forceinline__ void feed(const U64* f, const U64* w, int row, long long (&h)[6], long long (&g)[3]) {
+        const U64 c = f[0], jp = f[row], jm = f[-row], kp = f[1], km = f[-1], dc = w[0];
+        const U64 jd = jp - jm, kd = kp - km;
+        h[0] = (long long)(c + ca - 2 * cb), h[1] = (long long)syb, h[2] = (long long)szb;
+        h[3] = (long long)(jd - ja), h[4] = (long long)(kd - ka), h[5] = (long long)yzb;
+        g[0] = (long long)(dc - da), g[1] = (long long)gyb, g[2] = (long long)gzb;
+        syb = jp + jm - 2 * c, szb = kp + km - 2 * c;
+        yzb = (f[row + 1] - f[row - 1]) - (f[-row + 1] - f[-row - 1]);
+        gyb = w[row] - w[-row], gzb = w[1] - w[-1];
+        ca = cb, cb = c, ja = jb, jb = jd, ka = kb, kb = kd, da = db, db = dc;
+    }
+};
+
 // e U = alpha G from the integer sums: h = second differences (xx, yy, zz) at
-// scale 2^Q and four times the mixed ones (xy, xz, yz), g = twice the gradient
-// of dphi at scale 2^Qd.  Returns whether U (scale 2^kDispBits) is within its
+// scale 2^kPhiBits and four times the mixed ones (xy, xz, yz), g = twice the
+// gradient of dphi at scale 2^Qd.  Returns whether U (scale 2^kDispBits) is within its
 // last place or so.
 __device__ __forceinline__ bool solve_fixed(const DispScales& sc, const long long (&h)[6],
                                             const long long (&g)[3], long long (&out)[3]) {
@@ -27,8 +65,8 @@ __device__ __forceinline__ bool solve_fixed(const DispScales& sc, const long lon
     int top = 0;  // every sum below 64 at its scale, or the node is not for integers
 #pragma unroll
     for (int q = 0; q < 6; ++q) top = max(top, abs((int)(h[q] >> 32)));
-    if (top >= 1 << (sc.Q - 26)) return false;
-    const int low = sc.Q - 24;  // 22 .. 30: sums as 32-bit integers at scale 2^24
+    if (top >= 1 << (kPhiBits - 26)) return false;
+    constexpr int low = kPhiBits - 24;  // sums as 32-bit integers at scale 2^24
     const float ue = pow2f(-24);
     const float xx = 1.f + (float)(int)(h[0] >> low) * ue, yy = 1.f + (float)(int)(h[1] >> low) * ue,
                 zz = 1.f + (float)(int)(h[2] >> low) * ue;
@@ -41,17 +79,15 @@ __device__ __forceinline__ bool solve_fixed(const DispScales& sc, const long lon
     const float emax = fmaxf(fmaxf(fabsf(xx), fabsf(yy)), fmaxf(fabsf(zz), fmaxf(fabsf(xy), fmaxf(fabsf(xz), fabsf(yz)))));
     // the gradient brought to 62 bits first: most nodes' is far below the field's
     // largest, which set its scale
-    using U64 = unsigned long long;
     const U64 any = (U64)(g[0] ^ (g[0] >> 63)) | (U64)(g[1] ^ (g[1] >> 63)) | (U64)(g[2] ^ (g[2] >> 63));
     const int sh = max(__clzll((long long)any) - 2, 0);
     const float ug = pow2f(max(31 - sc.Qd - sc.kexp - sh, -126));
     auto upper = [&](long long v) { return upper_float((long long)((U64)v << sh), ug); };
     const float g0 = upper(g[0]), g1 = upper(g[1]), g2 = upper(g[2]);
-    // integers: e at scale 2^54 (Q <= 54)
-    const int up = 54 - sc.Q;
-    const U64 Exx = ((U64)h[0] << up) + (1ull << 54), Eyy = ((U64)h[1] << up) + (1ull << 54),
-              Ezz = ((U64)h[2] << up) + (1ull << 54);
-    auto mixed = [&](long long v) { return (U64)((((long long)((U64)v << up)) + 2) >> 2); };
+    // integers: e at scale 2^54
+    const U64 Exx = (U64)h[0] + (1ull << kPhiBits), Eyy = (U64)h[1] + (1ull << kPhiBits),
+              Ezz = (U64)h[2] + (1ull << kPhiBits);
+    auto mixed = [&](long long v) { return (U64)((v + 2) >> 2); };
     const U64 Exy = mixed(h[3]), Exz = mixed(h[4]), Eyz = mixed(h[5]);
     float u0, u1, u2, um;  // a piece and its largest magnitude
     auto piece = [&](float r0, float r1, float r2) {

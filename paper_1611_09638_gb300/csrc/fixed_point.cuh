@@ -1,8 +1,8 @@
 // fixed_point.cuh -- 64-bit fixed-point forms of the FP64 fields.  GB300
 // issues two FP64 operations a clock and SM against 64 or more integer ones,
 // so stencils of phi and dphi that need more than FP32 run on integers: a
-// value is scaled by a power of two 2^Q, chosen once per field from a bound on
-// its magnitude, and rounded; sums and differences of such values are exact.
+// value is scaled by a power of two 2^Q and rounded; sums and differences of
+// such values are exact, also modulo 2^64 where the result is known to fit.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -21,13 +21,16 @@ __device__ __forceinline__ long long to_fixed(double x, int Q) {
     return ((long long)v ^ s) - s;
 }
 
-// The largest Q <= most with bound 2^Q <= 2^60, for a bound >= 0; -1000 where
-// there is none to use (not finite, or above 2^90).
-__device__ __forceinline__ int fixed_bits(double bound, int most) {
-    const long long b = __double_as_longlong(bound);
-    const int e = (int)(b >> 52) & 0x7ff;  // bound < 2^(e - 1022)
-    if (b < 0 || e > 1022 + 90) return -1000;
-    return min(most, 60 - (e - 1022));
+// x 2^Q rounded to nearest modulo 2^64, for any finite x.
+__device__ __forceinline__ unsigned long long to_fixed_mod(double x, int Q) {
+    const long long b = __double_as_longlong(x);
+    const int e = (int)(b >> 52) & 0x7ff;
+    const unsigned long long m = e ? (((unsigned long long)b << 10) & 0x3ffffffffffffc00ull) | (1ull << 62) : 0ull;
+    const int r = 1085 - Q - e, t = min(max(r, 0), 63), l = min(max(-r, 0), 63);
+    // (r < -63 leaves nothing below 2^64: m is a multiple of 2^10)
+    const unsigned long long v = r > 63 ? 0ull : ((m + ((1ull << t) >> 1)) >> t) << l;
+    const unsigned long long s = (unsigned long long)(b >> 63);
+    return (v ^ s) - s;
 }
 
 // v 2^n modulo 2^64 for n >= 0, v 2^n rounded for n < 0.

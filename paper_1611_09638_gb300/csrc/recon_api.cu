@@ -499,9 +499,10 @@ void step_head(Handle* H, const CtlHandles& h) {
     if (H->ckpt) launch_ckpt_state(H->ctl, H->cells, H->phi, H->ox, H->oy, H->oz, H->ckpt, H->st);
     deposit_step(H, false);
     SourceParams sp{p.xi_m, p.v_m, p.climiter};
-    launch_source(H->d, sp, H->phi, H->phi32, H->m, H->t, H->part[1], H->st);
-    finish_reduces({2, {{H->part[0], 0, SC_SUM_M}, {H->part[1], 0, SC_SUM_T}}}, H->scal, H->st);
-    launch_smooth_S(H->d, p.s_side, H->t, H->scal + SC_SUM_T, H->s, nullptr, H->v3, nullptr, nullptr,
+    launch_source(H->d, sp, H->phi, H->phi32, H->m, H->t, H->part[1], H->part[3], H->st);
+    finish_reduces({3, {{H->part[0], 0, SC_SUM_M}, {H->part[1], 0, SC_SUM_T}, {H->part[3], 2, SC_WIDE}}}, H->scal,
+                   H->st);
+    launch_smooth_S(H->d, p.s_side, H->t, H->scal + SC_SUM_T, H->s, nullptr, H->v3, nullptr,
                     H->part[2], H->st);
     finish_reduce(H->part[2], 0, H->scal, SC_SUM_S2, H->st);
     launch_ctl_step_begin(H->ctl, H->scal, H->arr, (double)H->cells, p.tol_out, h, H->st);
@@ -591,17 +592,19 @@ void step_tail(Handle* H, const CtlHandles& h) {
     const recon_params& p = H->p;
     if (H->ckpt) launch_ckpt_phidot(H->ctl, H->cells, H->phidot, H->ckpt, H->st);
     launch_smooth_S(H->d, p.s_side, H->phidot, nullptr, H->dphi, H->dphi32, H->v3, H->part[0],
-                    H->part[3], nullptr, H->st);
-    FinishList fin{2, {{H->part[0], 0, SC_SUM_DPHI}, {H->part[3], 2, SC_MAX_DPHI}}};
-    if (!H->replay_d) {
+                    nullptr, H->st);
+    FinishList fin{1, {{H->part[0], 0, SC_SUM_DPHI}}};
+    // (with replayed step lengths the displacements still take the largest
+    // gradient from it)
+    if (!H->replay_d || p.density_update == 0) {
         launch_limiter(H->d, H->lp, H->phi, H->dphi, H->phi32, H->dphi32, H->part[1], H->part[2],
                        H->st);
         fin.f[fin.n++] = {H->part[1], 2, SC_MAX_K};
         fin.f[fin.n++] = {H->part[2], 2, SC_MAX_G};
     }
     finish_reduces(fin, H->scal, H->st);
-    launch_ctl_select_alpha(H->ctl, H->scal, H->arr, H->replay_d, H->lp.kmax, (double)H->cells, p.d_max,
-                            p.alpha_min, h, H->st);
+    launch_ctl_select_alpha(H->ctl, H->scal, H->arr, H->replay_d, H->lp.kmax, p.d_max, p.alpha_min,
+                            h, H->st);
 }
 
 // Advance by the chosen alpha: tracers and phi (or, App. A's variant, the
@@ -625,7 +628,7 @@ void advance(Handle* H, const CtlHandles& h) {
 
 // init: tracer c = node c with mass rho_c / rho_bar, phi = 0
 void solve_init(Handle* H) {
-    launch_ctl_init(H->ctl, H->scal, H->st);
+    launch_ctl_init(H->ctl, H->st);
     cudaMemsetAsync(H->phidot, 0, sizeof(double) * H->cells, H->st);  // the first step's initial guess
     launch_init_tracers(H->cells, H->rho, H->scal + SC_SUM_RHO, H->w, H->ox, H->oy, H->oz, H->phi,
                         H->phi32, H->st);
@@ -1076,7 +1079,7 @@ int solve(Handle* H, recon_stats* stats) {
 // adjoint's own control block; u is left in H->phidot.
 int adjoint_mg(Handle* H) {
     const CtlHandles none{};
-    launch_ctl_init(H->ctl, nullptr, H->st);
+    launch_ctl_init(H->ctl, H->st);
     launch_ctl_step_begin(H->ctl, H->scal, H->arr, (double)H->cells, -1.0, none, H->st);
     mg_head(H, none, false);  // each adjoint solve starts from 0
     int rc = read_ctl(H);
@@ -1121,7 +1124,7 @@ int adjoint(Handle* H, const double* gbar, double* grad) {
         launch_mass_coef(cells, H->mfix, 1.0 / scale, p.a_min, H->m, H->a64,
                          H->mixed ? H->c32[0] : nullptr, H->part[0], st);
         launch_triad(d, phi_k, H->e6, st);
-        launch_smooth_S(d, p.s_side, pd, nullptr, H->dphi, nullptr, H->v3, nullptr, nullptr, nullptr, st);
+        launch_smooth_S(d, p.s_side, pd, nullptr, H->dphi, nullptr, H->v3, nullptr, nullptr, st);
         launch_node_velocity(d, H->e6, H->dphi, H->v3, H->v3 + n, H->v3 + 2 * n, st);
         // back through the advance, V = e^-1 G and dphi = S phidot - mean
         CK(cudaMemsetAsync(A.vb, 0, 3 * n * sizeof(double), st));
@@ -1130,7 +1133,7 @@ int adjoint(Handle* H, const double* gbar, double* grad) {
         launch_adj_dbar(d, alpha, A.phibar, A.gb, A.dbar, H->part[0], st);
         finish_reduce(H->part[0], 0, H->scal, SC_ADJ_A, st);
         launch_smooth_S(d, p.s_side, A.dbar, H->scal + SC_ADJ_A, H->s, nullptr, H->v3, nullptr,
-                        nullptr, H->part[2], st);
+                        H->part[2], st);
         finish_reduce(H->part[2], 0, H->scal, SC_SUM_S2, st);
         // the linear solve: the adjoint solve with the same operator
         rc = adjoint_mg(H);
@@ -1140,7 +1143,7 @@ int adjoint(Handle* H, const double* gbar, double* grad) {
         launch_adj_coef(d, H->phidot, pd, H->m, p.a_min, A.mbar, H->part[0], st);
         finish_reduce(H->part[0], 0, H->scal, SC_ADJ_B, st);
         launch_smooth_S(d, p.s_side, H->phidot, H->scal + SC_ADJ_B, H->t, nullptr, H->v3, nullptr,
-                        nullptr, nullptr, st);
+                        nullptr, st);
         launch_adj_source(d, sp, H->e6, H->m, H->t, A.mbar, A.eb, st);
         launch_adj_hess(d, A.eb, A.phibar, st);
         launch_adj_deposit(d, ox, oy, oz, H->w, A.mbar, A.wbar, A.xib, st);

@@ -82,10 +82,9 @@ enum Scalar {
     SC_ALPHA,         // step length of the current step
     SC_ADJ_A,         // adjoint sweep: sums used for mean projections
     SC_ADJ_B,
-    SC_MAX_DPHI,      // a bound on max |dphi| of the step
+    SC_WIDE,          // nonzero unless FP32 shows every second difference of phi well below 512
     SC_MASS,          // total mass of the deposited particles
     SC_BAD_PARTICLE,  // nonzero if a particle was NaN/Inf or negative; 0 between deposits
-    SC_PHI_BOUND,     // a bound on max |phi|, grown by every advance
     SC_COUNT
 };
 
@@ -314,15 +313,17 @@ void launch_mass_coef(int cells, unsigned long long* mfix, double inv_scale, dou
 // e6 (6 x cells): the triad e = I + Hess phi (xx, yy, zz, xy, xz, yz), for the
 // adjoint and the carried mass of App. A's variant.
 void launch_triad(const Dims& d, const double* phi, double* e6, cudaStream_t st);
-// t = Sigma + C + E from phi (and its FP32 copy) and m, and partial sums of t.
+// t = Sigma + C + E from phi (and its FP32 copy) and m, partial sums of t and
+// the partials of SC_WIDE (to be finished by a maximum).
 void launch_source(const Dims& d, const SourceParams& sp, const double* phi, const float* phi32, const double* m,
-                   double* t, double* part_sum, cudaStream_t st);
-// S in three axis passes through tmp2 (2 x cells scratch); out32 (optional)
-// receives an FP32 copy of the result; part_sum (with out32 and part_max) its
-// sum and largest magnitude, part_sq its sum of squares, or neither.
+                   double* t, double* part_sum, double* part_wide, cudaStream_t st);
+// S in one pass, or in three axis passes through tmp2 (2 x cells scratch) on
+// grids that its tile does not fit; out32 (optional) receives an FP32 copy of
+// the result; part_sum (with out32) its sum, part_sq its sum of squares, or
+// neither.
 void launch_smooth_S(const Dims& d, double s_side, const double* in, const double* shift_scalar,
-                     double* out, float* out32, double* tmp2, double* part_sum, double* part_max,
-                     double* part_sq, cudaStream_t st);
+                     double* out, float* out32, double* tmp2, double* part_sum, double* part_sq,
+                     cudaStream_t st);
 // phi32, dphi32: FP32 copies of phi and dphi used to screen nodes that clear
 // the limiter's floor by a wide margin.
 void launch_limiter(const Dims& d, const LimiterParams& lp, const double* phi, const double* dphi,
@@ -331,7 +332,7 @@ void launch_limiter(const Dims& d, const LimiterParams& lp, const double* phi, c
 void launch_node_velocity(const Dims& d, const double* e6, const double* dphi, double* vx,
                           double* vy, double* vz, cudaStream_t st);
 // The step's node displacements alpha V in fixed point (2^-53 cells), for
-// launch_advance; scal: SC_ALPHA, SC_PHI_BOUND and SC_MAX_DPHI are read.
+// launch_advance; scal: SC_ALPHA, SC_MAX_G, SC_SUM_DPHI and SC_WIDE are read.
 void launch_node_displacement(const Dims& d, const double* scal, const double* phi, const double* dphi,
                               long long* dx, long long* dy, long long* dz, cudaStream_t st);
 // Tracers move by -alpha V(xi) (the fixed-point displacements CIC-interpolated
@@ -395,8 +396,7 @@ struct CtlHandles {
     cudaGraphConditionalHandle step, cont, mg, adv, fin, chk;
 };
 
-// scal: SC_PHI_BOUND starts at 0 (null: the scalars stay as they are)
-void launch_ctl_init(Ctl* c, double* scal, cudaStream_t st);
+void launch_ctl_init(Ctl* c, cudaStream_t st);
 void launch_ctl_step_begin(Ctl* c, const double* scal, const CtlArrays& a, double ncells,
                            double tol_out, const CtlHandles& h, cudaStream_t st);
 void launch_ctl_mg_begin(Ctl* c, const CtlArrays& a, int mixed, double tol_in,
@@ -417,8 +417,8 @@ void launch_warm_extrapolate(const Ctl* c, const double* alpha, double* u, doubl
 void launch_ctl_mg_check(Ctl* c, const double* scal, const CtlArrays& a, int per_launch,
                          double tol_in, int max_vcycles, const CtlHandles& h, cudaStream_t st);
 void launch_ctl_select_alpha(Ctl* c, double* scal, const CtlArrays& a, const double* replay,
-                             int kmax_exp, double ncells, double d_max, double alpha_min,
-                             const CtlHandles& h, cudaStream_t st);
+                             int kmax_exp, double d_max, double alpha_min, const CtlHandles& h,
+                             cudaStream_t st);
 void launch_ctl_step_end(Ctl* c, int k_max, const CtlHandles& h, cudaStream_t st);
 void launch_ctl_final(Ctl* c, int want, const CtlHandles& h, cudaStream_t st);
 void launch_ctl_final_mass(Ctl* c, const double* scal, cudaStream_t st);

@@ -188,14 +188,17 @@ __device__ __noinline__ double source64(const Dims& d, const SourceParams& sp, c
 
 // C = E = 0 where FP32 certifies that every eigenvalue of e exceeds xi_m
 // (Sylvester's criterion) and, e being positive definite then, that its trace
-// stays below 3 v_m^(1/3) (det e <= (tr e / 3)^3).
+// stays below 3 v_m^(1/3) (det e <= (tr e / 3)^3).  pwide: 1 where a second
+// difference of phi, or four times a mixed one, may reach 448 (or is not finite);
+// the displacements of the step know them modulo 1024 only.
 template <int GK>
 __global__ void __launch_bounds__(GT, GPERSM) k_source_stream(Dims d, SourceParams sp, float trace_max,
                                                                   const double* __restrict__ phi,
                                                                   const float* __restrict__ phi32,
                                                                   const double* __restrict__ m,
                                                                   double* __restrict__ t,
-                                                                  double* __restrict__ psum) {
+                                                                  double* __restrict__ psum,
+                                                                  double* __restrict__ pwide) {
     constexpr int GPK = Tile<GK>::PK;
     __shared__ float buf[2][1][Tile<GK>::N];
     __shared__ int list[GT / 32][64];
@@ -205,6 +208,7 @@ __global__ void __launch_bounds__(GT, GPERSM) k_source_stream(Dims d, SourcePara
     WarpList todo{list[threadIdx.x / 32], 0};
     Column32<GPK> col{};
     double s = 0.0;
+    bool wide = false;
     auto exact = [&] {
         const int c = todo.take();
         if (c >= 0) {
@@ -225,6 +229,8 @@ __global__ void __launch_bounds__(GT, GPERSM) k_source_stream(Dims d, SourcePara
             const float xx = 1.f + h.xx, yy = 1.f + h.yy, zz = 1.f + h.zz;
             const float big = fmaxf(fmaxf(fabsf(xx), fabsf(yy)), fabsf(zz));
             const float eps = 32.0f * kU * h.vmax + 4.0f * kU * (big + 1.0f);
+            const float mixed = fmaxf(fabsf(h.xy), fmaxf(fabsf(h.xz), fabsf(h.yz)));
+            wide |= !(fmaxf(big, 4.f * mixed) + 4.f * eps < 448.f);
             const bool plain = sp.climiter != 1 && sylvester32(xx, yy, zz, h.xy, h.xz, h.yz, xi, eps) > 0 &&
                                (xx + yy) + zz + 4.f * eps < trace_max;
             if (plain) {
@@ -237,12 +243,14 @@ __global__ void __launch_bounds__(GT, GPERSM) k_source_stream(Dims d, SourcePara
         });
     while (todo.n > 0) exact();
     s = block_reduce<OpSum>(s);
-    if (threadIdx.x == 0) put_partial(psum, s, kRedBlocks);
+    const int any = __syncthreads_or(wide);
+    if (threadIdx.x == 0) put_partial(psum, s, kRedBlocks), put_partial(pwide, any ? 1.0 : 0.0, kRedBlocks);
 }
 
 // Any grid, every node in FP64.
 __global__ void k_source_node(Dims d, SourceParams sp, const double* __restrict__ phi,
-                              const double* __restrict__ m, double* __restrict__ t, double* __restrict__ psum) {
+                              const double* __restrict__ m, double* __restrict__ t, double* __restrict__ psum,
+                              double* __restrict__ pwide) {
     double s = 0.0;
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells; c += gridDim.x * blockDim.x) {
         const double v = source64(d, sp, phi, m, c);
@@ -250,7 +258,8 @@ __global__ void k_source_node(Dims d, SourceParams sp, const double* __restrict_
         s += v;
     }
     s = block_reduce<OpSum>(s);
-    if (threadIdx.x == 0) psum[blockIdx.x] = s;
+    // (the displacements of these grids are FP64)
+    if (threadIdx.x == 0) psum[blockIdx.x] = s, pwide[blockIdx.x] = 1.0;
 }
 
 // Step limiter at one node in FP64: the smallest k in [0, kmax] with
@@ -526,15 +535,15 @@ int tile_k(const Dims& d) {
 }  // namespace
 
 void launch_source(const Dims& d, const SourceParams& sp, const double* phi, const float* phi32, const double* m,
-                   double* t, double* part_sum, cudaStream_t st) {
+                   double* t, double* part_sum, double* part_wide, cudaStream_t st) {
     launch_counter()++;
     if (const int tk = tile_k(d)) {
         const float trace_max = (float)(3.0 * cbrt(sp.v_m) * (1.0 - 1e-5));
         auto fn = tk == 32 ? k_source_stream<32> : k_source_stream<16>;
-        fn<<<GBLOCKS, GT, 0, st>>>(d, sp, trace_max, phi, phi32, m, t, part_sum);
+        fn<<<GBLOCKS, GT, 0, st>>>(d, sp, trace_max, phi, phi32, m, t, part_sum, part_wide);
         return;
     }
-    k_source_node<<<kRedBlocks, kRedThreads, 0, st>>>(d, sp, phi, m, t, part_sum);
+    k_source_node<<<kRedBlocks, kRedThreads, 0, st>>>(d, sp, phi, m, t, part_sum, part_wide);
 }
 
 void launch_limiter(const Dims& d, const LimiterParams& lp, const double* phi, const double* dphi,

@@ -294,12 +294,11 @@ __global__ void k_mass_coef(int cells, unsigned long long* __restrict__ mfix, do
 __global__ void k_smooth_axis(Dims d, int axis, double ws, const double* __restrict__ in,
                               const double* __restrict__ shift_sum, double* __restrict__ out,
                               float* __restrict__ out32, double* __restrict__ psum,
-                              double* __restrict__ pmax, double* __restrict__ psq) {
+                              double* __restrict__ psq) {
     const double w1 = 1.0 - 2.0 * ws;
     const double shift = shift_sum ? *shift_sum / (double)d.cells : 0.0;
     const int di = axis == 0, dj = axis == 1, dk = axis == 2;
     double s = 0.0, q = 0.0;
-    float mx = 0.f;
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells; c += gridDim.x * blockDim.x) {
         int i, j, k;
         cell_coords(d, c, i, j, k);
@@ -308,13 +307,8 @@ __global__ void k_smooth_axis(Dims d, int axis, double ws, const double* __restr
                              w1 * in[c]) - shift;
         out[c] = v;
         if (out32) out32[c] = (float)v;
-        mx = fmaxf(mx, fabsf((float)v));
         s += v;
         q = fma(v, v, q);
-    }
-    if (pmax) {
-        const double v = block_reduce<OpMax>((double)mx);
-        if (threadIdx.x == 0) pmax[blockIdx.x] = v;
     }
     if (psum) {
         s = block_reduce<OpSum>(s);
@@ -338,8 +332,8 @@ __global__ void k_smooth_axis(Dims d, int axis, double ws, const double* __restr
 //
 // Bound by the FP64 rate (2 lanes a clock and SM).  QUARTER (side weight 1/4,
 // the default): a + 2 b + c per axis and one exact factor 1/64 at the end, 2
-// instructions an axis instead of 3.  SUM: the FP32 copy, the sum and the
-// largest magnitude (of the FP32 copy); SQ: the sum of squares.  512^3: 3.87 -> 2.87 ms (FP64 pipe 72% busy), 32^3 (8 blocks in the
+// instructions an axis instead of 3.  SUM: the FP32 copy and the sum; SQ: the
+// sum of squares.  512^3: 3.87 -> 2.87 ms (FP64 pipe 72% busy), 32^3 (8 blocks in the
 // former split): 36.5 -> 9.8 us.
 constexpr int SJ = 8, SK = 32;
 constexpr int kSPerSM = 6, kSBlocks = kSPerSM * (kRedBlocks / 8);
@@ -347,7 +341,7 @@ constexpr int kSPerSM = 6, kSBlocks = kSPerSM * (kRedBlocks / 8);
 template <bool QUARTER, bool SUM, bool SQ>
 __global__ void __launch_bounds__(SJ* SK, kSPerSM) k_smooth_S_stream(
     Dims d, double ws, const double* __restrict__ in, const double* __restrict__ shift_sum,
-    double* __restrict__ out, float* __restrict__ out32, double* __restrict__ part, double* __restrict__ pmax) {
+    double* __restrict__ out, float* __restrict__ out32, double* __restrict__ part) {
     __shared__ double sk[2][SJ + 2][SK];  // planes smoothed along k
     const double w1 = 1.0 - 2.0 * ws;
     const double shift = shift_sum ? *shift_sum * inv_pow2(d.cells) : 0.0;
@@ -377,7 +371,6 @@ __global__ void __launch_bounds__(SJ* SK, kSPerSM) k_smooth_S_stream(
     long long at = planes * blockIdx.x / gridDim.x;
     const long long end = planes * (blockIdx.x + 1) / gridDim.x;
     double acc = 0.0;
-    float mx = 0.f;
     while (at < end) {
         const int col = (int)(at / d.n0), i0 = (int)(at % d.n0);
         const int i1 = (int)min((long long)d.n0, i0 + (end - at));
@@ -406,7 +399,6 @@ __global__ void __launch_bounds__(SJ* SK, kSPerSM) k_smooth_S_stream(
                 out[e] = o;
                 if (SUM) {
                     out32[e] = (float)o;
-                    mx = fmaxf(mx, fabsf((float)o));
                     acc += o;
                 }
                 if (SQ) acc = fma(o, o, acc);
@@ -419,21 +411,17 @@ __global__ void __launch_bounds__(SJ* SK, kSPerSM) k_smooth_S_stream(
         acc = block_reduce<OpSum>(acc);
         if (threadIdx.x == 0) put_partial(part, acc, kRedBlocks);
     }
-    if (SUM) {
-        const double v = block_reduce<OpMax>((double)mx);
-        if (threadIdx.x == 0) put_partial(pmax, v, kRedBlocks);
-    }
 }
 
 template <bool QUARTER>
 void launch_smooth_stream(const Dims& d, double ws, const double* in, const double* shift_sum, double* out,
-                          float* out32, double* part_sum, double* part_max, double* part_sq, cudaStream_t st) {
+                          float* out32, double* part_sum, double* part_sq, cudaStream_t st) {
     if (part_sum)
-        k_smooth_S_stream<QUARTER, true, false><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, part_sum, part_max);
+        k_smooth_S_stream<QUARTER, true, false><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, part_sum);
     else if (part_sq)
-        k_smooth_S_stream<QUARTER, false, true><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, part_sq, part_max);
+        k_smooth_S_stream<QUARTER, false, true><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, part_sq);
     else
-        k_smooth_S_stream<QUARTER, false, false><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, nullptr, part_max);
+        k_smooth_S_stream<QUARTER, false, false><<<kSBlocks, SJ * SK, 0, st>>>(d, ws, in, shift_sum, out, out32, nullptr);
 }
 
 // V = e^-1 G at every node: e = I + Hess phi (before the step; stored by
@@ -714,21 +702,21 @@ void launch_mass_coef(int cells, unsigned long long* mfix, double inv_scale, dou
 }
 
 void launch_smooth_S(const Dims& d, double s_side, const double* in, const double* shift_sum,
-                     double* out, float* out32, double* tmp2, double* part_sum, double* part_max,
-                     double* part_sq, cudaStream_t st) {
+                     double* out, float* out32, double* tmp2, double* part_sum, double* part_sq,
+                     cudaStream_t st) {
     if (d.n2 % SK == 0 && d.n1 % SJ == 0 && !(part_sum && part_sq)) {
         launch_counter()++;
         auto launch = s_side == 0.25 ? launch_smooth_stream<true> : launch_smooth_stream<false>;
-        launch(d, s_side, in, shift_sum, out, out32, part_sum, part_max, part_sq, st);
+        launch(d, s_side, in, shift_sum, out, out32, part_sum, part_sq, st);
         return;
     }
     launch_counter() += 3;
     k_smooth_axis<<<kRedBlocks, kRedThreads, 0, st>>>(d, 2, s_side, in, nullptr, tmp2, nullptr,
-                                                      nullptr, nullptr, nullptr);
+                                                      nullptr, nullptr);
     k_smooth_axis<<<kRedBlocks, kRedThreads, 0, st>>>(d, 1, s_side, tmp2, nullptr,
-                                                      tmp2 + d.cells, nullptr, nullptr, nullptr, nullptr);
+                                                      tmp2 + d.cells, nullptr, nullptr, nullptr);
     k_smooth_axis<<<kRedBlocks, kRedThreads, 0, st>>>(d, 0, s_side, tmp2 + d.cells, shift_sum,
-                                                      out, out32, part_sum, part_max, part_sq);
+                                                      out, out32, part_sum, part_sq);
 }
 
 void launch_node_velocity(const Dims& d, const double* e6, const double* dphi, double* vx,
