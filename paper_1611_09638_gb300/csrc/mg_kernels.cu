@@ -106,47 +106,53 @@ __global__ void k_residual64(Dims d, const double* __restrict__ u, const double*
 // Optionally also writes r in FP32 (the next V-cycle's right-hand side);
 // always the per-block partial sums of r^2.  With the FP32 copy (mixed mode)
 // r^2 is summed from it on the FP32 pipe, one FP64 instruction fewer per
-// node.  The norm only decides the multigrid stopping test: each thread's
-// FP32 sum covers cells / (kRedBlocks * kRedThreads) nodes (54 at 256^3, 431
-// at 512^3), so its relative error stays below ~3e-5, and the block sums
-// are FP64.  One round of four blocks per SM with 59 registers, so that a
+// node.  The norm only decides the multigrid stopping test: a thread's FP32
+// sum goes into its FP64 one every kRes32 nodes, so its relative error stays
+// below kRes32 2^-24 = 4e-6 on every grid, and the block sums are FP64.  One
+// round of four blocks per SM with 62 registers, so that a
 // node's fifteen loads are all in flight: 512^3 2.19 -> 1.98 ms, 256^3 274 -> 254
 // us against 38 registers in kRedBlocks blocks (eight FP64 instructions at 2
 // lanes a clock and SM take 1.71 ms; rounding the FP32 copy by integer
 // instructions instead took 2.3 ms).
+constexpr int kRes32 = 64;
 constexpr int kResPerSM = 4, kResBlocks = kResPerSM * (kRedBlocks / 8);
 __global__ void __launch_bounds__(kRedThreads, kResPerSM) k_residual64_to32(Dims d, const double* __restrict__ u,
                                   const double* __restrict__ f, const double* __restrict__ F,
                                   const double* __restrict__ D, float* __restrict__ r32,
                                   double* __restrict__ partials) {
     double acc = 0.0;
-    float acc32 = 0.f;
     const size_t n = (size_t)d.cells;
     const double* __restrict__ Fx = F;
     const double* __restrict__ Fy = F + n;
     const double* __restrict__ Fz = F + 2 * n;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells; c += gridDim.x * blockDim.x) {
-        int i, j, k;
-        cell_coords(d, c, i, j, k);
-        const int n0 = cell_index(d, i + 1, j, k), n1 = cell_index(d, i - 1, j, k);
-        const int n2 = cell_index(d, i, j + 1, k), n3 = cell_index(d, i, j - 1, k);
-        const int n4 = cell_index(d, i, j, k + 1), n5 = cell_index(d, i, j, k - 1);
-        double r = fma(D[c], u[c], f[c]);
-        r = fma(-Fx[c], u[n0], r);
-        r = fma(-Fx[n1], u[n1], r);
-        r = fma(-Fy[c], u[n2], r);
-        r = fma(-Fy[n3], u[n3], r);
-        r = fma(-Fz[c], u[n4], r);
-        r = fma(-Fz[n5], u[n5], r);
-        if (r32) {
-            const float rf = (float)r;
-            r32[c] = rf;
-            acc32 = fmaf(rf, rf, acc32);
-        } else {
-            acc = fma(r, r, acc);
+    const int stride = gridDim.x * blockDim.x;
+    // (a loop of its own for the nodes of an FP32 sum: with the test inside one
+    // loop the loads of several nodes are not in flight together, 256^3 solves 3% slower)
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells;) {
+        float acc32 = 0.f;
+        for (const int stop = min(d.cells, c + kRes32 * stride); c < stop; c += stride) {
+            int i, j, k;
+            cell_coords(d, c, i, j, k);
+            const int n0 = cell_index(d, i + 1, j, k), n1 = cell_index(d, i - 1, j, k);
+            const int n2 = cell_index(d, i, j + 1, k), n3 = cell_index(d, i, j - 1, k);
+            const int n4 = cell_index(d, i, j, k + 1), n5 = cell_index(d, i, j, k - 1);
+            double r = fma(D[c], u[c], f[c]);
+            r = fma(-Fx[c], u[n0], r);
+            r = fma(-Fx[n1], u[n1], r);
+            r = fma(-Fy[c], u[n2], r);
+            r = fma(-Fy[n3], u[n3], r);
+            r = fma(-Fz[c], u[n4], r);
+            r = fma(-Fz[n5], u[n5], r);
+            if (r32) {
+                const float rf = (float)r;
+                r32[c] = rf;
+                acc32 = fmaf(rf, rf, acc32);
+            } else {
+                acc = fma(r, r, acc);
+            }
         }
+        acc += (double)acc32;
     }
-    acc += (double)acc32;
     acc = block_reduce<OpSum>(acc);
     if (threadIdx.x == 0) put_partial(partials, acc, kRedBlocks);
 }
