@@ -188,17 +188,14 @@ __device__ __noinline__ double source64(const Dims& d, const SourceParams& sp, c
 
 // C = E = 0 where FP32 certifies that every eigenvalue of e exceeds xi_m
 // (Sylvester's criterion) and, e being positive definite then, that its trace
-// stays below 3 v_m^(1/3) (det e <= (tr e / 3)^3).  pwide: 1 where a second
-// difference of phi, or four times a mixed one, may reach 448 (or is not finite);
-// the displacements of the step know them modulo 1024 only.
+// stays below 3 v_m^(1/3) (det e <= (tr e / 3)^3).
 template <int GK>
 __global__ void __launch_bounds__(GT, GPERSM) k_source_stream(Dims d, SourceParams sp, float trace_max,
                                                                   const double* __restrict__ phi,
                                                                   const float* __restrict__ phi32,
                                                                   const double* __restrict__ m,
                                                                   double* __restrict__ t,
-                                                                  double* __restrict__ psum,
-                                                                  double* __restrict__ pwide) {
+                                                                  double* __restrict__ psum) {
     constexpr int GPK = Tile<GK>::PK;
     __shared__ float buf[2][1][Tile<GK>::N];
     __shared__ int list[GT / 32][64];
@@ -208,7 +205,6 @@ __global__ void __launch_bounds__(GT, GPERSM) k_source_stream(Dims d, SourcePara
     WarpList todo{list[threadIdx.x / 32], 0};
     Column32<GPK> col{};
     double s = 0.0;
-    bool wide = false;
     auto exact = [&] {
         const int c = todo.take();
         if (c >= 0) {
@@ -229,8 +225,6 @@ __global__ void __launch_bounds__(GT, GPERSM) k_source_stream(Dims d, SourcePara
             const float xx = 1.f + h.xx, yy = 1.f + h.yy, zz = 1.f + h.zz;
             const float big = fmaxf(fmaxf(fabsf(xx), fabsf(yy)), fabsf(zz));
             const float eps = 32.0f * kU * h.vmax + 4.0f * kU * (big + 1.0f);
-            const float mixed = fmaxf(fabsf(h.xy), fmaxf(fabsf(h.xz), fabsf(h.yz)));
-            wide |= !(fmaxf(big, 4.f * mixed) + 4.f * eps < 448.f);
             const bool plain = sp.climiter != 1 && sylvester32(xx, yy, zz, h.xy, h.xz, h.yz, xi, eps) > 0 &&
                                (xx + yy) + zz + 4.f * eps < trace_max;
             if (plain) {
@@ -243,14 +237,12 @@ __global__ void __launch_bounds__(GT, GPERSM) k_source_stream(Dims d, SourcePara
         });
     while (todo.n > 0) exact();
     s = block_reduce<OpSum>(s);
-    const int any = __syncthreads_or(wide);
-    if (threadIdx.x == 0) put_partial(psum, s, kRedBlocks), put_partial(pwide, any ? 1.0 : 0.0, kRedBlocks);
+    if (threadIdx.x == 0) put_partial(psum, s, kRedBlocks);
 }
 
 // Any grid, every node in FP64.
 __global__ void k_source_node(Dims d, SourceParams sp, const double* __restrict__ phi,
-                              const double* __restrict__ m, double* __restrict__ t, double* __restrict__ psum,
-                              double* __restrict__ pwide) {
+                              const double* __restrict__ m, double* __restrict__ t, double* __restrict__ psum) {
     double s = 0.0;
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells; c += gridDim.x * blockDim.x) {
         const double v = source64(d, sp, phi, m, c);
@@ -258,8 +250,7 @@ __global__ void k_source_node(Dims d, SourceParams sp, const double* __restrict_
         s += v;
     }
     s = block_reduce<OpSum>(s);
-    // (the displacements of these grids are FP64)
-    if (threadIdx.x == 0) psum[blockIdx.x] = s, pwide[blockIdx.x] = 1.0;
+    if (threadIdx.x == 0) psum[blockIdx.x] = s;
 }
 
 // Step limiter at one node in FP64: the smallest k in [0, kmax] with
@@ -289,13 +280,106 @@ __device__ inline double gradient64(const Dims& d, const double* __restrict__ dp
     return fmax(fabs(gx), fmax(fabs(gy), fabs(gz)));
 }
 
+// The Hessian of an FP32 field at one node (Column32's values from memory) and
+// twice its gradient.
+__device__ inline Hess32 hess32_at(const Dims& d, const float* __restrict__ f, int i, int j, int k, float& gx,
+                                   float& gy, float& gz) {
+    auto at = [&](int a, int b, int c) { return f[cell_index(d, i + a, j + b, k + c)]; };
+    Hess32 h;
+    const float c = at(0, 0, 0);
+    h.vmax = fabsf(c);
+    auto second = [&](float p, float m, float& g) {
+        h.vmax = fmaxf(h.vmax, fmaxf(fabsf(p), fabsf(m)));
+        g = p - m;
+        return (p - 2.f * c) + m;
+    };
+    auto mixed = [&](float pp, float pm, float mp, float mm) {
+        h.vmax = fmaxf(fmaxf(h.vmax, fmaxf(fabsf(pp), fabsf(pm))), fmaxf(fabsf(mp), fabsf(mm)));
+        return 0.25f * ((pp - pm) - (mp - mm));
+    };
+    h.xx = second(at(1, 0, 0), at(-1, 0, 0), gx);
+    h.yy = second(at(0, 1, 0), at(0, -1, 0), gy);
+    h.zz = second(at(0, 0, 1), at(0, 0, -1), gz);
+    h.xy = mixed(at(1, 1, 0), at(1, -1, 0), at(-1, 1, 0), at(-1, -1, 0));
+    h.xz = mixed(at(1, 0, 1), at(1, 0, -1), at(-1, 0, 1), at(-1, 0, -1));
+    h.yz = mixed(at(0, 1, 1), at(0, 1, -1), at(0, -1, 1), at(0, -1, -1));
+    return h;
+}
+
 // Step limiter: the largest over the nodes of the smallest k in [0, kmax] with
 // lambda_min(e + 2^-k Hess dphi) > floor (kmax + 1 if none), and max_a |central
 // grad_a dphi|.  A node that passes at the largest k its warp has found so far
 // does not change the result, and where it fails FP32 finds its own k, unless a
 // verdict on the way is open (then the FP64 form does).  The gradient's maximum is FP64 too: a node
 // is evaluated only where FP32 does not show it to be below the largest value
-// its warp has found.
+// its warp has found.  wide: a second difference of phi, or four times a mixed
+// one, may reach 448 (or is not finite); the displacements of the step know them
+// modulo 1024 only.  Every lane of a warp takes part in each call.
+struct LimiterScreen {
+    int kk = 0;            // the warp's largest k so far, and 2^-kk
+    float al = 1.f;
+    double gm = 0.0;       // this lane's largest |2 G|
+    float gw = 0.f;        // the warp's, rounded down
+    bool wide = false;
+
+    __device__ __forceinline__ void raise(int k) {
+        kk = max(kk, __reduce_max_sync(0xffffffffu, k));
+        al = kk < 126 ? __int_as_float((127 - kk) << 23) : 0.f;
+    }
+    // g: FP32's largest |difference| (within 8 u vmax of the FP64 one, exact())
+    template <typename Exact>
+    __device__ __forceinline__ void gradient(float g, float vmax, Exact&& exact) {
+        const bool higher = !(g + 8.f * kU * vmax < gw);
+        if (__any_sync(0xffffffffu, higher)) {
+            if (higher) gm = fmax(gm, exact());
+            float f = __double2float_rd(gm);
+            for (int o = 16; o > 0; o >>= 1) f = fmaxf(f, __shfl_xor_sync(0xffffffffu, f, o));
+            gw = f;
+        }
+    }
+    // a node's Hessians of phi and dphi; returns whether the FP64 form has to
+    // find its k
+    __device__ __forceinline__ bool node(const LimiterParams& lp, float floor32, const Hess32& a, const Hess32& b) {
+        const float diag = fmaxf(fabsf(a.xx), fmaxf(fabsf(a.yy), fabsf(a.zz)));
+        const float mixed = fmaxf(fabsf(a.xy), fmaxf(fabsf(a.xz), fabsf(a.yz)));
+        wide |= !(fmaxf(diag, 4.f * mixed) + 128.f * kU * a.vmax < 448.f);
+        // FP32's verdict at step length l: the entries' error is that of
+        // the inputs and Hessians, then of the two additions forming M
+        auto verdict = [&](float l) {
+            const float mxx = 1.0f + a.xx + l * b.xx, myy = 1.0f + a.yy + l * b.yy;
+            const float mzz = 1.0f + a.zz + l * b.zz, mxy = a.xy + l * b.xy;
+            const float mxz = a.xz + l * b.xz, myz = a.yz + l * b.yz;
+            const float big = fmaxf(fmaxf(fabsf(mxx), fabsf(myy)),
+                                    fmaxf(fabsf(mzz), fmaxf(fabsf(mxy), fmaxf(fabsf(mxz), fabsf(myz)))));
+            const float eps = 32.0f * kU * (a.vmax + l * b.vmax) + 4.0f * kU * (big + 1.0f);
+            return sylvester32(mxx, myy, mzz, mxy, mxz, myz, floor32, eps);
+        };
+        bool unsure = false;
+        if (kk <= lp.kmax) {
+            const bool passes = verdict(al) > 0;
+            if (__any_sync(0xffffffffu, !passes)) {
+                int k = 0;
+                if (!passes) {  // the node's own k, as far as FP32 tells
+                    float l = 1.f;
+                    int v = -1;
+                    for (; k <= lp.kmax && (v = verdict(l)) < 0; ++k) l *= 0.5f;
+                    unsure = v == 0;
+                }
+                raise(unsure ? 0 : k);
+            }
+        }
+        return unsure;
+    }
+    // the block's partials (threads of a block: blockDim.x)
+    __device__ __forceinline__ void put(double* pk, double* pg, double* pw) {
+        const double k = block_reduce<OpMax>((double)kk);
+        const double g = block_reduce<OpMax>(0.5 * gm);
+        const int w = __syncthreads_or(wide);
+        if (threadIdx.x == 0)
+            put_partial(pk, k, kRedBlocks), put_partial(pg, g, kRedBlocks), put_partial(pw, w ? 1.0 : 0.0, kRedBlocks);
+    }
+};
+
 template <int GK>
 __global__ void __launch_bounds__(GT, GPERSM) k_limiter_stream(Dims d, LimiterParams lp,
                                                                    const double* __restrict__ phi,
@@ -303,7 +387,8 @@ __global__ void __launch_bounds__(GT, GPERSM) k_limiter_stream(Dims d, LimiterPa
                                                                    const float* __restrict__ phi32,
                                                                    const float* __restrict__ dphi32,
                                                                    double* __restrict__ pk,
-                                                                   double* __restrict__ pg) {
+                                                                   double* __restrict__ pg,
+                                                                   double* __restrict__ pw) {
     constexpr int GPK = Tile<GK>::PK;
     __shared__ float buf[2][2][Tile<GK>::N];
     __shared__ int list[GT / 32][64];
@@ -312,15 +397,10 @@ __global__ void __launch_bounds__(GT, GPERSM) k_limiter_stream(Dims d, LimiterPa
     const float floor32 = (float)lp.lambda_floor;
     WarpList todo{list[threadIdx.x / 32], 0};
     Column32<GPK> A{}, B{};
-    int kk = 0;            // the warp's largest k so far, and 2^-kk
-    float al = 1.f;
-    double gm = 0.0;       // this lane's largest |2 G|
-    float gw = 0.f;        // the warp's, rounded down
+    LimiterScreen screen;
     auto exact = [&] {
         const int c = todo.take();
-        const int k = c >= 0 ? limiter64(d, lp, phi, dphi, c) : 0;
-        kk = max(kk, __reduce_max_sync(0xffffffffu, k));
-        al = kk < 126 ? __int_as_float((127 - kk) << 23) : 0.f;
+        screen.raise(c >= 0 ? limiter64(d, lp, phi, dphi, c) : 0);
     };
     const float* const fields[2] = {phi32, dphi32};
     stream_planes<GK, 2>(
@@ -331,65 +411,36 @@ __global__ void __launch_bounds__(GT, GPERSM) k_limiter_stream(Dims d, LimiterPa
             const Hess32 b = B.feed(buf[w][1] + own, gy, gz);
             if (!done) return;
             const int c = cell_index(d, p - 1, j0 + lj, k0 + lk);
-            // the FP32 differences are within 8 u vmax of the FP64 ones
             const float g = fmaxf(fabsf(B.gx), fmaxf(fabsf(gy), fabsf(gz)));
-            const bool higher = !(g + 8.f * kU * b.vmax < gw);
-            if (__any_sync(0xffffffffu, higher)) {
-                if (higher) gm = fmax(gm, gradient64(d, dphi, p - 1, j0 + lj, k0 + lk));
-                float f = __double2float_rd(gm);
-                for (int o = 16; o > 0; o >>= 1) f = fmaxf(f, __shfl_xor_sync(0xffffffffu, f, o));
-                gw = f;
-            }
-            // FP32's verdict at step length l: the entries' error is that of
-            // the inputs and Hessians, then of the two additions forming M
-            auto verdict = [&](float l) {
-                const float mxx = 1.0f + a.xx + l * b.xx, myy = 1.0f + a.yy + l * b.yy;
-                const float mzz = 1.0f + a.zz + l * b.zz, mxy = a.xy + l * b.xy;
-                const float mxz = a.xz + l * b.xz, myz = a.yz + l * b.yz;
-                const float big = fmaxf(fmaxf(fabsf(mxx), fabsf(myy)),
-                                        fmaxf(fabsf(mzz), fmaxf(fabsf(mxy), fmaxf(fabsf(mxz), fabsf(myz)))));
-                const float eps = 32.0f * kU * (a.vmax + l * b.vmax) + 4.0f * kU * (big + 1.0f);
-                return sylvester32(mxx, myy, mzz, mxy, mxz, myz, floor32, eps);
-            };
-            bool unsure = false;
-            if (kk <= lp.kmax) {
-                const bool passes = verdict(al) > 0;
-                if (__any_sync(0xffffffffu, !passes)) {
-                    int k = 0;
-                    if (!passes) {  // the node's own k, as far as FP32 tells
-                        float l = 1.f;
-                        int v = -1;
-                        for (; k <= lp.kmax && (v = verdict(l)) < 0; ++k) l *= 0.5f;
-                        unsure = v == 0;
-                    }
-                    kk = max(kk, __reduce_max_sync(0xffffffffu, unsure ? 0 : k));
-                    al = kk < 126 ? __int_as_float((127 - kk) << 23) : 0.f;
-                }
-            }
-            todo.add(unsure, c);
+            screen.gradient(g, b.vmax, [&] { return gradient64(d, dphi, p - 1, j0 + lj, k0 + lk); });
+            todo.add(screen.node(lp, floor32, a, b), c);
             if (todo.n >= 32) exact();
         });
     while (todo.n > 0) exact();
-    const double k = block_reduce<OpMax>((double)kk);
-    const double g = block_reduce<OpMax>(0.5 * gm);
-    if (threadIdx.x == 0) put_partial(pk, k, kRedBlocks), put_partial(pg, g, kRedBlocks);
+    screen.put(pk, pg, pw);
 }
 
-// Any grid, every node in FP64.
+// Any grid, a thread a node from memory (whole warps have nodes or none: the
+// cells are a multiple of 32).  1024 x 512 x 8: 577 us with the FP64 form at
+// every node, 66 with this screen.
 __global__ void k_limiter_node(Dims d, LimiterParams lp, const double* __restrict__ phi,
-                               const double* __restrict__ dphi, double* __restrict__ pk,
-                               double* __restrict__ pg) {
-    double kk = 0.0, gm = 0.0;
+                               const double* __restrict__ dphi, const float* __restrict__ phi32,
+                               const float* __restrict__ dphi32, double* __restrict__ pk,
+                               double* __restrict__ pg, double* __restrict__ pw) {
+    const float floor32 = (float)lp.lambda_floor;
+    LimiterScreen screen;
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells; c += gridDim.x * blockDim.x) {
         int i, j, k;
         cell_coords(d, c, i, j, k);
-        gm = fmax(gm, gradient64(d, dphi, i, j, k));
-        kk = fmax(kk, (double)limiter64(d, lp, phi, dphi, c));
+        float gx, gy, gz, ax, ay, az;
+        const Hess32 a = hess32_at(d, phi32, i, j, k, ax, ay, az);
+        const Hess32 b = hess32_at(d, dphi32, i, j, k, gx, gy, gz);
+        screen.gradient(fmaxf(fabsf(gx), fmaxf(fabsf(gy), fabsf(gz))), b.vmax,
+                        [&] { return gradient64(d, dphi, i, j, k); });
+        const bool unsure = screen.node(lp, floor32, a, b);
+        if (__any_sync(0xffffffffu, unsure)) screen.raise(unsure ? limiter64(d, lp, phi, dphi, c) : 0);
     }
-    kk = block_reduce<OpMax>(kk);
-    if (threadIdx.x == 0) pk[blockIdx.x] = kk;
-    gm = block_reduce<OpMax>(0.5 * gm);
-    if (threadIdx.x == 0) pg[blockIdx.x] = gm;
+    screen.put(pk, pg, pw);
 }
 
 // The outputs of one node in FP64.  Not inlined, so that the fields and the
@@ -535,27 +586,28 @@ int tile_k(const Dims& d) {
 }  // namespace
 
 void launch_source(const Dims& d, const SourceParams& sp, const double* phi, const float* phi32, const double* m,
-                   double* t, double* part_sum, double* part_wide, cudaStream_t st) {
+                   double* t, double* part_sum, cudaStream_t st) {
     launch_counter()++;
     if (const int tk = tile_k(d)) {
         const float trace_max = (float)(3.0 * cbrt(sp.v_m) * (1.0 - 1e-5));
         auto fn = tk == 32 ? k_source_stream<32> : k_source_stream<16>;
-        fn<<<GBLOCKS, GT, 0, st>>>(d, sp, trace_max, phi, phi32, m, t, part_sum, part_wide);
+        fn<<<GBLOCKS, GT, 0, st>>>(d, sp, trace_max, phi, phi32, m, t, part_sum);
         return;
     }
-    k_source_node<<<kRedBlocks, kRedThreads, 0, st>>>(d, sp, phi, m, t, part_sum, part_wide);
+    k_source_node<<<kRedBlocks, kRedThreads, 0, st>>>(d, sp, phi, m, t, part_sum);
 }
 
 void launch_limiter(const Dims& d, const LimiterParams& lp, const double* phi, const double* dphi,
                     const float* phi32, const float* dphi32, double* part_k, double* part_g,
-                    cudaStream_t st) {
+                    double* part_wide, cudaStream_t st) {
     launch_counter()++;
     if (const int tk = tile_k(d)) {
         auto fn = tk == 32 ? k_limiter_stream<32> : k_limiter_stream<16>;
-        fn<<<GBLOCKS, GT, 0, st>>>(d, lp, phi, dphi, phi32, dphi32, part_k, part_g);
+        fn<<<GBLOCKS, GT, 0, st>>>(d, lp, phi, dphi, phi32, dphi32, part_k, part_g, part_wide);
         return;
     }
-    k_limiter_node<<<kRedBlocks, kRedThreads, 0, st>>>(d, lp, phi, dphi, part_k, part_g);
+    k_limiter_node<<<kRedBlocks, kRedThreads, 0, st>>>(d, lp, phi, dphi, phi32, dphi32, part_k, part_g,
+                                                       part_wide);
 }
 
 void launch_delta_r(const Dims& d, const double* phi, double* out, double* part_max,
