@@ -3,8 +3,8 @@
 //     L u = sum_a h_a^-2 [A+ (u+ - u) - A- (u - u-)],  A+- = (a + a+-) / 2,
 // red-black Gauss-Seidel smoothing (red = (i+j+k) even first), residual,
 // full-weighting restriction, trilinear prolongation, and a dense solve of the
-// 4^3 coarsest level with the mean constraint.  Templated on float (mixed mode)
-// and double.
+// 4^3 coarsest level with the mean constraint, for the FP32 levels (mixed mode)
+// and the FP64 ones.
 #include "mg_stencil.cuh"
 #include "recon_internal.cuh"
 #include "reduce.cuh"
@@ -19,9 +19,8 @@ inline int nblocks(long long work) { return (int)((work + kThreads - 1) / kThrea
 
 // One colour of a red-black Gauss-Seidel sweep; thread t owns the t-th node
 // of that colour (nodes of a colour alternate along the fastest axis).
-template <typename T>
-__global__ void k_rbgs_colour(Dims d, T hx, T hy, T hz, int colour, T* __restrict__ u,
-                              const T* __restrict__ f, const T* __restrict__ a, int face) {
+__global__ void k_rbgs_colour(Dims d, float hx, float hy, float hz, int colour, float* __restrict__ u,
+                              const float* __restrict__ f, const float* __restrict__ a, int face) {
     const int half = d.cells >> 1;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= half) return;
@@ -31,7 +30,7 @@ __global__ void k_rbgs_colour(Dims d, T hx, T hy, T hz, int colour, T* __restric
     const int i = t >> (d.s1 + hs2);
     const int k = 2 * kk + ((i + j + colour) & 1);
     const int c = cell_index(d, i, j, k);
-    Stencil7<T> s = stencil7_any<T>(d, hx, hy, hz, i, j, k, c, u, a, face);
+    Stencil7 s = stencil7_any(d, hx, hy, hz, i, j, k, c, u, a, face);
     u[c] = (s.off - f[c]) / s.diag;
 }
 
@@ -193,21 +192,20 @@ __global__ void k_faces64(Dims d, int ex, int ey, int ez, const double* __restri
 }
 
 // Full weighting: weights (1/4, 1/2, 1/4) along every coarsened axis.
-template <typename T>
-__global__ void k_restrict(Dims df, Dims dc, int cx, int cy, int cz, const T* __restrict__ in,
-                           T* __restrict__ out) {
+__global__ void k_restrict(Dims df, Dims dc, int cx, int cy, int cz, const float* __restrict__ in,
+                           float* __restrict__ out) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= dc.cells) return;
     int I, J, K;
     cell_coords(dc, c, I, J, K);
     const int fi = cx ? 2 * I : I, fj = cy ? 2 * J : J, fk = cz ? 2 * K : K;
-    T acc = T(0);
+    float acc = 0.f;
     for (int oi = -cx; oi <= cx; ++oi) {
-        const T wi = cx ? (oi == 0 ? T(0.5) : T(0.25)) : T(1);
+        const float wi = cx ? (oi == 0 ? 0.5f : 0.25f) : 1.f;
         for (int oj = -cy; oj <= cy; ++oj) {
-            const T wj = cy ? (oj == 0 ? T(0.5) : T(0.25)) : T(1);
+            const float wj = cy ? (oj == 0 ? 0.5f : 0.25f) : 1.f;
             for (int ok = -cz; ok <= cz; ++ok) {
-                const T wk = cz ? (ok == 0 ? T(0.5) : T(0.25)) : T(1);
+                const float wk = cz ? (ok == 0 ? 0.5f : 0.25f) : 1.f;
                 acc += wi * wj * wk * in[cell_index(df, fi + oi, fj + oj, fk + ok)];
             }
         }
@@ -246,28 +244,27 @@ __global__ void k_restrict64(Dims df, Dims dc, int cx, int cy, int cz, const dou
 // stored): per node the 7-point residual f - L u followed by the full weighting.
 // red: u has just been swept, so black nodes have none (but for rounding) and
 // are left out, half the evaluations (128 x 64 x 32 nodes: 8.5 -> 7.2 us a level).
-template <typename T>
-__global__ void k_resid_restrict(Dims df, Dims dc, int cx, int cy, int cz, T hx, T hy, T hz,
-                                 const T* __restrict__ u, const T* __restrict__ f,
-                                 const T* __restrict__ a, int face, int red, T* __restrict__ out) {
+__global__ void k_resid_restrict(Dims df, Dims dc, int cx, int cy, int cz, float hx, float hy, float hz,
+                                 const float* __restrict__ u, const float* __restrict__ f,
+                                 const float* __restrict__ a, int face, int red, float* __restrict__ out) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= dc.cells) return;
     int I, J, K;
     cell_coords(dc, c, I, J, K);
     const int fi = cx ? 2 * I : I, fj = cy ? 2 * J : J, fk = cz ? 2 * K : K;
-    T acc = T(0);
+    float acc = 0.f;
     for (int oi = -cx; oi <= cx; ++oi) {
-        const T wi = cx ? (oi == 0 ? T(0.5) : T(0.25)) : T(1);
+        const float wi = cx ? (oi == 0 ? 0.5f : 0.25f) : 1.f;
         for (int oj = -cy; oj <= cy; ++oj) {
-            const T wj = cy ? (oj == 0 ? T(0.5) : T(0.25)) : T(1);
+            const float wj = cy ? (oj == 0 ? 0.5f : 0.25f) : 1.f;
             for (int ok = -cz; ok <= cz; ++ok) {
                 if (red && ((fi + oi + fj + oj + fk + ok) & 1)) continue;
-                const T wk = cz ? (ok == 0 ? T(0.5) : T(0.25)) : T(1);
+                const float wk = cz ? (ok == 0 ? 0.5f : 0.25f) : 1.f;
                 const int i = (fi + oi) & (df.n0 - 1), j = (fj + oj) & (df.n1 - 1),
                           k = (fk + ok) & (df.n2 - 1);
                 const int n = cell_index(df, i, j, k);
-                Stencil7<T> s = stencil7_any<T>(df, hx, hy, hz, i, j, k, n, u, a, face);
-                const T r = f[n] - (s.off - s.diag * u[n]);
+                Stencil7 s = stencil7_any(df, hx, hy, hz, i, j, k, n, u, a, face);
+                const float r = f[n] - (s.off - s.diag * u[n]);
                 acc += wi * wj * wk * r;
             }
         }
@@ -321,26 +318,25 @@ __global__ void k_faces_line(Dims df, Dims dc, const float* __restrict__ in, int
 }
 
 // Trilinear prolongation of the coarse correction, added to the fine field.
-template <typename T>
-__global__ void k_prolong_add(Dims df, Dims dc, int cx, int cy, int cz, const T* __restrict__ uc,
-                              T* __restrict__ u) {
+__global__ void k_prolong_add(Dims df, Dims dc, int cx, int cy, int cz, const float* __restrict__ uc,
+                              float* __restrict__ u) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= df.cells) return;
     int i, j, k;
     cell_coords(df, c, i, j, k);
     int ii[2], jj[2], kk[2];
-    T wi[2], wj[2], wk[2];
+    float wi[2], wj[2], wk[2];
     int ni, nj, nk;
-    if (!cx) { ii[0] = i; wi[0] = T(1); ni = 1; }
-    else if (!(i & 1)) { ii[0] = i >> 1; wi[0] = T(1); ni = 1; }
-    else { ii[0] = i >> 1; ii[1] = (i >> 1) + 1; wi[0] = wi[1] = T(0.5); ni = 2; }
-    if (!cy) { jj[0] = j; wj[0] = T(1); nj = 1; }
-    else if (!(j & 1)) { jj[0] = j >> 1; wj[0] = T(1); nj = 1; }
-    else { jj[0] = j >> 1; jj[1] = (j >> 1) + 1; wj[0] = wj[1] = T(0.5); nj = 2; }
-    if (!cz) { kk[0] = k; wk[0] = T(1); nk = 1; }
-    else if (!(k & 1)) { kk[0] = k >> 1; wk[0] = T(1); nk = 1; }
-    else { kk[0] = k >> 1; kk[1] = (k >> 1) + 1; wk[0] = wk[1] = T(0.5); nk = 2; }
-    T acc = T(0);
+    if (!cx) { ii[0] = i; wi[0] = 1.f; ni = 1; }
+    else if (!(i & 1)) { ii[0] = i >> 1; wi[0] = 1.f; ni = 1; }
+    else { ii[0] = i >> 1; ii[1] = (i >> 1) + 1; wi[0] = wi[1] = 0.5f; ni = 2; }
+    if (!cy) { jj[0] = j; wj[0] = 1.f; nj = 1; }
+    else if (!(j & 1)) { jj[0] = j >> 1; wj[0] = 1.f; nj = 1; }
+    else { jj[0] = j >> 1; jj[1] = (j >> 1) + 1; wj[0] = wj[1] = 0.5f; nj = 2; }
+    if (!cz) { kk[0] = k; wk[0] = 1.f; nk = 1; }
+    else if (!(k & 1)) { kk[0] = k >> 1; wk[0] = 1.f; nk = 1; }
+    else { kk[0] = k >> 1; kk[1] = (k >> 1) + 1; wk[0] = wk[1] = 0.5f; nk = 2; }
+    float acc = 0.f;
     for (int p = 0; p < ni; ++p)
         for (int q = 0; q < nj; ++q)
             for (int r = 0; r < nk; ++r)
@@ -547,16 +543,6 @@ __global__ void __launch_bounds__(kInvThreads) k_coarse_invert(Dims d, double hx
     }
 }
 
-template <typename T>
-__global__ void k_coarse_solve(const double* __restrict__ minv, const T* __restrict__ f,
-                               T* __restrict__ u) {
-    const int r = threadIdx.x;
-    if (r >= kNc) return;
-    double acc = 0.0;
-    for (int c = 0; c < kNc; ++c) acc += minv[r * kNc + c] * (double)f[c];
-    u[r] = (T)acc;
-}
-
 __global__ void k_to_f32(int cells, const double* __restrict__ x, float* __restrict__ y) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c < cells) y[c] = (float)x[c];
@@ -569,20 +555,19 @@ __global__ void k_correct(int cells, double* __restrict__ u, const float* __rest
 
 }  // namespace
 
-template <typename T>
-void launch_rbgs_sweep(const Level& L, T* u, const T* f, const T* a, cudaStream_t st) {
+void launch_rbgs_sweep(const Level& L, float* u, const float* f, const float* a, cudaStream_t st) {
     const int half = L.d.cells >> 1;
     launch_counter() += 2;
     for (int colour = 0; colour < 2; ++colour)
-        k_rbgs_colour<T><<<nblocks(half), kThreads, 0, st>>>(L.d, (T)L.h2i[0], (T)L.h2i[1],
-                                                             (T)L.h2i[2], colour, u, f, a, L.face);
+        k_rbgs_colour<<<nblocks(half), kThreads, 0, st>>>(L.d, (float)L.h2i[0], (float)L.h2i[1],
+                                                          (float)L.h2i[2], colour, u, f, a, L.face);
 }
 
 template <>
 void launch_restrict<float>(const Level& fine, const Level& coarse, const float* in, float* out,
                             cudaStream_t st) {
     launch_counter()++;
-    k_restrict<float><<<nblocks(coarse.d.cells), kThreads, 0, st>>>(
+    k_restrict<<<nblocks(coarse.d.cells), kThreads, 0, st>>>(
         fine.d, coarse.d, fine.coarsen[0], fine.coarsen[1], fine.coarsen[2], in, out);
 }
 
@@ -594,13 +579,12 @@ void launch_restrict<double>(const Level& fine, const Level& coarse, const doubl
         fine.d, coarse.d, fine.coarsen[0], fine.coarsen[1], fine.coarsen[2], in, out);
 }
 
-template <typename T>
-void launch_resid_restrict(const Level& fine, const Level& coarse, const T* u, const T* f,
-                           const T* a, T* out, bool swept, cudaStream_t st) {
+void launch_resid_restrict(const Level& fine, const Level& coarse, const float* u, const float* f,
+                           const float* a, float* out, bool swept, cudaStream_t st) {
     launch_counter()++;
-    k_resid_restrict<T><<<nblocks(coarse.d.cells), kThreads, 0, st>>>(
-        fine.d, coarse.d, fine.coarsen[0], fine.coarsen[1], fine.coarsen[2], (T)fine.h2i[0],
-        (T)fine.h2i[1], (T)fine.h2i[2], u, f, a, fine.face, swept ? 1 : 0, out);
+    k_resid_restrict<<<nblocks(coarse.d.cells), kThreads, 0, st>>>(
+        fine.d, coarse.d, fine.coarsen[0], fine.coarsen[1], fine.coarsen[2], (float)fine.h2i[0],
+        (float)fine.h2i[1], (float)fine.h2i[2], u, f, a, fine.face, swept ? 1 : 0, out);
 }
 
 void launch_faces_line(const Level& fine, const Level& coarse, const float* in, float* out,
@@ -613,7 +597,7 @@ template <>
 void launch_prolong_add<float>(const Level& fine, const Level& coarse, const float* uc, float* u,
                                cudaStream_t st) {
     launch_counter()++;
-    k_prolong_add<float><<<nblocks(fine.d.cells), kThreads, 0, st>>>(
+    k_prolong_add<<<nblocks(fine.d.cells), kThreads, 0, st>>>(
         fine.d, coarse.d, fine.coarsen[0], fine.coarsen[1], fine.coarsen[2], uc, u);
 }
 
@@ -635,12 +619,6 @@ void launch_coarse_invert(const Level& L, const T* a, double* minv, cudaStream_t
     launch_counter()++;
     k_coarse_invert<T><<<1, kInvThreads, 0, st>>>(L.d, L.h2i[0], L.h2i[1], L.h2i[2], a,
                                                          L.face, minv);
-}
-
-template <typename T>
-void launch_coarse_solve(const double* minv, const T* f, T* u, cudaStream_t st) {
-    launch_counter()++;
-    k_coarse_solve<T><<<1, kNc, 0, st>>>(minv, f, u);
 }
 
 void launch_to_f32(int cells, const double* x, float* y, cudaStream_t st) {
@@ -688,12 +666,8 @@ void launch_correct(int cells, double* u, const float* e, cudaStream_t st) {
     k_correct<<<nblocks(cells), kThreads, 0, st>>>(cells, u, e);
 }
 
-template void launch_rbgs_sweep<float>(const Level&, float*, const float*, const float*, cudaStream_t);
-template void launch_resid_restrict<float>(const Level&, const Level&, const float*, const float*,
-                                           const float*, float*, bool, cudaStream_t);
 template void launch_coarse_invert<float>(const Level&, const float*, double*, cudaStream_t);
 template void launch_coarse_invert<double>(const Level&, const double*, double*, cudaStream_t);
-template void launch_coarse_solve<float>(const double*, const float*, float*, cudaStream_t);
 
 }  // namespace recon
 

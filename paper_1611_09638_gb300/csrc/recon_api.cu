@@ -202,48 +202,42 @@ void prof_mark(Handle* H) {
     else cudaEventRecord(e, H->st);
 }
 
-template <typename T>
-void sweeps_unprofiled(Handle* H, int l, int nu, T** cur, T** oth, const T* f, const T* c,
+void sweeps_unprofiled(Handle* H, int l, int nu, float** cur, float** oth, const float* f, const float* c,
                        bool zero_first) {
     bool zero = zero_first;
-    for (int s = 0; s < nu;) {
-        const int k = launch_rbgs_fused<T>(H->lv[l], zero ? nullptr : *cur, *oth, f, c, nu - s, H->st);
-        if (k > 0) {
-            T* t = *cur;
-            *cur = *oth, *oth = t;
-            s += k;
+    for (int s = 0; s < nu; ++s) {
+        if (launch_rbgs_fused(H->lv[l], zero ? nullptr : *cur, *oth, f, c, H->st)) {
+            std::swap(*cur, *oth);
         } else {
-            if (zero) cudaMemsetAsync(*cur, 0, sizeof(T) * H->lv[l].d.cells, H->st);
-            launch_rbgs_sweep<T>(H->lv[l], *cur, f, c, H->st);
-            s += 1;
+            if (zero) cudaMemsetAsync(*cur, 0, sizeof(float) * H->lv[l].d.cells, H->st);
+            launch_rbgs_sweep(H->lv[l], *cur, f, c, H->st);
         }
         zero = false;
     }
-    if (zero) cudaMemsetAsync(*cur, 0, sizeof(T) * H->lv[l].d.cells, H->st);  // nu == 0
+    if (zero) cudaMemsetAsync(*cur, 0, sizeof(float) * H->lv[l].d.cells, H->st);  // nu == 0
 }
 
-// nu red-black sweeps of level l on the field held in *cur (zero_first: it is
+// nu red-black sweeps of FP32 level l on the field held in *cur (zero_first: it is
 // 0 on entry and need not be read or cleared).  Where the level fits the
-// streaming kernel (FP32 levels) the sweeps run out of place, ping-ponging
+// streaming kernel the sweeps run out of place, ping-ponging
 // between *cur and *oth, and the two pointers are swapped so that *cur holds
 // the result; elsewhere the two colour passes run in place.  With
 // params.profile the finest level's full sweeps (read u, a, f; write u) are
 // bracketed with events; a sweep from u = 0 reads no u and is left out.
-template <typename T>
-void smooth_sweeps(Handle* H, int l, int nu, T** cur, T** oth, const T* f, const T* c,
+void smooth_sweeps(Handle* H, int l, int nu, float** cur, float** oth, const float* f, const float* c,
                    bool zero_first) {
     if (!(H->p.profile && l == 0)) {
-        sweeps_unprofiled<T>(H, l, nu, cur, oth, f, c, zero_first);
+        sweeps_unprofiled(H, l, nu, cur, oth, f, c, zero_first);
         return;
     }
     if (zero_first) {
         const int first = nu > 0 ? 1 : 0;
-        sweeps_unprofiled<T>(H, l, first, cur, oth, f, c, true);
+        sweeps_unprofiled(H, l, first, cur, oth, f, c, true);
         nu -= first;
     }
     if (nu <= 0) return;
     prof_mark(H);
-    sweeps_unprofiled<T>(H, l, nu, cur, oth, f, c, false);
+    sweeps_unprofiled(H, l, nu, cur, oth, f, c, false);
     prof_mark(H);
     H->prof_sweeps += nu;
 }
@@ -342,72 +336,52 @@ int sync_scalars(Handle* H) {
 
 // ------------------------------------------------------------ V-cycles
 
-template <typename T>
-struct MG {
-    std::vector<T*>& u;
-    std::vector<T*>& f;
-    std::vector<T*>& c;
-    std::vector<T*>& r;
-};
-
-// One V(nu1, nu2) cycle of level l on L u = f; zero_u: u = 0 on entry.  The
+// One V(nu1, nu2) cycle of FP32 level l on L u = f; zero_u: u = 0 on entry.  The
 // level's residual buffer doubles as the ping-pong partner of the streaming
 // smoother; with even sweep counts the result is back in u, otherwise it is
 // copied there.
-// correct_into (mixed mode, finest level): if not null, the V-cycle's
+// correct_into (finest level): if not null, the V-cycle's
 // result is also added to this FP64 field, by the last sweep where it can be;
 // returns whether it was.
-template <typename T>
-bool vcycle(Handle* H, MG<T>& g, int l, T* u, const T* f, bool zero_u,
-            double* correct_into = nullptr) {
-    const int last = (int)H->lv.size() - 1;
+bool vcycle(Handle* H, int l, float* u, const float* f, bool zero_u, double* correct_into = nullptr) {
+    // (every hierarchy ends in one of these two)
     const Level& L = H->lv[l];
     if (l == H->lc && launch_coarse_cluster(H->cc, f, u, H->minv, zero_u, 1, H->st)) return false;
     if (l == H->l0 && launch_coarse_vcycle(H->cs, f, u, H->minv, zero_u, H->st)) return false;
-    if (l == last) {
-        launch_coarse_solve<T>(H->minv, f, u, H->st);
-        return false;
-    }
-    T* cur = u;
-    T* oth = g.r[l];
-    smooth_sweeps<T>(H, l, H->p.nu1, &cur, &oth, f, g.c[l], zero_u);
-    bool streamed = false;
-    if constexpr (sizeof(T) == sizeof(float))
-        streamed = launch_resid_restrict_stream(L, H->lv[l + 1], cur, f, g.c[l], g.f[l + 1], H->st);
-    if (!streamed)
-        launch_resid_restrict<T>(L, H->lv[l + 1], cur, f, g.c[l], g.f[l + 1], H->p.nu1 > 0, H->st);
-    vcycle<T>(H, g, l + 1, g.u[l + 1], g.f[l + 1], true);
+    const float* c = H->c32[l];
+    const float* uc = H->u32[l + 1];
+    float* cur = u;
+    float* oth = H->r32[l];
+    smooth_sweeps(H, l, H->p.nu1, &cur, &oth, f, c, zero_u);
+    if (!launch_resid_restrict_stream(L, H->lv[l + 1], cur, f, c, H->f32[l + 1], H->st))
+        launch_resid_restrict(L, H->lv[l + 1], cur, f, c, H->f32[l + 1], H->p.nu1 > 0, H->st);
+    vcycle(H, l + 1, H->u32[l + 1], H->f32[l + 1], true);
     int nu2 = H->p.nu2;
     bool folded = false, corrected = false;
-    if constexpr (sizeof(T) == sizeof(float)) {
-        // the coarse correction folded into the first post-smoothing sweep,
-        // and the defect correction too where that sweep is the last
-        double* c64 = nu2 == 1 ? correct_into : nullptr;
-        if (nu2 >= 1 &&
-            launch_rbgs_prolong(L, H->lv[l + 1], g.u[l + 1], cur, oth, f, g.c[l], H->st, c64)) {
+    // the coarse correction folded into the first post-smoothing sweep,
+    // and the defect correction too where that sweep is the last
+    double* c64 = nu2 == 1 ? correct_into : nullptr;
+    if (nu2 >= 1 && launch_rbgs_prolong(L, H->lv[l + 1], uc, cur, oth, f, c, H->st, c64)) {
+        std::swap(cur, oth);
+        nu2 -= 1;
+        folded = true;
+        corrected = c64 != nullptr;
+    }
+    if (!folded) launch_prolong_add<float>(L, H->lv[l + 1], uc, cur, H->st);
+    // the defect correction folded into the last sweep
+    if (correct_into && !corrected && nu2 >= 1) {
+        smooth_sweeps(H, l, nu2 - 1, &cur, &oth, f, c, false);
+        if (launch_rbgs_correct(L, cur, oth, f, c, correct_into, H->st)) {
             std::swap(cur, oth);
-            nu2 -= 1;
-            folded = true;
-            corrected = c64 != nullptr;
+            corrected = true;
+        } else {
+            smooth_sweeps(H, l, 1, &cur, &oth, f, c, false);
         }
+        nu2 = 0;
     }
-    if (!folded) launch_prolong_add<T>(L, H->lv[l + 1], g.u[l + 1], cur, H->st);
-    if constexpr (sizeof(T) == sizeof(float)) {
-        // the defect correction folded into the last sweep
-        if (correct_into && !corrected && nu2 >= 1) {
-            smooth_sweeps<T>(H, l, nu2 - 1, &cur, &oth, f, g.c[l], false);
-            if (launch_rbgs_correct(L, cur, oth, f, g.c[l], correct_into, H->st)) {
-                std::swap(cur, oth);
-                corrected = true;
-            } else {
-                smooth_sweeps<T>(H, l, 1, &cur, &oth, f, g.c[l], false);
-            }
-            nu2 = 0;
-        }
-    }
-    smooth_sweeps<T>(H, l, nu2, &cur, &oth, f, g.c[l], false);
+    smooth_sweeps(H, l, nu2, &cur, &oth, f, c, false);
     if (cur != u)
-        cudaMemcpyAsync(u, cur, sizeof(T) * L.d.cells, cudaMemcpyDeviceToDevice, H->st);
+        cudaMemcpyAsync(u, cur, sizeof(float) * L.d.cells, cudaMemcpyDeviceToDevice, H->st);
     return corrected;
 }
 
@@ -437,28 +411,26 @@ void vcycle64(Handle* H, int l, double* u, const double* f, bool zero_u) {
     sweeps(H->p.nu2, false);
 }
 
-template <typename T>
-void build_hierarchy(Handle* H, std::vector<T*>& c) {
-    if constexpr (sizeof(T) == sizeof(double)) {
-        for (size_t l = 0; l < H->lv.size(); ++l) {
-            if (l) launch_restrict<double>(H->lv[l - 1], H->lv[l], c[l - 1], c[l], H->st);
-            if (l + 1 < H->lv.size())
-                launch_faces64(H->lv[l], c[l], H->F64l[l], H->D64l[l], H->I64l[l], H->st);
-        }
-        launch_coarse_invert<double>(H->lv.back(), c.back(), H->minv, H->st);
-        return;
-    }
+// The coefficient hierarchy of a step and the inverse of its 4^3 level.
+void build_hierarchy(Handle* H) {
     launch_faces64(H->lv[0], H->a64, H->F64, H->D64, nullptr, H->st);
     for (size_t l = 0; l + 1 < H->lv.size(); ++l) {
-        if constexpr (sizeof(T) == sizeof(float)) {
-            if (H->lv[l + 1].face) {
-                launch_faces_line(H->lv[l], H->lv[l + 1], c[l], c[l + 1], H->st);
-                continue;
-            }
-        }
-        launch_restrict<T>(H->lv[l], H->lv[l + 1], c[l], c[l + 1], H->st);
+        if (H->lv[l + 1].face)
+            launch_faces_line(H->lv[l], H->lv[l + 1], H->c32[l], H->c32[l + 1], H->st);
+        else
+            launch_restrict<float>(H->lv[l], H->lv[l + 1], H->c32[l], H->c32[l + 1], H->st);
     }
-    launch_coarse_invert<T>(H->lv.back(), c.back(), H->minv, H->st);
+    launch_coarse_invert<float>(H->lv.back(), H->c32.back(), H->minv, H->st);
+}
+
+// The same in FP64, with every level's faces and diagonals.
+void build_hierarchy64(Handle* H) {
+    for (size_t l = 0; l < H->lv.size(); ++l) {
+        if (l) launch_restrict<double>(H->lv[l - 1], H->lv[l], H->c64[l - 1], H->c64[l], H->st);
+        if (l + 1 < H->lv.size())
+            launch_faces64(H->lv[l], H->c64[l], H->F64l[l], H->D64l[l], H->I64l[l], H->st);
+    }
+    launch_coarse_invert<double>(H->lv.back(), H->c64.back(), H->minv, H->st);
 }
 
 // Mass per current curvilinear cell (tracer CIC deposit, or the carried m
@@ -514,8 +486,8 @@ void step_head(Handle* H, const CtlHandles& h) {
 // and the first defect is the FP64 residual s - L phidot; otherwise
 // phidot = 0 and the defect is s itself (its FP32 copy).
 void mg_head(Handle* H, const CtlHandles& h, bool warm) {
-    if (H->mixed) build_hierarchy<float>(H, H->c32);
-    else build_hierarchy<double>(H, H->c64);
+    if (H->mixed) build_hierarchy(H);
+    else build_hierarchy64(H);
     if (warm && H->p.warm_start == 2)
         launch_warm_extrapolate(H->ctl, H->arr.alpha, H->phidot, H->phidot_prev, H->cells, H->st);
     if (warm) {
@@ -534,12 +506,11 @@ void mg_head(Handle* H, const CtlHandles& h, bool warm) {
 // correction starts), then the control's decision whether the correction
 // ends after this block.
 void mg_block(Handle* H, const CtlHandles& h) {
-    MG<float> g{H->u32, H->f32, H->c32, H->r32};
     launch_zero_if_fresh(H->ctl, H->u32[0], H->cells, H->st);
     // (a 32^3 finest level: all of them in one launch)
     if (!(H->lc == 0 && launch_coarse_cluster(H->cc, H->f32[0], H->u32[0], H->minv, false, H->p.inner_vcycles, H->st)))
         for (int v = 0; v < H->p.inner_vcycles; ++v)
-            vcycle<float>(H, g, 0, H->u32[0], H->f32[0], false, nullptr);
+            vcycle(H, 0, H->u32[0], H->f32[0], false);
     launch_ctl_block(H->ctl, H->arr, H->p.inner_vcycles, H->p.max_vcycles, h, H->st);
 }
 
@@ -569,13 +540,12 @@ void mg_iter(Handle* H, const CtlHandles& h) {
         vcycle64(H, 0, H->phidot, H->s, false);
         launch_residual_norm64(L0, H->phidot, H->s, H->F64, H->D64, H->part[0], H->st);
     } else {
-        MG<float> g{H->u32, H->f32, H->c32, H->r32};
         bool corrected = false;
         if (!(H->lc == 0 &&
               launch_coarse_cluster(H->cc, H->f32[0], H->u32[0], H->minv, true, H->p.inner_vcycles, H->st)))
             for (int v = 0; v < H->p.inner_vcycles; ++v) {
                 const bool last = v + 1 == H->p.inner_vcycles;
-                corrected = vcycle<float>(H, g, 0, H->u32[0], H->f32[0], v == 0, last ? H->phidot : nullptr);
+                corrected = vcycle(H, 0, H->u32[0], H->f32[0], v == 0, last ? H->phidot : nullptr);
             }
         if (!corrected) launch_correct(H->cells, H->phidot, H->u32[0], H->st);
         launch_residual64_to32(L0, H->phidot, H->s, H->F64, H->D64, H->f32[0], H->part[0], H->st);

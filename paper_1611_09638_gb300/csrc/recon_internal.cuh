@@ -168,13 +168,14 @@ struct FinishList {
 void finish_reduces(const FinishList& l, double* scalars, cudaStream_t st);
 void finish_reduce(const double* partials, int op, double* scalars, int slot, cudaStream_t st);
 
-// ---- multigrid (T = float or double) --------------------------------------
-template <typename T>
-void launch_rbgs_sweep(const Level& L, T* u, const T* f, const T* a, cudaStream_t st);
-// Up to nsweeps full red-black sweeps u_new <- RBGS^k(u_old) in a single
-// streaming pass (smoother.cu); u_old == nullptr means u_old = 0.  Returns k,
-// the sweeps done; 0 (nothing launched) when the level is not a multiple of
-// the kernel's tile or the precision does not use the streaming kernel.
+// ---- multigrid ------------------------------------------------------------
+// A red-black sweep of an FP32 level in place, a launch per colour.
+void launch_rbgs_sweep(const Level& L, float* u, const float* f, const float* a, cudaStream_t st);
+// A red-black sweep u_new <- RBGS(u_old) in a single streaming pass
+// (smoother.cu); u_old == nullptr means u_old = 0.  Returns false, with nothing
+// launched, when the level is not a multiple of the kernel's tile.
+bool launch_rbgs_fused(const Level& L, const float* u_old, float* u_new, const float* f, const float* a,
+                       cudaStream_t st);
 // Residual and full-weighting restriction of an FP32 level in one streaming
 // pass; returns 1, or 0 with nothing launched where the level does not fit
 // its tiles (then launch_resid_restrict does the work).
@@ -216,15 +217,6 @@ int launch_rbgs_correct(const Level& L, const float* u_old, float* u_new, const 
                         const float* a, double* u64, cudaStream_t st);
 
 template <typename T>
-int launch_rbgs_fused(const Level& L, const T* u_old, T* u_new, const T* f, const T* a,
-                      int nsweeps, cudaStream_t st);
-template <>
-int launch_rbgs_fused<float>(const Level&, const float*, float*, const float*, const float*,
-                             int, cudaStream_t);
-template <>
-int launch_rbgs_fused<double>(const Level&, const double*, double*, const double*,
-                              const double*, int, cudaStream_t);
-template <typename T>
 void launch_restrict(const Level& fine, const Level& coarse, const T* in, T* out, cudaStream_t st);
 // Face sums of a coarse level (every axis halved) from the level above
 // (nodal coefficient, or its face sums when fine.face): along each axis the
@@ -236,17 +228,15 @@ void launch_faces_line(const Level& fine, const Level& coarse, const float* in, 
 void launch_to_f32(int cells, const double* x, float* y, cudaStream_t st);
 // full-weighting restriction of the residual f - L u, without storing it;
 // swept: u comes from a red-black sweep, so only red nodes have one
-template <typename T>
-void launch_resid_restrict(const Level& fine, const Level& coarse, const T* u, const T* f,
-                           const T* a, T* out, bool swept, cudaStream_t st);
+void launch_resid_restrict(const Level& fine, const Level& coarse, const float* u, const float* f,
+                           const float* a, float* out, bool swept, cudaStream_t st);
 template <typename T>
 void launch_prolong_add(const Level& fine, const Level& coarse, const T* uc, T* u, cudaStream_t st);
 // Coarsest (4x4x4) level: the 64 x 64 matrix of the mean-free solution, once
-// per coefficient (FP64), then each solve is one matrix-vector product.
+// per coefficient (FP64); each solve is one matrix-vector product then, done
+// by the kernels that hold the coarse levels.
 template <typename T>
 void launch_coarse_invert(const Level& L, const T* a, double* minv, cudaStream_t st);
-template <typename T>
-void launch_coarse_solve(const double* minv, const T* f, T* u, cudaStream_t st);
 // The FP64 levels from the first one of at most kCoarse64Cells nodes down, in
 // one block from their stored faces, diagonals and inverse diagonals.
 constexpr int kCoarse64Cells = 512;

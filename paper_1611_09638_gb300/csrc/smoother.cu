@@ -638,14 +638,13 @@ bool iso_level(const Level& L) { return L.h2i[0] == L.h2i[1] && L.h2i[1] == L.h2
 
 }  // namespace
 
-// One sweep u_new <- RBGS(u_old) in one pass when the level is a multiple of
-// the tile; returns the number of sweeps done (1), or 0 with nothing launched.
-template <>
-int launch_rbgs_fused<float>(const Level& L, const float* u_old, float* u_new, const float* f,
-                             const float* a, int nsweeps, cudaStream_t st) {
-    if (nsweeps < 1 || !stream_fits(L.d) || (L.face && !iso_level(L))) return 0;
+// (FP64 levels are bound by the FP64 issue rate, not by memory: the ring nodes
+// this kernel recomputes would cost them more than the traffic it saves.)
+bool launch_rbgs_fused(const Level& L, const float* u_old, float* u_new, const float* f, const float* a,
+                       cudaStream_t st) {
+    if (!stream_fits(L.d) || (L.face && !iso_level(L))) return false;
     launch_sweep<false, false>(L, u_old, u_new, f, a, nullptr, L.d, nullptr, st);
-    return 1;
+    return true;
 }
 
 bool rbgs_prolong_fits(const Level& fine) {
@@ -731,15 +730,6 @@ bool sweep_wait_failed() {
     if (cudaMemcpyFromSymbol(&v, g_sweep_wait_fail, sizeof(int)) != cudaSuccess) return false;
     if (v) cudaMemcpyToSymbol(g_sweep_wait_fail, &zero, sizeof(int));
     return v != 0;
-}
-
-// FP64 levels are bound by the FP64 issue rate, not by memory: the ring nodes
-// the streaming kernel recomputes would cost more than the traffic they save,
-// so FP64 sweeps use the in-place two-colour kernels.
-template <>
-int launch_rbgs_fused<double>(const Level&, const double*, double*, const double*,
-                              const double*, int, cudaStream_t) {
-    return 0;
 }
 
 }  // namespace recon
