@@ -279,8 +279,10 @@ __global__ void __cluster_dims__(kCR, 1, 1) __launch_bounds__(kCT)
     // the neighbour that takes this thread's value of a colour, and the slot
     // there: pair 1 goes to the next block's slot 0, pair 0 to the previous
     // one's slot 3.  Red: (j + k) even holds plane 0, odd plane 3.
-    float* const outR = s0 ? cluster.map_shared_rank(sR, next) + t : cluster.map_shared_rank(sR, prev) + 3 * kCol + t;
-    float* const outB = s0 ? cluster.map_shared_rank(sB, prev) + 3 * kCol + t : cluster.map_shared_rank(sB, next) + t;
+    // (RC_OFF: checked against the extent in the RECON_CHECKED build)
+    const int first = RC_OFF(t, kTop, 302), fourth = RC_OFF(3 * kCol + t, kTop, 303);
+    float* const outR = cluster.map_shared_rank(sR, s0 ? next : prev) + (s0 ? first : fourth);
+    float* const outB = cluster.map_shared_rank(sB, s0 ? prev : next) + (s0 ? fourth : first);
 
     if (self == 0) {
         s_fetch<N1, FACE>(L1, cs.a[1]);
@@ -297,7 +299,7 @@ __global__ void __cluster_dims__(kCR, 1, 1) __launch_bounds__(kCT)
     {
         const float* a = cs.a[0];
         constexpr int n = kCN * kCol;
-        auto plane = [&](int p) { return ((4 * self + p) & m) * kCol; };
+        auto plane = [&](int p) { return RC_OFF(((4 * self + p) & m) * kCol, kCN * kCol - kCol + 1, 306); };
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int pr = plane(2 * q + s0), pb = plane(2 * q + 1 - s0);
@@ -392,7 +394,7 @@ __global__ void __cluster_dims__(kCR, 1, 1) __launch_bounds__(kCT)
             // plane p of the block (-1 .. 3): pair p >> 1
             auto r = [&](int p, int jj, int kk) {
                 jj &= m, kk &= m;
-                const int at = ((p >> 1) + 1) * kCol + jj * kCN + kk;
+                const int at = RC_OFF(((p >> 1) + 1) * kCol + jj * kCN + kk, kTop, 304);
                 return ((p + jj + kk) & 1) ? sQ[at] : sP[at];
             };
             const float v = weighted<kCN>(r, q, J, K, cs.nu1 > 0);
@@ -416,7 +418,8 @@ __global__ void __cluster_dims__(kCR, 1, 1) __launch_bounds__(kCT)
         cluster.sync();
         // the 16^3 correction around this block, then u += P of it, on the
         // neighbours' pairs too, so that no exchange is needed
-        sC[t] = cluster.map_shared_rank(L1.u, 0)[((2 * self - 1 + t / (N1 * N1)) & (N1 - 1)) * (N1 * N1) + (t & (N1 * N1 - 1))];
+        sC[t] = cluster.map_shared_rank(L1.u, 0)[RC_OFF(
+            ((2 * self - 1 + t / (N1 * N1)) & (N1 - 1)) * (N1 * N1) + (t & (N1 * N1 - 1)), N1 * N1 * N1, 305)];
         static_assert(kCoarse == kCT, "one coarse value a thread");
         __syncthreads();
         // interpolated in the coarse planes -1 .. 2, then P on planes -1 .. 4
@@ -440,7 +443,7 @@ __global__ void __cluster_dims__(kCR, 1, 1) __launch_bounds__(kCT)
         for (int s = 0; s < cs.nu2; ++s) sweep(false);
     }
     {
-        auto plane = [&](int p) { return ((4 * self + p) & m) * kCol; };
+        auto plane = [&](int p) { return RC_OFF(((4 * self + p) & m) * kCol, kCN * kCol - kCol + 1, 306); };
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             u_top[plane(2 * q + s0) + t] = uR[q];

@@ -27,6 +27,7 @@
 // are converted once and read back from shared memory 14 times a thread.
 // Bound by instruction issue: 512^3 10.06 -> 3.32 ms; it reads 16 and writes
 // 24 bytes a node (0.8 ms at the copy rate).
+#include "checked.cuh"
 #include "displacement_solve.cuh"
 #include "geometry.cuh"
 #include "recon_internal.cuh"
@@ -74,7 +75,9 @@ __global__ void __launch_bounds__(DT, DPERSM) k_displacement_stream(
     const double alpha = scal[SC_ALPHA];
     const DispScales sc = disp_scales(alpha, scal[SC_MAX_G], scal[SC_SUM_DPHI], scal[SC_WIDE] != 0.0);
     const int t = threadIdx.x, lj = t / DK, lk = t % DK;
-    const int own = (lj + 1) * DPK + lk + 1;
+    // (with the ring around it; RC_OFF: checked against the extent in the
+    // RECON_CHECKED build)
+    const int own = DPK + 1 + RC_OFF(lj * DPK + lk, DN - 2 * DPK - 2, 501);
     const int tiles_k = d.n2 / DK;
     const long long planes = (long long)tiles_k * (d.n1 / DJ) * d.n0;
     long long at = planes * blockIdx.x / gridDim.x;
@@ -104,8 +107,9 @@ __global__ void __launch_bounds__(DT, DPERSM) k_displacement_stream(
         double p0, p1 = 0.0, q0, q1 = 0.0;
         auto load = [&](int i) {
             const int b = (i & (d.n0 - 1)) * plane;
-            p0 = phi[b + c0], q0 = dphi[b + c0];
-            if (two) p1 = phi[b + c1], q1 = dphi[b + c1];
+            const int g0 = RC_OFF(b + c0, d.cells, 502), g1 = RC_OFF(b + c1, d.cells, 503);
+            p0 = phi[g0], q0 = dphi[g0];
+            if (two) p1 = phi[g1], q1 = dphi[g1];
         };
         DispColumn sums{};
         load(i0 - 1);
@@ -159,6 +163,8 @@ __global__ void k_displacement_node(Dims d, const double* __restrict__ scal, con
 }
 
 }  // namespace
+
+int bounds_fail_displacement() { return bounds_fail_take(); }
 
 void launch_node_displacement(const Dims& d, const double* scal, const double* phi, const double* dphi,
                               long long* dx, long long* dy, long long* dz, cudaStream_t st) {

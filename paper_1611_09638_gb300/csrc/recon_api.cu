@@ -1166,6 +1166,8 @@ static int bounds_status() {
     int id = bounds_fail_smoother();
     if (!id) id = bounds_fail_transfer();
     if (!id) id = bounds_fail_cluster();
+    if (!id) id = bounds_fail_screened();
+    if (!id) id = bounds_fail_displacement();
     if (id) return fail(RECON_E_CUDA, "index bounds check %d failed (RECON_CHECKED build)", id);
     return RECON_OK;
 }

@@ -207,6 +207,8 @@ bool sweep_wait_failed();
 int bounds_fail_smoother();
 int bounds_fail_transfer();
 int bounds_fail_cluster();
+int bounds_fail_screened();
+int bounds_fail_displacement();
 int launch_rbgs_prolong(const Level& fine, const Level& coarse, const float* uc, const float* u_old,
                         float* u_new, const float* f, const float* a, cudaStream_t st,
                         double* u64 = nullptr);

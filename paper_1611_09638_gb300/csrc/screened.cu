@@ -16,6 +16,7 @@
 //
 // 512^3: the source 11.9 -> 1.08 ms (it formed and stored e in FP64), the
 // limiter 5.35 -> 1.12 ms; both are bound by instruction issue.
+#include "checked.cuh"
 #include "eigen32.cuh"
 #include "geometry.cuh"
 #include "recon_internal.cuh"
@@ -31,6 +32,11 @@ constexpr int GT = 256;
 template <int GK>
 struct Tile {
     static constexpr int J = GT / GK, PK = GK + 2, N = (J + 2) * PK;
+    // the thread's node in a plane's buffer, which holds the ring around it
+    // (RC_OFF: checked against the extent in the RECON_CHECKED build)
+    __device__ static int own() {
+        return PK + 1 + RC_OFF((int)(threadIdx.x / GK) * PK + (int)(threadIdx.x % GK), N - 2 * PK - 2, 401);
+    }
 };
 constexpr int GPERSM = 3, GBLOCKS = GPERSM * (kRedBlocks / 8);
 
@@ -122,8 +128,8 @@ __device__ __forceinline__ void stream_planes(const Dims& d, const float* const 
             const int b = (i & (d.n0 - 1)) * np;
 #pragma unroll
             for (int q = 0; q < NF; ++q) {
-                v0[q] = field[q][b + c0];
-                v1[q] = two ? field[q][b + c1] : 0.f;
+                v0[q] = field[q][RC_OFF(b + c0, d.cells, 402)];
+                v1[q] = two ? field[q][RC_OFF(b + c1, d.cells, 403)] : 0.f;
             }
         };
         begin();
@@ -150,14 +156,14 @@ struct WarpList {
     // adds node c of the lanes with `on`, in lane order
     __device__ __forceinline__ void add(bool on, int c) {
         const unsigned b = __ballot_sync(0xffffffffu, on);
-        if (on) slot[n + __popc(b & ((1u << (threadIdx.x & 31)) - 1))] = c;
+        if (on) slot[RC_OFF(n + __popc(b & ((1u << (threadIdx.x & 31)) - 1)), 64, 404)] = c;
         n += __popc(b);
         __syncwarp();
     }
     // takes up to 32 nodes off the end; -1 in lanes without one
     __device__ __forceinline__ int take() {
         const int lane = threadIdx.x & 31, have = min(n, 32);
-        const int c = lane < have ? slot[n - have + lane] : -1;
+        const int c = lane < have ? slot[RC_OFF(n - have + lane, 64, 405)] : -1;
         n -= have;
         __syncwarp();
         return c;
@@ -200,7 +206,7 @@ __global__ void __launch_bounds__(GT, GPERSM) k_source_stream(Dims d, SourcePara
     __shared__ float buf[2][1][Tile<GK>::N];
     __shared__ int list[GT / 32][64];
     const int lj = threadIdx.x / GK, lk = threadIdx.x % GK;
-    const int own = (lj + 1) * GPK + lk + 1;
+    const int own = Tile<GK>::own();
     const float xi = (float)sp.xi_m * (1.f + 4.f * kU);  // not below xi_m
     WarpList todo{list[threadIdx.x / 32], 0};
     Column32<GPK> col{};
@@ -393,7 +399,7 @@ __global__ void __launch_bounds__(GT, GPERSM) k_limiter_stream(Dims d, LimiterPa
     __shared__ float buf[2][2][Tile<GK>::N];
     __shared__ int list[GT / 32][64];
     const int lj = threadIdx.x / GK, lk = threadIdx.x % GK;
-    const int own = (lj + 1) * GPK + lk + 1;
+    const int own = Tile<GK>::own();
     const float floor32 = (float)lp.lambda_floor;
     WarpList todo{list[threadIdx.x / 32], 0};
     Column32<GPK> A{}, B{};
@@ -519,7 +525,7 @@ __global__ void __launch_bounds__(GT, GPERSM) k_extrema_stream(Dims d, const dou
     constexpr int GPK = Tile<GK>::PK;
     __shared__ float buf[2][1][Tile<GK>::N];
     const int lj = threadIdx.x / GK, lk = threadIdx.x % GK;
-    const int own = (lj + 1) * GPK + lk + 1;
+    const int own = Tile<GK>::own();
     const float bd = EXACT ? __double2float_ru(bounds[0]) : 0.f, bl = EXACT ? __double2float_ru(bounds[1]) : 0.f,
                 br = EXACT ? __double2float_rd(bounds[2]) : 0.f;
     Column32<GPK> col{};
@@ -584,6 +590,8 @@ int tile_k(const Dims& d) {
 }
 
 }  // namespace
+
+int bounds_fail_screened() { return bounds_fail_take(); }
 
 void launch_source(const Dims& d, const SourceParams& sp, const double* phi, const float* phi32, const double* m,
                    double* t, double* part_sum, cudaStream_t st) {
