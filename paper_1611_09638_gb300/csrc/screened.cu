@@ -1,6 +1,7 @@
 // screened.cu -- the passes of a step that decide something at every node from
-// the triad e = I + Hess phi: the limited source (App. A Eq. elliptic) and the
-// step limiter.  Both need FP64 only near a threshold (the compression limit
+// the triad e = I + Hess phi: the limited source (App. A Eq. elliptic), the
+// step limiter and the closing statistics; and the outputs det e, lambda0 and
+// delta_r.  Source and limiter need FP64 only near a threshold (the compression limit
 // xi_m, the volume limit v_m, the eigenvalue floor): everywhere else FP32
 // values with a bound on their error settle the question, and the result is
 // the FP64 one.
@@ -14,8 +15,10 @@
 // do not depend on timing.  The grid is one round of resident blocks over the
 // planes of all tiles.
 //
-// 512^3: the source 11.9 -> 1.08 ms (it formed and stored e in FP64), the
-// limiter 5.35 -> 1.12 ms; both are bound by instruction issue.
+// 512^3: the source 11.9 -> 1.07 ms (it formed and stored e in FP64), the
+// limiter 5.35 -> 1.16 ms.  With three blocks of 80 registers an SM the issue
+// slots are 57% and 63% busy (256^3, first step) and the FP64 pipe 62% in the
+// source, whose 1 - m and sum are FP64 at every node; DRAM is far from its rate.
 #include "checked.cuh"
 #include "eigen32.cuh"
 #include "geometry.cuh"
@@ -513,8 +516,8 @@ __global__ void k_geometry_out(Dims d, const double* __restrict__ phi, double* _
 // the FP64 value of the node that attains it.  The first pass (EXACT = false)
 // bounds them from FP32 values (the smallest upper bounds, the largest lower
 // one), the second evaluates in FP64 the nodes that the bounds leave open.
-// 512^3: 26 -> 2.0 ms for all three (FP64 at every node, 23 of them for det and
-// lambda0).
+// Bound by instruction issue (79% of the slots).  512^3: 26 -> 2.0 ms for all
+// three (FP64 at every node, 23 of them for det and lambda0).
 template <int GK, bool EXACT>
 __global__ void __launch_bounds__(GT, GPERSM) k_extrema_stream(Dims d, const double* __restrict__ phi,
                                                                    const float* __restrict__ phi32,

@@ -1,7 +1,8 @@
-// step_kernels.cu -- kernels of one moving-mesh step (Sec. II, App. A) other
-// than the multigrid solve: CIC deposits in 64-bit fixed point, geometry of
-// the map x = xi + grad phi, the limited source of Eq. (elliptic), the
-// smoothing operator S, the step limiter, the mesh advance and the outputs.
+// step_kernels.cu -- kernels of one moving-mesh step (Sec. II, App. A): CIC
+// deposits in 64-bit fixed point, the checks of the inputs, the smoothing
+// operator S, the mesh advance, App. A's density update, the mesh positions, and
+// the ends of the reductions.  (Source, limiter, triad and the outputs det,
+// lambda0 and delta_r: screened.cu; node displacements: displacement.cu.)
 #include "fixed_point.cuh"
 #include "geometry.cuh"
 #include "recon_internal.cuh"
