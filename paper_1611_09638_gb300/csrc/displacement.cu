@@ -73,8 +73,7 @@ __global__ void __launch_bounds__(DT, DPERSM) k_displacement_stream(
     constexpr int DJ = DT / DK, DPK = DK + 2, DN = (DJ + 2) * DPK;  // rows, and with the ring
     static_assert(DN <= 2 * DT, "two values a thread and field");
     __shared__ U64 sp[2][DN], sd[2][DN];
-    const double alpha = scal[SC_ALPHA];
-    const DispScales sc = disp_scales(alpha, scal[SC_MAX_G], scal[SC_SUM_DPHI], scal[SC_WIDE] != 0.0);
+    const DispScales sc = disp_scales(scal[SC_ALPHA], scal[SC_MAX_G], scal[SC_SUM_DPHI], scal[SC_WIDE] != 0.0);
     const int t = threadIdx.x, lj = t / DK, lk = t % DK;
     // (with the ring around it; RC_OFF: checked against the extent in the
     // RECON_CHECKED build)
@@ -88,7 +87,7 @@ __global__ void __launch_bounds__(DT, DPERSM) k_displacement_stream(
             const int col = (int)(at / d.n0), i = (int)(at % d.n0);
             const int j = (col / tiles_k) * DJ + lj, k = (col % tiles_k) * DK + lk;
             long long o[3];
-            displacement64(d, phi, dphi, alpha, i, j, k, o);
+            displacement64(d, phi, dphi, scal[SC_ALPHA], i, j, k, o);
             const int c = cell_index(d, i, j, k);
             dx[c] = o[0], dy[c] = o[1], dz[c] = o[2];
         }
@@ -124,7 +123,7 @@ __global__ void __launch_bounds__(DT, DPERSM) k_displacement_stream(
             sums.feed(sp[buf] + own, sd[buf] + own, DPK, h, g);
             if (p > i0) {  // node (p - 1)
                 long long o[3];
-                if (!solve_fixed(sc, h, g, o)) displacement64(d, phi, dphi, alpha, p - 1, j0 + lj, k0 + lk, o);
+                if (!solve_fixed(sc, h, g, o)) displacement64(d, phi, dphi, scal[SC_ALPHA], p - 1, j0 + lj, k0 + lk, o);
                 const int cell = cell_index(d, p - 1, j0 + lj, k0 + lk);
                 dx[cell] = o[0], dy[cell] = o[1], dz[cell] = o[2];
             }

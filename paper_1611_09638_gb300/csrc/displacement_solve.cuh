@@ -77,13 +77,19 @@ __device__ __forceinline__ bool solve_fixed(const DispScales& sc, const long lon
     const float rdet = __fdividef(1.f, xx * Xxx + xy * Xxy + xz * Xxz);
     Xxx *= rdet, Xyy *= rdet, Xzz *= rdet, Xxy *= rdet, Xxz *= rdet, Xyz *= rdet;
     const float emax = fmaxf(fmaxf(fabsf(xx), fabsf(yy)), fmaxf(fabsf(zz), fmaxf(fabsf(xy), fmaxf(fabsf(xz), fabsf(yz)))));
-    // the gradient brought to 62 bits first: most nodes' is far below the field's
-    // largest, which set its scale
-    const U64 any = (U64)(g[0] ^ (g[0] >> 63)) | (U64)(g[1] ^ (g[1] >> 63)) | (U64)(g[2] ^ (g[2] >> 63));
-    const int sh = max(__clzll((long long)any) - 2, 0);
-    const float ug = pow2f(max(31 - sc.Qd - sc.kexp - sh, -126));
-    auto upper = [&](long long v) { return upper_float((long long)((U64)v << sh), ug); };
-    const float g0 = upper(g[0]), g1 = upper(g[1]), g2 = upper(g[2]);
+    float ug = pow2f(max(31 - sc.Qd - sc.kexp, -126));
+    float g0 = upper_float(g[0], ug), g1 = upper_float(g[1], ug), g2 = upper_float(g[2], ug);
+    float gm = fmaxf(fabsf(g0), fmaxf(fabsf(g1), fabsf(g2)));
+    if (gm < 1048576.f * ug) {
+        // far below the field's largest gradient, which set the scale: brought to
+        // 62 bits first, or the first piece would have too few of them
+        const U64 any = (U64)(g[0] ^ (g[0] >> 63)) | (U64)(g[1] ^ (g[1] >> 63)) | (U64)(g[2] ^ (g[2] >> 63));
+        const int sh = max(__clzll((long long)any) - 2, 0);
+        ug = pow2f(max(31 - sc.Qd - sc.kexp - sh, -126));
+        g0 = upper_float((long long)((U64)g[0] << sh), ug), g1 = upper_float((long long)((U64)g[1] << sh), ug),
+        g2 = upper_float((long long)((U64)g[2] << sh), ug);
+        gm = fmaxf(fabsf(g0), fmaxf(fabsf(g1), fabsf(g2)));
+    }
     // integers: e at scale 2^54
     const U64 Exx = (U64)h[0] + (1ull << kPhiBits), Eyy = (U64)h[1] + (1ull << kPhiBits),
               Ezz = (U64)h[2] + (1ull << kPhiBits);
@@ -99,7 +105,6 @@ __device__ __forceinline__ bool solve_fixed(const DispScales& sc, const long lon
     piece(g0, g1, g2);
     // The residual of a piece must fit 62 bits: the error of X is about
     // 2^-22 |e|^2 / det; where that is more, smaller pieces.
-    const float gm = fmaxf(fabsf(g0), fmaxf(fabsf(g1), fabsf(g2)));
     const float crit = emax * emax * emax * fabsf(rdet) * __fdividef(gm, fmaxf(um, 1e-30f));
     if (!(um < 32.f && crit < 3e5f)) return false;
     const int bits = 17 - max(((__float_as_int(crit) >> 23) & 255) - 127 - 9, 0);
@@ -111,7 +116,6 @@ __device__ __forceinline__ bool solve_fixed(const DispScales& sc, const long lon
     float last = um, err = um;
     constexpr float done = 7e-18f;  // 2^-57 cells
     if (err >= done) {
-        const float xmax = fmaxf(fmaxf(fmaxf(fabsf(Xxx), fabsf(Xyy)), fmaxf(fabsf(Xzz), fabsf(Xxy))), fmaxf(fabsf(Xxz), fabsf(Xyz)));
         const int n = 53 + s - sc.Qd - sc.kexp;
         U64 R0 = shift_fixed(g[0], n), R1 = shift_fixed(g[1], n), R2 = shift_fixed(g[2], n);
 #pragma unroll 1
@@ -129,13 +133,17 @@ __device__ __forceinline__ bool solve_fixed(const DispScales& sc, const long lon
             const float sc2 = pow2f(s);
             a0 = __float2int_rn(u0 * sc2), a1 = __float2int_rn(u1 * sc2), a2 = __float2int_rn(u2 * sc2);
             D0 = (D0 << m) + a0, D1 = (D1 << m) + a1, D2 = (D2 << m) + a2;
-            // what remains: the piece's rounding, the residual's (half a unit
-            // of its upper half each, through X), or X's error as the last two
-            // pieces show it
-            err = fmaxf(fmaxf(pow2f(-1 - s), 1.5f * xmax * ur), um * __fdividef(um, last));
-            if (err < done) break;
+            // what remains: the piece's rounding, X's error as the last two
+            // pieces show it, or the residual's rounding (half a unit of each
+            // upper half, through X)
+            err = fmaxf(pow2f(-1 - s), um * __fdividef(um, last));
+            if (err < done) {
+                err = fmaxf(fmaxf(fmaxf(fabsf(Xxx), fabsf(Xyy)), fmaxf(fabsf(Xzz), fabsf(Xxy))), fmaxf(fabsf(Xxz), fabsf(Xyz))) *
+                      (1.5f * ur);
+                if (err < done) break;
+            }
             if (!(um < 0.25f * last)) return false;
-            last = fmaxf(um, 6.f * xmax * ur);
+            last = fmaxf(um, ur);  // (a residual of no unit: its rounding may show next)
             R0 <<= m, R1 <<= m, R2 <<= m;
         }
     }

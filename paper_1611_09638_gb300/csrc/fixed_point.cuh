@@ -26,9 +26,10 @@ __device__ __forceinline__ unsigned long long to_fixed_mod(double x, int Q) {
     const long long b = __double_as_longlong(x);
     const int e = (int)(b >> 52) & 0x7ff;
     const unsigned long long m = e ? (((unsigned long long)b << 10) & 0x3ffffffffffffc00ull) | (1ull << 62) : 0ull;
-    const int r = 1085 - Q - e, t = min(max(r, 0), 63), l = min(max(-r, 0), 63);
+    const int r = 1085 - Q - e, t = min(max(r, 0), 63);
+    unsigned long long v = r > 63 ? 0ull : (m + ((1ull << t) >> 1)) >> t;
     // (r < -63 leaves nothing below 2^64: m is a multiple of 2^10)
-    const unsigned long long v = r > 63 ? 0ull : ((m + ((1ull << t) >> 1)) >> t) << l;
+    if (__builtin_expect(r < 0, 0)) v <<= min(-r, 63);
     const unsigned long long s = (unsigned long long)(b >> 63);
     return (v ^ s) - s;
 }
