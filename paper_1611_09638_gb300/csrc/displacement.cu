@@ -7,7 +7,7 @@
 // division, three products), 10 ms at 512^3 with the Hessian read back from
 // memory.  Here only FP32 and integer instructions run: phi and dphi are
 // brought to 64-bit fixed point as a plane is loaded (phi to 2^-54 whatever its
-// size, modulo 2^64: the limiter's pass over the same phi shows that every
+// size, modulo 2^64: the source's pass over the same phi shows that every
 // second difference fits; dphi to 2^-Qd from the limiter's largest gradient), Hessian and gradient are
 // exact integer sums, and e U = alpha G is solved by iterative refinement: X ~
 // e^-1 in FP32 gives a first U, and each further piece comes from the exact

@@ -471,8 +471,9 @@ void step_head(Handle* H, const CtlHandles& h) {
     if (H->ckpt) launch_ckpt_state(H->ctl, H->cells, H->phi, H->ox, H->oy, H->oz, H->ckpt, H->st);
     deposit_step(H, false);
     SourceParams sp{p.xi_m, p.v_m, p.climiter};
-    launch_source(H->d, sp, H->phi, H->phi32, H->m, H->t, H->part[1], H->st);
-    finish_reduces({2, {{H->part[0], 0, SC_SUM_M}, {H->part[1], 0, SC_SUM_T}}}, H->scal, H->st);
+    launch_source(H->d, sp, H->phi, H->phi32, H->m, H->t, H->part[1], H->part[3], H->st);
+    finish_reduces({3, {{H->part[0], 0, SC_SUM_M}, {H->part[1], 0, SC_SUM_T}, {H->part[3], 2, SC_WIDE}}}, H->scal,
+                   H->st);
     launch_smooth_S(H->d, p.s_side, H->t, H->scal + SC_SUM_T, H->s, nullptr, H->v3, nullptr,
                     H->part[2], H->st);
     finish_reduce(H->part[2], 0, H->scal, SC_SUM_S2, H->st);
@@ -563,16 +564,15 @@ void step_tail(Handle* H, const CtlHandles& h) {
     launch_smooth_S(H->d, p.s_side, H->phidot, nullptr, H->dphi, H->dphi32, H->v3, H->part[0],
                     nullptr, H->st);
     FinishList fin{1, {{H->part[0], 0, SC_SUM_DPHI}}};
-    // (with replayed step lengths, kmax = -1, it finds only what the displacements
-    // need: the largest gradient and the mark on phi's differences)
+    // (with replayed step lengths, kmax = -1, it finds only the largest gradient,
+    // which the displacements need)
     if (!H->replay_d || p.density_update == 0) {
         LimiterParams lp = H->lp;
         if (H->replay_d) lp.kmax = -1;
         launch_limiter(H->d, lp, H->phi, H->dphi, H->phi32, H->dphi32, H->part[1], H->part[2],
-                       H->part[3], H->st);
+                       H->st);
         fin.f[fin.n++] = {H->part[1], 2, SC_MAX_K};
         fin.f[fin.n++] = {H->part[2], 2, SC_MAX_G};
-        fin.f[fin.n++] = {H->part[3], 2, SC_WIDE};
     }
     finish_reduces(fin, H->scal, H->st);
     launch_ctl_select_alpha(H->ctl, H->scal, H->arr, H->replay_d, H->lp.kmax, p.d_max, p.alpha_min,

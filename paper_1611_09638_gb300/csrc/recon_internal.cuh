@@ -82,7 +82,7 @@ enum Scalar {
     SC_ALPHA,         // step length of the current step
     SC_ADJ_A,         // adjoint sweep: sums used for mean projections
     SC_ADJ_B,
-    SC_WIDE,          // nonzero unless FP32 shows every second difference of phi well below 512
+    SC_WIDE,          // nonzero unless every second difference of phi is below 448
     SC_MASS,          // total mass of the deposited particles
     SC_BAD_PARTICLE,  // nonzero if a particle was NaN/Inf or negative; 0 between deposits
     SC_COUNT
@@ -305,9 +305,10 @@ void launch_mass_coef(int cells, unsigned long long* mfix, double inv_scale, dou
 // e6 (6 x cells): the triad e = I + Hess phi (xx, yy, zz, xy, xz, yz), for the
 // adjoint and the carried mass of App. A's variant.
 void launch_triad(const Dims& d, const double* phi, double* e6, cudaStream_t st);
-// t = Sigma + C + E from phi (and its FP32 copy) and m, and partial sums of t.
+// t = Sigma + C + E from phi (and its FP32 copy) and m, partial sums of t, and
+// partials of SC_WIDE (to be finished by a maximum).
 void launch_source(const Dims& d, const SourceParams& sp, const double* phi, const float* phi32, const double* m,
-                   double* t, double* part_sum, cudaStream_t st);
+                   double* t, double* part_sum, double* part_wide, cudaStream_t st);
 // S in one pass, or in three axis passes through tmp2 (2 x cells scratch) on
 // grids that its tile does not fit; out32 (optional) receives an FP32 copy of
 // the result; part_sum (with out32) its sum, part_sq its sum of squares, or
@@ -316,11 +317,11 @@ void launch_smooth_S(const Dims& d, double s_side, const double* in, const doubl
                      double* out, float* out32, double* tmp2, double* part_sum, double* part_sq,
                      cudaStream_t st);
 // phi32, dphi32: FP32 copies of phi and dphi, from which every node is decided
-// that FP32's error bounds leave no doubt about.  Partials of SC_MAX_K, SC_MAX_G
-// and SC_WIDE, to be finished by maxima.
+// that FP32's error bounds leave no doubt about.  Partials of SC_MAX_K and
+// SC_MAX_G, to be finished by maxima.
 void launch_limiter(const Dims& d, const LimiterParams& lp, const double* phi, const double* dphi,
                     const float* phi32, const float* dphi32, double* part_k, double* part_g,
-                    double* part_wide, cudaStream_t st);
+                    cudaStream_t st);
 void launch_node_velocity(const Dims& d, const double* e6, const double* dphi, double* vx,
                           double* vy, double* vz, cudaStream_t st);
 // The step's node displacements alpha V in fixed point (2^-53 cells), for

@@ -177,12 +177,18 @@ struct WarpList {
 // Sigma = 1 - m, C(lambda0) the compression limiter of the triad
 // e = I + Hess phi and E = -2 H(sqrt_g - v_m) |Sigma| the expansion limiter, at
 // one node in FP64.  lambda0 only matters where it is below xi_m (for the soft
-// and step readings C vanishes above it).
+// and step readings C vanishes above it).  *wide: set to 1 where a second difference
+// of phi, or four times a mixed one, reaches 448 (or is not finite), by the upper
+// words, without FP64 work; the displacements of the step know them modulo 1024 only.
 __device__ __noinline__ double source64(const Dims& d, const SourceParams& sp, const double* __restrict__ phi,
-                                        const double* __restrict__ m, int c) {
+                                        const double* __restrict__ m, int c, int* wide) {
     int i, j, k;
     cell_coords(d, c, i, j, k);
     Sym3 e = hessian(d, phi, i, j, k);
+    auto upper = [](double x) { return __double2hiint(x) & 0x7fffffff; };
+    const int diag = max(upper(e.xx), max(upper(e.yy), upper(e.zz)));
+    const int mixed = max(upper(e.xy), max(upper(e.xz), upper(e.yz)));
+    if (diag >= 0x407c0000 || mixed >= 0x405c0000) *wide = 1;  // 448 and 112
     e.xx += 1.0, e.yy += 1.0, e.zz += 1.0;
     const double g = det3(e);
     double C = 0.0;
@@ -197,14 +203,17 @@ __device__ __noinline__ double source64(const Dims& d, const SourceParams& sp, c
 
 // C = E = 0 where FP32 certifies that every eigenvalue of e exceeds xi_m
 // (Sylvester's criterion) and, e being positive definite then, that its trace
-// stays below 3 v_m^(1/3) (det e <= (tr e / 3)^3).
+// stays below 3 v_m^(1/3) (det e <= (tr e / 3)^3) and below 100, which bounds
+// every entry; the FP64 form looks for wide nodes among the others.  pwide: 1
+// where there is one.
 template <int GK>
 __global__ void __launch_bounds__(GT, GPERSM) k_source_stream(Dims d, SourceParams sp, float trace_max,
                                                                   const double* __restrict__ phi,
                                                                   const float* __restrict__ phi32,
                                                                   const double* __restrict__ m,
                                                                   double* __restrict__ t,
-                                                                  double* __restrict__ psum) {
+                                                                  double* __restrict__ psum,
+                                                                  double* __restrict__ pwide) {
     constexpr int GPK = Tile<GK>::PK;
     __shared__ float buf[2][1][Tile<GK>::N];
     __shared__ int list[GT / 32][64];
@@ -214,10 +223,12 @@ __global__ void __launch_bounds__(GT, GPERSM) k_source_stream(Dims d, SourcePara
     WarpList todo{list[threadIdx.x / 32], 0};
     Column32<GPK> col{};
     double s = 0.0;
+    __shared__ int wide;
+    if (threadIdx.x == 0) wide = 0;  // (a barrier comes before the first node)
     auto exact = [&] {
         const int c = todo.take();
         if (c >= 0) {
-            const double v = source64(d, sp, phi, m, c);
+            const double v = source64(d, sp, phi, m, c, &wide);
             t[c] = v;
             s += v;
         }
@@ -246,20 +257,24 @@ __global__ void __launch_bounds__(GT, GPERSM) k_source_stream(Dims d, SourcePara
         });
     while (todo.n > 0) exact();
     s = block_reduce<OpSum>(s);
-    if (threadIdx.x == 0) put_partial(psum, s, kRedBlocks);
+    if (threadIdx.x == 0) put_partial(psum, s, kRedBlocks), put_partial(pwide, wide ? 1.0 : 0.0, kRedBlocks);
 }
 
 // Any grid, every node in FP64.
 __global__ void k_source_node(Dims d, SourceParams sp, const double* __restrict__ phi,
-                              const double* __restrict__ m, double* __restrict__ t, double* __restrict__ psum) {
+                              const double* __restrict__ m, double* __restrict__ t, double* __restrict__ psum,
+                              double* __restrict__ pwide) {
     double s = 0.0;
+    __shared__ int wide;
+    if (threadIdx.x == 0) wide = 0;
+    __syncthreads();
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells; c += gridDim.x * blockDim.x) {
-        const double v = source64(d, sp, phi, m, c);
+        const double v = source64(d, sp, phi, m, c, &wide);
         t[c] = v;
         s += v;
     }
     s = block_reduce<OpSum>(s);
-    if (threadIdx.x == 0) psum[blockIdx.x] = s;
+    if (threadIdx.x == 0) psum[blockIdx.x] = s, pwide[blockIdx.x] = wide ? 1.0 : 0.0;
 }
 
 // Step limiter at one node in FP64: the smallest k in [0, kmax] with
@@ -321,15 +336,12 @@ __device__ inline Hess32 hess32_at(const Dims& d, const float* __restrict__ f, i
 // does not change the result, and where it fails FP32 finds its own k, unless a
 // verdict on the way is open (then the FP64 form does).  The gradient's maximum is FP64 too: a node
 // is evaluated only where FP32 does not show it to be below the largest value
-// its warp has found.  wide: a second difference of phi, or four times a mixed
-// one, may reach 448 (or is not finite); the displacements of the step know them
-// modulo 1024 only.  Every lane of a warp takes part in each call.
+// its warp has found.  Every lane of a warp takes part in each call.
 struct LimiterScreen {
     int kk = 0;            // the warp's largest k so far, and 2^-kk
     float al = 1.f;
     double gm = 0.0;       // this lane's largest |2 G|
     float gw = 0.f;        // the warp's, rounded down
-    bool wide = false;
 
     __device__ __forceinline__ void raise(int k) {
         kk = max(kk, __reduce_max_sync(0xffffffffu, k));
@@ -349,9 +361,6 @@ struct LimiterScreen {
     // a node's Hessians of phi and dphi; returns whether the FP64 form has to
     // find its k
     __device__ __forceinline__ bool node(const LimiterParams& lp, float floor32, const Hess32& a, const Hess32& b) {
-        const float diag = fmaxf(fabsf(a.xx), fmaxf(fabsf(a.yy), fabsf(a.zz)));
-        const float mixed = fmaxf(fabsf(a.xy), fmaxf(fabsf(a.xz), fabsf(a.yz)));
-        wide |= !(fmaxf(diag, 4.f * mixed) + 128.f * kU * a.vmax < 448.f);
         // FP32's verdict at step length l: the entries' error is that of
         // the inputs and Hessians, then of the two additions forming M
         auto verdict = [&](float l) {
@@ -379,13 +388,11 @@ struct LimiterScreen {
         }
         return unsure;
     }
-    // the block's partials (threads of a block: blockDim.x)
-    __device__ __forceinline__ void put(double* pk, double* pg, double* pw) {
+    // the block's partials
+    __device__ __forceinline__ void put(double* pk, double* pg) {
         const double k = block_reduce<OpMax>((double)kk);
         const double g = block_reduce<OpMax>(0.5 * gm);
-        const int w = __syncthreads_or(wide);
-        if (threadIdx.x == 0)
-            put_partial(pk, k, kRedBlocks), put_partial(pg, g, kRedBlocks), put_partial(pw, w ? 1.0 : 0.0, kRedBlocks);
+        if (threadIdx.x == 0) put_partial(pk, k, kRedBlocks), put_partial(pg, g, kRedBlocks);
     }
 };
 
@@ -396,8 +403,7 @@ __global__ void __launch_bounds__(GT, GPERSM) k_limiter_stream(Dims d, LimiterPa
                                                                    const float* __restrict__ phi32,
                                                                    const float* __restrict__ dphi32,
                                                                    double* __restrict__ pk,
-                                                                   double* __restrict__ pg,
-                                                                   double* __restrict__ pw) {
+                                                                   double* __restrict__ pg) {
     constexpr int GPK = Tile<GK>::PK;
     __shared__ float buf[2][2][Tile<GK>::N];
     __shared__ int list[GT / 32][64];
@@ -426,7 +432,7 @@ __global__ void __launch_bounds__(GT, GPERSM) k_limiter_stream(Dims d, LimiterPa
             if (todo.n >= 32) exact();
         });
     while (todo.n > 0) exact();
-    screen.put(pk, pg, pw);
+    screen.put(pk, pg);
 }
 
 // Any grid, a thread a node from memory (whole warps have nodes or none: the
@@ -435,7 +441,7 @@ __global__ void __launch_bounds__(GT, GPERSM) k_limiter_stream(Dims d, LimiterPa
 __global__ void k_limiter_node(Dims d, LimiterParams lp, const double* __restrict__ phi,
                                const double* __restrict__ dphi, const float* __restrict__ phi32,
                                const float* __restrict__ dphi32, double* __restrict__ pk,
-                               double* __restrict__ pg, double* __restrict__ pw) {
+                               double* __restrict__ pg) {
     const float floor32 = (float)lp.lambda_floor;
     LimiterScreen screen;
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < d.cells; c += gridDim.x * blockDim.x) {
@@ -449,7 +455,7 @@ __global__ void k_limiter_node(Dims d, LimiterParams lp, const double* __restric
         const bool unsure = screen.node(lp, floor32, a, b);
         if (__any_sync(0xffffffffu, unsure)) screen.raise(unsure ? limiter64(d, lp, phi, dphi, c) : 0);
     }
-    screen.put(pk, pg, pw);
+    screen.put(pk, pg);
 }
 
 // The outputs of one node in FP64.  Not inlined, so that the fields and the
@@ -597,28 +603,27 @@ int tile_k(const Dims& d) {
 int bounds_fail_screened() { return bounds_fail_take(); }
 
 void launch_source(const Dims& d, const SourceParams& sp, const double* phi, const float* phi32, const double* m,
-                   double* t, double* part_sum, cudaStream_t st) {
+                   double* t, double* part_sum, double* part_wide, cudaStream_t st) {
     launch_counter()++;
     if (const int tk = tile_k(d)) {
-        const float trace_max = (float)(3.0 * cbrt(sp.v_m) * (1.0 - 1e-5));
+        const float trace_max = (float)fmin(100.0, 3.0 * cbrt(sp.v_m) * (1.0 - 1e-5));
         auto fn = tk == 32 ? k_source_stream<32> : k_source_stream<16>;
-        fn<<<GBLOCKS, GT, 0, st>>>(d, sp, trace_max, phi, phi32, m, t, part_sum);
+        fn<<<GBLOCKS, GT, 0, st>>>(d, sp, trace_max, phi, phi32, m, t, part_sum, part_wide);
         return;
     }
-    k_source_node<<<kRedBlocks, kRedThreads, 0, st>>>(d, sp, phi, m, t, part_sum);
+    k_source_node<<<kRedBlocks, kRedThreads, 0, st>>>(d, sp, phi, m, t, part_sum, part_wide);
 }
 
 void launch_limiter(const Dims& d, const LimiterParams& lp, const double* phi, const double* dphi,
                     const float* phi32, const float* dphi32, double* part_k, double* part_g,
-                    double* part_wide, cudaStream_t st) {
+                    cudaStream_t st) {
     launch_counter()++;
     if (const int tk = tile_k(d)) {
         auto fn = tk == 32 ? k_limiter_stream<32> : k_limiter_stream<16>;
-        fn<<<GBLOCKS, GT, 0, st>>>(d, lp, phi, dphi, phi32, dphi32, part_k, part_g, part_wide);
+        fn<<<GBLOCKS, GT, 0, st>>>(d, lp, phi, dphi, phi32, dphi32, part_k, part_g);
         return;
     }
-    k_limiter_node<<<kRedBlocks, kRedThreads, 0, st>>>(d, lp, phi, dphi, phi32, dphi32, part_k, part_g,
-                                                       part_wide);
+    k_limiter_node<<<kRedBlocks, kRedThreads, 0, st>>>(d, lp, phi, dphi, phi32, dphi32, part_k, part_g);
 }
 
 void launch_delta_r(const Dims& d, const double* phi, double* out, double* part_max,
