@@ -25,8 +25,8 @@
 // A block streams planes along i over an 8 x 32 (or 16 x 16) tile; a thread keeps its
 // column's sums of the last planes in registers, so that a plane's 340 nodes
 // are converted once and read back from shared memory 14 times a thread.
-// Bound by instruction issue (70% of the slots, 56% of the integer pipe):
-// 512^3 10.06 -> 3.54 ms; it reads 16 and writes 24 bytes a node (0.8 ms at the
+// Bound by instruction issue (70% of the slots, 54% of the integer pipe):
+// 512^3 10.06 -> 3.49 ms; it reads 16 and writes 24 bytes a node (0.8 ms at the
 // copy rate).
 #include "checked.cuh"
 #include "displacement_solve.cuh"

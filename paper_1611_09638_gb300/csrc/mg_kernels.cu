@@ -109,7 +109,7 @@ __global__ void k_residual64(Dims d, const double* __restrict__ u, const double*
 // sum goes into its FP64 one every kRes32 nodes, so its relative error stays
 // below kRes32 2^-24 = 4e-6 on every grid, and the block sums are FP64.  One
 // round of four blocks per SM with 62 registers, so that a
-// node's fifteen loads are all in flight: 512^3 2.19 -> 1.98 ms, 256^3 274 -> 254
+// node's fifteen loads are all in flight: 512^3 2.19 -> 1.90 ms, 256^3 274 -> 246
 // us against 38 registers in kRedBlocks blocks (eight FP64 instructions at 2
 // lanes a clock and SM take 1.71 ms; rounding the FP32 copy by integer
 // instructions instead took 2.3 ms).

@@ -15,9 +15,9 @@
 // do not depend on timing.  The grid is one round of resident blocks over the
 // planes of all tiles.
 //
-// 512^3: the source 11.9 -> 1.07 ms (it formed and stored e in FP64), the
-// limiter 5.35 -> 1.16 ms.  With three blocks of 80 registers an SM the issue
-// slots are 57% and 63% busy (256^3, first step) and the FP64 pipe 62% in the
+// 512^3: the source 11.9 -> 1.08 ms (it formed and stored e in FP64), the
+// limiter 5.35 -> 1.13 ms.  With three blocks of 80 registers an SM the issue
+// slots are 58% and 62% busy (256^3, first step) and the FP64 pipe 60% in the
 // source, whose 1 - m and sum are FP64 at every node; DRAM is far from its rate.
 #include "checked.cuh"
 #include "eigen32.cuh"
